@@ -266,7 +266,8 @@ void hisq_destroy(hisq_ctx *ctx)
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     tc_forget(ctx);
     for (int p = 0; p < 2; p++) {
-        cudaFree(ctx->links_d[p]);
+        cudaFree(ctx->links_x[p]);
+        cudaFree(ctx->links_xe[p]);
         cudaFree(ctx->links_f[p]);
         cudaFree(ctx->links_f12[p]);
         cudaFree(ctx->links_h[p]);
@@ -307,8 +308,10 @@ hisq_status hisq_load_links(hisq_ctx *ctx, const double *fat, const double *lng,
     const size_t nlink = size_t(ctx->g.V) * 4 * 18 * sizeof(double);
     // (re)allocate gathered arrays
     for (int p = 0; p < 2; p++) {
-        dev_free(ctx, ctx->links_d[p], size_t(Vh) * 16 * 9 * 16);
-        ctx->links_d[p] = nullptr;
+        dev_free(ctx, ctx->links_x[p], links_x_bytes(Vh));
+        ctx->links_x[p] = nullptr;
+        dev_free(ctx, ctx->links_xe[p], size_t(Vh) * 2);
+        ctx->links_xe[p] = nullptr;
         dev_free(ctx, ctx->links_f[p], size_t(Vh) * (ctx->long_recon == 18 ? 8 : 4) * 9 * 16);
         ctx->links_f[p] = nullptr;
         dev_free(ctx, ctx->links_f12[p], size_t(Vh) * long_f32_bytes_per_site(ctx->long_recon));
@@ -322,10 +325,11 @@ hisq_status hisq_load_links(hisq_ctx *ctx, const double *fat, const double *lng,
     }
     ctx->links_loaded = false;
     for (int p = 0; p < 2; p++) {
-        ctx->links_d[p] = (double2 *)dev_alloc(ctx, size_t(Vh) * 16 * 9 * 16);
+        ctx->links_x[p] = (int4 *)dev_alloc(ctx, links_x_bytes(Vh));
+        ctx->links_xe[p] = (short *)dev_alloc(ctx, size_t(Vh) * 2);
         ctx->links_f[p] = (float4 *)dev_alloc(ctx, size_t(Vh) * (long_recon == 18 ? 8 : 4) * 9 * 16);
         if (long_recon != 18) ctx->links_f12[p] = (float4 *)dev_alloc(ctx, size_t(Vh) * long_f32_bytes_per_site(long_recon));
-        if (!ctx->links_d[p] || !ctx->links_f[p] || (long_recon != 18 && !ctx->links_f12[p])) return HISQ_ERR_OOM;
+        if (!ctx->links_x[p] || !ctx->links_xe[p] || !ctx->links_f[p] || (long_recon != 18 && !ctx->links_f12[p])) return HISQ_ERR_OOM;
         // FP16 links are built from the FP32 ones on first use (ensure_half_links)
     }
     ctx->long_recon = long_recon;

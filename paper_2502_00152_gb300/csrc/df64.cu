@@ -19,7 +19,7 @@
 //   colour vectors: float4 [3][Vh] = (re_hi, re_lo, im_hi, im_lo)   48 B / site
 #include <algorithm>
 
-#include "internal.cuh"
+#include "fx64.cuh"
 
 namespace hisq {
 
@@ -168,6 +168,19 @@ __global__ void k_split_df(size_t n, const double2 *__restrict__ in, float4 *__r
     }
 }
 
+// the double-float split of the gathered FP64 links (mantissas, fx64.cuh)
+__global__ void k_split_df_links(int Vh, const int4 *__restrict__ w, const short *__restrict__ e,
+                                 float4 *__restrict__ out)
+{
+    const size_t n = size_t(Vh) * 144;
+    for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
+        const int cb = int(i % size_t(Vh));
+        const double2 d = fx_link(w[fx_link_index(cb, int(i / size_t(Vh)))], e[cb]);
+        const float2 re = split_df(d.x), im = split_df(d.y);
+        out[i] = make_float4(re.x, re.y, im.x, im.y);
+    }
+}
+
 // ------------------------------------------------------------- launch glue
 static hisq_status launch_split(hisq_ctx *ctx, size_t n, const double2 *in, float4 *out)
 {
@@ -186,7 +199,12 @@ hisq_status ensure_df_links(hisq_ctx *ctx)
     float4 *d[2] = {(float4 *)dev_alloc(ctx, n * sizeof(float4)), nullptr};
     if (d[0]) d[1] = (float4 *)dev_alloc(ctx, n * sizeof(float4));
     hisq_status s = (d[0] && d[1]) ? HISQ_OK : HISQ_ERR_OOM;
-    for (int p = 0; p < 2 && s == HISQ_OK; p++) s = launch_split(ctx, n, ctx->links_d[p], d[p]);
+    for (int p = 0; p < 2 && s == HISQ_OK; p++) {
+        ctx->launches++;
+        k_split_df_links<<<ctx->num_sms * 8, 256, 0, ctx->stream>>>(ctx->g.Vh, ctx->links_x[p], ctx->links_xe[p], d[p]);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) s = cuda_err(ctx, e, "double-float link split");
+    }
     if (s != HISQ_OK) { // neither parity is kept, so the next call starts over (message set by the failing call)
         for (int p = 0; p < 2; p++) dev_free(ctx, d[p], d[p] ? n * sizeof(float4) : 0);
         return s;

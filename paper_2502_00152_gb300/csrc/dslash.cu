@@ -7,7 +7,7 @@
 // 16 neighbour colour vectors are gathered from the opposite parity (they stay
 // in L2: a parity field is at most a few hundred MB and the sweep order keeps
 // the +-3 time-slice window resident).
-#include "internal.cuh"
+#include "fx64.cuh"
 
 namespace hisq {
 
@@ -209,6 +209,87 @@ static int blocks_per_sm(K kernel)
     return n;
 }
 
+// ------------------------------------------------- the FP64 kernel
+// Fixed-point sums (fx64.cuh) of FP64 links and vectors, one thread per site, or
+// SPLIT = 4 warps per group of 32 sites, one per direction, whose integer sums are
+// added in shared memory (exact, so the result is the same bit for bit).
+//
+// Bound by the 2304 B of links per site.  Each thread holds the links and the
+// neighbour of two hops (96 registers), so that a warp has 6.5 KB of loads in flight
+// while it multiplies; 4 blocks of 128 threads at 128 registers (136 B spilled) gave
+// 441 us per application on 32^3x64 (split included), 3 blocks at 168 registers 470,
+// 2 at 206 registers 510, blocks of 64 or 32 threads 455 to 471, one hop in flight as
+// the compiler ordered the loads 812; the FP64 kernel took 1040.
+//
+// Split where one thread per site leaves fewer than 16 warps per SM: 8^4 16 us per
+// application instead of 23, 14x10x12x22 26.7 instead of 27.3, 16^3x32 even; on
+// 24^3x48 (68 warps per SM) the split costs 181 instead of 162.
+constexpr int kFxSplitWarps = 16;
+
+template <class Epi, int SPLIT>
+__global__ void __launch_bounds__(128, SPLIT == 1 ? 4 : 3)
+    k_dslash_fx(Geom g, int par, LinksX L, FxField in0, Epi epi, RedArgs ra, int do_red, int fp64)
+{
+    constexpr int kGroups = SPLIT == 1 ? 4 : 1; // site groups of a block
+    __shared__ long long sh[SPLIT == 1 ? 1 : 3][12][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int grp = SPLIT == 1 ? warp : 0, part = SPLIT == 1 ? 0 : warp;
+    double red = 0;
+    for (int b0 = blockIdx.x * kGroups * 32; b0 < g.Vh; b0 += gridDim.x * kGroups * 32) {
+        const int cb = b0 + grp * 32 + lane;
+        const bool on = cb < g.Vh;
+        int c[4] = {0, 0, 0, 0}, s = 0, le = 0, E[1] = {0};
+        FxAcc acc[1];
+        acc[0].zero();
+        const FxField in[1] = {in0};
+        const int4 *w = L.w + fx_link_index(on ? cb : 0, 0);
+        if (on) {
+            cb_coords(g, par, cb, c);
+            s = full_site(g, c);
+            le = L.e[cb];
+            E[0] = fp64 ? kFxMark : fx_site_exponent(g, c, s, in0.e);
+            if (E[0] != kFxMark && le != kFxMark) {
+                if (SPLIT == 1)
+                    fx_directions<1, false>(g, c, s, 0, 4, w, in, E, acc);
+                else
+                    fx_directions<1, false>(g, c, s, part, part + 1, w, in, E, acc);
+            }
+        }
+        if (SPLIT > 1) {
+            if (part > 0) {
+#pragma unroll
+                for (int k = 0; k < 6; k++) {
+                    sh[part - 1][k][lane] = acc[0].h[k];
+                    sh[part - 1][6 + k][lane] = acc[0].m[k];
+                }
+            }
+            __syncthreads();
+            if (part == 0) {
+#pragma unroll
+                for (int k = 0; k < 6; k++)
+#pragma unroll
+                    for (int w = 0; w < 3; w++) {
+                        acc[0].h[k] += sh[w][k][lane];
+                        acc[0].m[k] += sh[w][6 + k][lane];
+                    }
+            }
+            __syncthreads();
+        }
+        if (on && part == 0) {
+            CVec<double> o;
+            if (E[0] != kFxMark && le != kFxMark)
+                o = fx_value(acc[0], E[0], le);
+            else
+                o = fx_site_fp64(g, c, s, w, le, in0.src);
+            epi(cb, o, red);
+        }
+    }
+    if (do_red) {
+        double v[1] = {red};
+        grid_reduce<1>(v, ra);
+    }
+}
+
 template <class SIn, class Lk, class L12T, bool R12, class Epi>
 static hisq_status run_dslash(hisq_ctx *ctx, int par, const Lk &L, const L12T &L12, const SIn &in, const Epi &epi,
                               RedArgs ra, int do_red)
@@ -223,6 +304,35 @@ static hisq_status run_dslash(hisq_ctx *ctx, int par, const Lk &L, const L12T &L
     return HISQ_OK;
 }
 
+// FP64: the input field to mantissas, then the fixed-point kernel.  Without room for
+// the mantissas (50 B per site) every site takes the FP64 path.
+template <class Epi>
+static hisq_status run_fx(hisq_ctx *ctx, int par, const SpinorD &in, const Epi &epi, RedArgs ra, int do_red)
+{
+    const int Vh = ctx->g.Vh;
+    const std::string err = ctx->err;
+    void *buf = get_buf(ctx, BUF_FX, fx_field_bytes(Vh));
+    if (buf) {
+        const hisq_status st = launch_fx_split(ctx, in.p, buf);
+        if (st != HISQ_OK) return st;
+    } else {
+        ctx->err = err;
+    }
+    const LinksX L{ctx->links_x[par], ctx->links_xe[par]};
+    const FxField f = fx_field(buf, in.p, Vh);
+    auto launch = [&](auto kern, int threads, int sites, int *bps) -> hisq_status {
+        if (*bps < 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, kern, threads, 0) != cudaSuccess || *bps < 1))
+            *bps = 1;
+        const int grid = grid_for(ctx, Vh, sites, *bps);
+        kern<<<grid, threads, 0, ctx->stream>>>(ctx->g, par, L, f, epi, ra, do_red, buf ? 0 : 1);
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? HISQ_OK : cuda_err(ctx, e, "FP64 dslash launch");
+    };
+    static int bps1 = -1, bps4 = -1;
+    if (Vh < ctx->num_sms * 32 * kFxSplitWarps) return launch(k_dslash_fx<Epi, 4>, 128, 32, &bps4);
+    return launch(k_dslash_fx<Epi, 1>, 128, 128, &bps1);
+}
+
 // Run the Dslash with output parity `par` on links of precision link_prec
 // (64, 32 or 16) in the context's long-link format.
 template <class S, class Epi>
@@ -233,9 +343,7 @@ static hisq_status run_any(hisq_ctx *ctx, int par, int link_prec, const S &in, c
     const bool r12 = ctx->long_recon == 12, r8 = ctx->long_recon == 8;
     const int nk = (r12 || r8) ? 1 : 2;
     if (link_prec == 64) {
-        if constexpr (sizeof(R) == 8)
-            return run_dslash<S, LinksD, LinksF12, false>(ctx, par, LinksD{ctx->links_d[par], Vh}, LinksF12{nullptr, Vh},
-                                                          in, epi, ra, dored);
+        if constexpr (sizeof(R) == 8) return run_fx(ctx, par, in, epi, ra, dored);
         return set_err(ctx, HISQ_ERR_INVALID_ARG, "FP64 links need FP64 vectors");
     }
     if constexpr (sizeof(R) == 4) {

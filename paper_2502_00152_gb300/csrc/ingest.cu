@@ -6,10 +6,11 @@
 //   fwd, n hops:  W = eta_mu(x) * bc(x, n)        * U_mu(x)
 //   bwd, n hops:  W = -eta_mu(x) * bc(x - n mu, n) * U_mu(x - n mu)^dag
 // with bc = -1 for a hop that wraps the time boundary of an antiperiodic
-// lattice.  They are written in FP64, FP32 and FP16 (see internal.cuh for layouts).
+// lattice.  They are written in FP64 (then turned into the fixed-point operator's
+// mantissas in place, fx64.cuh) and FP32 (see internal.cuh for layouts).
 // With 12-real long links only rows 0 and 1 of S = U_long / long_scale are kept
 // (for fwd and bwd); the Dslash rebuilds row 2 and applies the sign and scale.
-#include "internal.cuh"
+#include "fx64.cuh"
 
 namespace hisq {
 
@@ -66,7 +67,7 @@ __device__ __forceinline__ void atomic_max_nonneg(float *addr, float v)
 }
 
 struct IngestOut {
-    double2 *d;    // FP64 [mu][kind][fb][k][Vh] for this parity
+    double2 *d;    // FP64, fx_link_index, for this parity
     float4 *f;     // FP32 [mu][nk][k][Vh]
     float4 *f12;   // FP32 compressed long: recon 12 [mu][6][Vh], recon 8 [mu][4][Vh], or null
     int nk;
@@ -107,11 +108,11 @@ __global__ void k_ingest(Geom g, int par, const double2 *__restrict__ fat, const
                 bad |= !isfinite(Mf[k].x) | !isfinite(Mf[k].y) | !isfinite(Mb[k].x) | !isfinite(Mb[k].y);
             if (bad) atomicOr(nonfinite, 1);
             // FP64 copy, signs folded
-            double2 *qd = o.d + size_t((mu * 2 + kind) * 2) * 9 * Vh + cb;
+            double2 *qd = o.d + fx_link_index(cb, (mu * 2 + kind) * 2 * 9);
 #pragma unroll
             for (int k = 0; k < 9; k++) {
-                qd[size_t(k) * Vh] = make_double2(sf * Mf[k].x, sf * Mf[k].y);
-                qd[size_t(9 + k) * Vh] = make_double2(sbk * Mb[k].x, sbk * Mb[k].y);
+                qd[32 * k] = make_double2(sf * Mf[k].x, sf * Mf[k].y);
+                qd[32 * (9 + k)] = make_double2(sbk * Mb[k].x, sbk * Mb[k].y);
             }
             if (kind == 1 && recon != 18) {
                 // SU(3) factor, rows 0 and 1
@@ -161,7 +162,7 @@ hisq_status ingest_links(hisq_ctx *ctx, const double *fat_dev, const double *lng
     HISQ_CUDA(cudaMemsetAsync(d_dev, 0, sizeof(float) + sizeof(int), ctx->stream));
     const int nk = recon == 18 ? 2 : 1;
     for (int par = 0; par < 2; par++) {
-        IngestOut o{ctx->links_d[par], ctx->links_f[par], recon != 18 ? ctx->links_f12[par] : nullptr, nk};
+        IngestOut o{(double2 *)ctx->links_x[par], ctx->links_f[par], recon != 18 ? ctx->links_f12[par] : nullptr, nk};
         int grid = (4 * Vh + 255) / 256;
         if (grid > ctx->num_sms * 16) grid = ctx->num_sms * 16;
         ctx->launches++;
@@ -169,6 +170,8 @@ hisq_status ingest_links(hisq_ctx *ctx, const double *fat_dev, const double *lng
                                                 1.0 / long_scale, recon, d_dev, d_bad);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_err(ctx, e, "ingest launch");
+        const hisq_status fs = launch_links_fx(ctx, par);
+        if (fs != HISQ_OK) return fs;
     }
     float hdev = 0;
     int hbad = 0;

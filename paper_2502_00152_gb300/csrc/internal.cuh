@@ -427,7 +427,8 @@ __device__ __forceinline__ CVec<To> cvt(const CVec<From> &v)
 //   (D psi)(x) = sum_mu sum_{kind} [ W_fwd psi(x + n mu) + W_bwd psi(x - n mu) ]
 // (kind 0: fat, n = 1; kind 1: long, n = 3).
 //
-// FP64 (recon 18): double2 [p][mu][kind][fwd,bwd][k=0..8][Vh]
+// FP64 (recon 18): [p][group of 32 sites][mu][kind][fwd,bwd][k=0..8][32], 16 B per complex
+//   element: 56-bit mantissas under one exponent per output site (fx64.cuh)
 // FP32 (recon 18): float4  [p][mu][kind][k=0..8][Vh], float4 = (fwd_k, bwd_k)
 // FP32 long links with recon 12: float4 [p][mu][k=0..5][Vh] holding rows 0,1
 //   of the SU(3) factor S of fwd and bwd; W = sign * long_scale * S, with
@@ -437,25 +438,6 @@ __device__ __forceinline__ CVec<To> cvt(const CVec<From> &v)
 //   factor (a = row 0, b = row 1, c = row 2); the rest follows from unitarity.
 // FP16 (recon 18): uint2 [p][mu][kind][k=0..8][Vh], uint2 = (fwd_k, bwd_k) as
 //   two half2; FP16 long links with recon 12: uint2 [p][mu][k=0..5][Vh].
-struct LinksD {
-    const double2 *base; // parity offset applied
-    int Vh;
-    typedef double real;
-    __device__ __forceinline__ void load(int mu, int kind, int i, CMat<double> &f, CMat<double> &b) const
-    {
-        const double2 *q = base + size_t((mu * 2 + kind) * 2) * 9 * Vh + i;
-#pragma unroll
-        for (int k = 0; k < 9; k++) {
-            double2 a = __ldcs(q + size_t(k) * Vh);
-            double2 c = __ldcs(q + size_t(9 + k) * Vh);
-            f.re[k] = a.x;
-            f.im[k] = a.y;
-            b.re[k] = c.x;
-            b.im[k] = c.y;
-        }
-    }
-};
-
 struct LinksF {
     const float4 *base; // parity offset applied
     int Vh;
@@ -551,6 +533,9 @@ struct LinksF8 { // long links only, 8 reals per SU(3) factor
         su3_from8(b0, b1, b);
     }
 };
+
+// bytes of the FP64 links of one parity (whole groups of 32 sites)
+inline size_t links_x_bytes(int Vh) { return size_t((Vh + 31) / 32) * 32 * 144 * 16; }
 
 // floats of compressed FP32 long links per output site and parity (0: none)
 inline size_t long_f32_bytes_per_site(int recon) { return recon == 12 ? 4 * 6 * 16 : (recon == 8 ? 4 * 4 * 16 : 0); }
@@ -735,6 +720,7 @@ enum BufId : int {
     BUF_DF_X,          // double-float residual: x split into (hi, lo)
     BUF_DF_T,          // double-float residual: odd temporary D_oe x
     BUF_PERSIST,       // persistent batched CG: per-block partials, thresholds
+    BUF_FX,            // FP64 operator: mantissas and exponents of its input field
     BUF_COUNT
 };
 
@@ -765,12 +751,13 @@ struct hisq_ctx {
     double long_scale = 1.0;
 
     // gathered links; index [parity]
-    double2 *links_d[2] = {nullptr, nullptr};  // FP64, 16 hops
+    int4 *links_x[2] = {nullptr, nullptr};     // FP64, 16 hops: mantissas as two limbs (fx64.cuh)
+    short *links_xe[2] = {nullptr, nullptr};   // their exponents, one per output site
     float4 *links_f[2] = {nullptr, nullptr};   // FP32: fat (+ long when recon 18)
     float4 *links_f12[2] = {nullptr, nullptr}; // FP32 long, recon 12
     uint2 *links_h[2] = {nullptr, nullptr};    // FP16: fat (+ long when recon 18)
     uint2 *links_h12[2] = {nullptr, nullptr};  // FP16 long, recon 12
-    float4 *links_df[2] = {nullptr, nullptr};  // double-float split of links_d (built on first use)
+    float4 *links_df[2] = {nullptr, nullptr};  // double-float split of links_x (built on first use)
 
     // reduction scratch
     double *partials = nullptr;
@@ -1067,6 +1054,9 @@ hisq_status launch_dslash_df_xpay(hisq_ctx *ctx, int out_parity, const void *in,
                                   const double *x, double b, const double *y, double c, int norm_slot);
 // r = b - (4m^2 - D_eo D_oe) x on even fields, |r|^2 -> slot
 hisq_status launch_residual_df(hisq_ctx *ctx, const double *b, const double *x, double *r, int slot);
+
+// the gathered FP64 links of one parity to the operator's mantissas, in place (fx64.cu)
+hisq_status launch_links_fx(hisq_ctx *ctx, int par);
 
 // link ingest (ingest.cu)
 hisq_status ingest_links(hisq_ctx *ctx, const double *fat_dev, const double *lng_dev, int recon,
