@@ -336,8 +336,9 @@ hisq_status hisq_set_profiling(hisq_ctx *ctx, int on);
 
 /* CUDA-event time (*seconds) and number (*launches) of the FP64 Dslash launches
  * (reliable-update residuals, source preparation, odd reconstruction, residual
- * checks) made while profiling was on, since it was last switched on.  Waits
- * for the pending launches.  HISQ_ERR_INVALID_ARG for a null argument. */
+ * checks) made while profiling was on, since it was last switched on; a launch
+ * that serves several right-hand sides counts once for each.  Waits for the
+ * pending launches.  HISQ_ERR_INVALID_ARG for a null argument. */
 hisq_status hisq_profiled_fp64(hisq_ctx *ctx, double *seconds, unsigned long long *launches);
 
 /* Failure injection on the host (tests of the error paths; the paper has no

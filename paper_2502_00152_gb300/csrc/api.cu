@@ -113,12 +113,21 @@ double *eig_eps_dev(hisq_ctx *ctx)
     return ctx->eig.eps_dev;
 }
 
+// a bounded device wait that ran out since the last check (after a synchronisation)
+hisq_status check_waits(hisq_ctx *ctx)
+{
+    const int code = *(volatile int *)ctx->wait_status_h;
+    if (code == 0) return HISQ_OK;
+    *ctx->wait_status_h = 0;
+    return set_err(ctx, HISQ_ERR_TIMEOUT, "operator: a pipeline wait ran out (code %d)", code);
+}
+
 // scalar slot readback (synchronises the stream)
 hisq_status read_slots(hisq_ctx *ctx, int slot0, int n, double *out)
 {
     HISQ_CUDA(cudaMemcpyAsync(out, &ctx->scal->slot[slot0], sizeof(double) * n, cudaMemcpyDeviceToHost, ctx->stream));
     HISQ_CUDA(cudaStreamSynchronize(ctx->stream));
-    return HISQ_OK;
+    return check_waits(ctx);
 }
 
 } // namespace hisq
@@ -373,7 +382,7 @@ static hisq_status download_full(hisq_ctx *ctx, const double *dev, double *host)
     const size_t bytes = size_t(ctx->g.V) * 6 * sizeof(double);
     HISQ_CUDA(cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, ctx->stream));
     HISQ_CUDA(cudaStreamSynchronize(ctx->stream));
-    return HISQ_OK;
+    return check_waits(ctx);
 }
 
 #define TRY(x)                                  \
@@ -484,12 +493,7 @@ hisq_status hisq_apply_dslash_batch(hisq_ctx *ctx, int out_parity, int precision
         HISQ_CUDA(cudaMemcpyAsync(out + size_t(j) * ctx->g.V * 6, full, full_bytes, cudaMemcpyDeviceToHost, ctx->stream));
         HISQ_CUDA(cudaStreamSynchronize(ctx->stream));
     }
-    if (*(volatile int *)ctx->wait_status_h != 0) {
-        const int code = *ctx->wait_status_h;
-        *ctx->wait_status_h = 0;
-        return set_err(ctx, HISQ_ERR_TIMEOUT, "batched operator: a pipeline wait ran out (code %d)", code);
-    }
-    return HISQ_OK;
+    return check_waits(ctx);
 }
 
 hisq_status hisq_inject_wait_timeout(hisq_ctx *ctx, int on)

@@ -14,7 +14,7 @@
 
 #include <algorithm>
 
-#include "internal.cuh"
+#include "fx64.cuh"
 
 namespace hisq {
 
@@ -54,7 +54,7 @@ static bool dual_residual(const hisq_ctx *ctx) { return ctx->eig.prec == 32; }
         if (s_ != HISQ_OK) return s_;           \
     } while (0)
 
-enum { BS_Y = 0, BS_ETAE = 1, BS_ETAO = 2, BS_R = 3, BS_RE = 4, BS_RO = 5, BS_PP = 6 };
+enum { BS_Y = 0, BS_ETAE = 1, BS_ETAO = 2, BS_R = 3, BS_RE = 4, BS_RO = 5, BS_PP = 6, BS_RHS = 16 };
 
 static hisq_status residual_hi_b(hisq_ctx *ctx, const double *b, const double *x, double *r, double *tmp_odd, int slot)
 {
@@ -102,6 +102,46 @@ static hisq_status set_active(hisq_ctx *ctx, const std::vector<int> &act)
                               ctx->stream));
     HISQ_CUDA(cudaStreamSynchronize(ctx->stream));
     return HISQ_OK;
+}
+
+// Right-hand sides whose FP64 operators run as one launch (fx64.cuh): scratch for
+// their mantissas (in, and of D_oe x) and D_oe x, 148 B per site and right-hand side.
+// At most kFxGroup, and no more than an eighth of the free device memory, so that the
+// buffers a solve allocates later still fit; with room for one only, the operators run
+// one by one.  (Four share the links well enough: 576 B of links per site and right-hand
+// side pass in 27 clocks beside 40 clocks of arithmetic.)
+struct FxScratch {
+    int group = 0;
+    char *mant = nullptr, *mant_t = nullptr;
+    double2 *t = nullptr;
+};
+static FxScratch fx_scratch(hisq_ctx *ctx, int k)
+{
+    FxScratch f;
+    const int Vh = ctx->g.Vh;
+    const size_t ms = fx_field_bytes(Vh), s64 = spinor_bytes(64, Vh);
+    int n = std::min(k, kFxGroup);
+    if (n > 1 && (ctx->buf_cap[BUF_FX] < 2 * ms * n || ctx->buf_cap[BUF_FX_T] < s64 * n)) {
+        // kept from an earlier call, or grown into an eighth of what is free
+        const int have = int(std::min(ctx->buf_cap[BUF_FX] / (2 * ms), ctx->buf_cap[BUF_FX_T] / s64));
+        size_t avail = 0, total = 0;
+        if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
+            cudaGetLastError();
+            avail = 0;
+        }
+        n = std::min(n, std::max(have, int(std::min(size_t(kFxGroup), avail / 8 / (2 * ms + s64)))));
+    }
+    if (n < 2) return f;
+    const std::string err = ctx->err;
+    f.mant = (char *)get_buf(ctx, BUF_FX, 2 * ms * n);
+    f.t = f.mant ? (double2 *)get_buf(ctx, BUF_FX_T, s64 * n) : nullptr;
+    if (!f.t) {
+        ctx->err = err;
+        return FxScratch{};
+    }
+    f.mant_t = f.mant + ms * n;
+    f.group = n;
+    return f;
 }
 
 // Solve M psi_j = eta_j for k <= kMaxBatch right-hand sides together; eta, psi:
@@ -197,11 +237,40 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
     std::vector<char> tok(k, 0), tval(k, 0);
     // |r_e|^2 of the full residual left by the FP64 confirmation of j (-1: none)
     std::vector<double> re2f(k, -1.0);
+    std::vector<const double *> tsrc(k, t_hi); // where the D_oe x_j of tok[j] lies
     auto keep_t = [&](int j) -> hisq_status {
         if (!tok[j]) return HISQ_OK;
-        HISQ_CUDA(cudaMemcpyAsync(rh(j), t_hi, s64, cudaMemcpyDeviceToDevice, ctx->stream));
+        HISQ_CUDA(cudaMemcpyAsync(rh(j), tsrc[j], s64, cudaMemcpyDeviceToDevice, ctx->stream));
         tval[j] = 1;
         return HISQ_OK;
+    };
+    // groups of right-hand sides for the FP64 operators that share their links
+    if (P->precision_reliable == HISQ_PREC_DF64) TRY(ensure_df_links(ctx)); // before the optional scratch
+    const FxScratch fx = fx_scratch(ctx, k);
+    auto fx_groups = [&](const std::vector<int> &ids, auto &&run) -> hisq_status {
+        for (size_t q0 = 0; q0 < ids.size(); q0 += fx.group) {
+            FxGroup g;
+            g.k = int(std::min(ids.size() - q0, size_t(fx.group)));
+            for (int q = 0; q < g.k; q++) g.id[q] = ids[q0 + q];
+            TRY(run(g));
+        }
+        return HISQ_OK;
+    };
+    const FxArray fx_x{(double2 *)XH, false}, fx_y{(double2 *)Y, false}, fx_r{(double2 *)RH, false}, fx_t{fx.t, true},
+        fx_none{nullptr, false};
+    double fx_norm[kMaxBatch]; // |out|^2 by right-hand side
+    auto fx_norms = [&]() -> hisq_status {
+        HISQ_CUDA(cudaMemcpyAsync(fx_norm, ctx->bscal->out, sizeof fx_norm, cudaMemcpyDeviceToHost, ctx->stream));
+        HISQ_CUDA(cudaStreamSynchronize(ctx->stream));
+        return check_waits(ctx);
+    };
+    // r = y - A x of a group (x += the sloppy increment first, if given), D_oe x left in
+    // fx.t by slot
+    auto fx_residual = [&](const FxGroup &g, const void *add) -> hisq_status {
+        TRY(launch_fx_batch_split(ctx, g, fx_x, fx.mant, add));
+        TRY(launch_fx_batch(ctx, 1, g, FxBatch{fx_x, fx_t, fx_none, fx_none, 0, 0, 1.0, fx.mant, fx.mant_t, false}));
+        TRY(launch_fx_batch(ctx, 0, g, FxBatch{fx_t, fx_r, fx_x, fx_y, -m4, 1.0, 1.0, fx.mant_t, nullptr, true}));
+        return fx_norms();
     };
     // the FP64 confirmation is the even part of the full residual (see
     // cg_reliable in solver.cu): t = D_oe x_j, psi_o = (eta_o - t) / 2m,
@@ -218,6 +287,7 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
         TRY(read_slots(ctx, BS_R, 1, &re2));
         rt[j] = 2.0 * m * std::sqrt(re2);
         tok[j] = 1;
+        tsrc[j] = t_hi;
         re2f[j] = re2;
         if (!(rt[j] <= target[j])) {
             // not confirmed: rh(j) = 2m r_e = y_j - A x_j, FP64 residuals from here
@@ -230,24 +300,53 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
         return HISQ_OK;
     };
 
-    // (a2) sources, (a8) deflated guesses
-    for (int j = 0; j < k; j++) {
-        const double *e = eta + full * j;
-        TRY(launch_gather_parity(ctx, e, 0, 64, eta_e));
-        TRY(launch_gather_parity(ctx, e, 1, 64, eta_o));
-        TRY(launch_norm2(ctx, 64, eta_e, BS_ETAE));
-        TRY(launch_norm2(ctx, 64, eta_o, BS_ETAO));
-        TRY(launch_dslash(ctx, 0, 64, 64, eta_o, y(j), 2.0 * m, eta_e, 0, nullptr, -1.0, BS_Y));
-        double nrm[3];
-        TRY(read_slots(ctx, BS_Y, 3, nrm));
-        ynorm[j] = std::sqrt(nrm[0]);
-        etanorm[j] = std::sqrt(nrm[1] + nrm[2]);
+    // (a2) sources
+    auto source_norms = [&](int j, double y2, double e2, double o2) -> hisq_status {
+        ynorm[j] = std::sqrt(y2);
+        etanorm[j] = std::sqrt(e2 + o2);
         if (!std::isfinite(ynorm[j]) || !std::isfinite(etanorm[j]))
             return set_err(ctx, HISQ_ERR_NUMERICAL, "non-finite source %d", j);
         target[j] = P->tol * std::fmin(ynorm[j], 2.0 * m * etanorm[j]);
         HISQ_CUDA(cudaMemsetAsync(xh(j), 0, s64, ctx->stream));
-        if (P->guess) { // start from the caller's guess (even sites of psi_j)
+        return HISQ_OK;
+    };
+    std::vector<int> all(k);
+    for (int j = 0; j < k; j++) all[j] = j;
+    if (fx.group > 1) {
+        // eta_e in y, eta_o in r: y = 2m eta_e - D_eo eta_o for a group at a time
+        TRY(fx_groups(all, [&](const FxGroup &g) -> hisq_status {
+            for (int q = 0; q < g.k; q++) {
+                const int j = g.id[q];
+                TRY(launch_gather_parity(ctx, eta + full * j, 0, 64, y(j)));
+                TRY(launch_gather_parity(ctx, eta + full * j, 1, 64, rh(j)));
+                TRY(launch_norm2(ctx, 64, y(j), BS_RHS + 2 * j));
+                TRY(launch_norm2(ctx, 64, rh(j), BS_RHS + 2 * j + 1));
+            }
+            TRY(launch_fx_batch_split(ctx, g, fx_r, fx.mant, nullptr));
+            return launch_fx_batch(ctx, 0, g, FxBatch{fx_r, fx_y, fx_y, fx_none, 2.0 * m, 0, -1.0, fx.mant, nullptr, true});
+        }));
+        double n2[2 * kMaxBatch];
+        TRY(fx_norms());
+        TRY(read_slots(ctx, BS_RHS, 2 * k, n2));
+        for (int j = 0; j < k; j++) TRY(source_norms(j, fx_norm[j], n2[2 * j], n2[2 * j + 1]));
+    } else {
+        for (int j = 0; j < k; j++) {
+            const double *e = eta + full * j;
+            TRY(launch_gather_parity(ctx, e, 0, 64, eta_e));
+            TRY(launch_gather_parity(ctx, e, 1, 64, eta_o));
+            TRY(launch_norm2(ctx, 64, eta_e, BS_ETAE));
+            TRY(launch_norm2(ctx, 64, eta_o, BS_ETAO));
+            TRY(launch_dslash(ctx, 0, 64, 64, eta_o, y(j), 2.0 * m, eta_e, 0, nullptr, -1.0, BS_Y));
+            double nrm[3];
+            TRY(read_slots(ctx, BS_Y, 3, nrm));
+            TRY(source_norms(j, nrm[0], nrm[1], nrm[2]));
+        }
+    }
+    // the starting point: zero, or the caller's guess (even sites of psi_j)
+    for (int j = 0; j < k; j++) {
+        if (P->guess) {
             TRY(launch_gather_parity(ctx, psi + full * j, 0, 64, xh(j)));
+            if (fx.group > 1) continue;
             TRY(residual_hi_b(ctx, y(j), xh(j), rh(j), t_hi, BS_R));
             double r2;
             TRY(read_slots(ctx, BS_R, 1, &r2));
@@ -257,6 +356,13 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
             rt[j] = ynorm[j];
         }
     }
+    if (P->guess && fx.group > 1)
+        TRY(fx_groups(all, [&](const FxGroup &g) -> hisq_status {
+            TRY(fx_residual(g, nullptr));
+            for (int q = 0; q < g.k; q++) rt[g.id[q]] = std::sqrt(fx_norm[g.id[q]]);
+            return HISQ_OK;
+        }));
+    // (a8) deflated guesses
     // deflated guesses of all right-hand sides: one tensor-core projection and
     // one expansion for the whole batch, else one pair of passes per RHS
     if (n_defl > 0) {
@@ -491,16 +597,8 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
         } else {
             gdf.clear();
         }
-        for (int j : upd) {
-            // reliable update of right-hand side j (FP64 or double-float true residual)
-            double r2;
-            if (std::find(gdf.begin(), gdf.end(), j) != gdf.end()) {
-                r2 = r2df[j];
-            } else {
-                TRY(launch_axpy_d(ctx, 1.0, xs(j), xprec, xh(j)));
-                TRY(residual_rel(ctx, use_df[j], y(j), xh(j), rh(j), t_hi, BS_R));
-                TRY(read_slots(ctx, BS_R, 1, &r2));
-            }
+        // reliable update of right-hand side j, whose new |r|^2 is r2 (FP64 or double-float)
+        auto update = [&](int j, double r2) -> hisq_status {
             tok[j] = !use_df[j];
             if (!std::isfinite(r2)) return set_err(ctx, HISQ_ERR_NUMERICAL, "non-finite true residual");
             rt[j] = std::sqrt(r2);
@@ -524,14 +622,40 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
                 TRY(keep_t(j));
                 done[j] = 1;
                 changed = true;
-                continue;
+                return HISQ_OK;
             }
             const bool restart = rt[j] > 10.0 * rn_seen[j];
             if (n_defl > 0 && P->delta_tr > 0 && rt[j] < P->delta_tr * r_defl[j]) {
                 redefl.push_back(j);
-                continue;
+                return HISQ_OK;
             }
-            TRY(finalize(j, restart));
+            return finalize(j, restart);
+        };
+        // the FP64 residuals of this round by groups, the others one by one
+        std::vector<int> g64;
+        for (int j : upd)
+            if (!use_df[j]) g64.push_back(j);
+        if (fx.group < 2 || g64.size() < 2) g64.clear();
+        TRY(fx_groups(g64, [&](const FxGroup &g) -> hisq_status {
+            TRY(fx_residual(g, XS));
+            for (int q = 0; q < g.k; q++) {
+                tsrc[g.id[q]] = (const double *)(fx.t + size_t(3) * Vh * q);
+                TRY(update(g.id[q], fx_norm[g.id[q]]));
+            }
+            return HISQ_OK;
+        }));
+        for (int j : upd) {
+            if (std::find(g64.begin(), g64.end(), j) != g64.end()) continue;
+            double r2;
+            if (std::find(gdf.begin(), gdf.end(), j) != gdf.end()) {
+                r2 = r2df[j];
+            } else {
+                TRY(launch_axpy_d(ctx, 1.0, xs(j), xprec, xh(j)));
+                TRY(residual_rel(ctx, use_df[j], y(j), xh(j), rh(j), t_hi, BS_R));
+                TRY(read_slots(ctx, BS_R, 1, &r2));
+            }
+            tsrc[j] = t_hi;
+            TRY(update(j, r2));
         }
         // re-deflations of this round, together on the tensor cores when possible
         if (!redefl.empty()) {
@@ -577,17 +701,50 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
 
     // (a9) reconstruction and FP64 full residuals
     hisq_status worst = HISQ_OK;
+    // right-hand sides that finished on an FP64 residual of their last x, whose D_oe x
+    // was kept and whose |r_e|^2 is still to be formed: by groups, psi_o in the place
+    // of y, which is no longer needed
+    std::vector<int> gfin;
+    if (fx.group > 1 && P->compute_full_residual)
+        for (int j = 0; j < k; j++)
+            if (tval[j] && etanorm[j] > 0 && re2f[j] < 0) gfin.push_back(j);
+    if (gfin.size() < 2) gfin.clear();
+    double ro2[2 * kMaxBatch];
+    TRY(fx_groups(gfin, [&](const FxGroup &g) -> hisq_status {
+        for (int q = 0; q < g.k; q++) {
+            const int j = g.id[q];
+            TRY(launch_gather_parity(ctx, eta + full * j, 0, 64, fx.t + size_t(3) * Vh * q));
+            TRY(launch_gather_parity(ctx, eta + full * j, 1, 64, eta_o));
+            TRY(odd_from_t(ctx, m, eta_o, rh(j), y(j)));
+            TRY(odd_residual_from_t(ctx, m, eta_o, y(j), rh(j), BS_RHS + j));
+        }
+        // r_e = eta_e - 2m x - D_eo psi_o, its norm only
+        TRY(launch_fx_batch_split(ctx, g, fx_y, fx.mant, nullptr));
+        return launch_fx_batch(ctx, 0, g, FxBatch{fx_y, fx_none, fx_x, fx_t, -2.0 * m, 1.0, -1.0, fx.mant, nullptr, true});
+    }));
+    if (!gfin.empty()) {
+        TRY(fx_norms());
+        TRY(read_slots(ctx, BS_RHS, k, ro2));
+    }
     for (int j = 0; j < k; j++) {
         const double *e = eta + full * j;
         double *out = psi + full * j;
-        TRY(launch_gather_parity(ctx, e, 0, 64, eta_e));
-        TRY(launch_gather_parity(ctx, e, 1, 64, eta_o));
-        if (tval[j]) {
+        const bool grouped = std::find(gfin.begin(), gfin.end(), j) != gfin.end();
+        const double *odd = grouped ? y(j) : psi_o;
+        if (!grouped) {
+            TRY(launch_gather_parity(ctx, e, 0, 64, eta_e));
+            TRY(launch_gather_parity(ctx, e, 1, 64, eta_o));
+        }
+        if (grouped) {
+            st[j].full_residual = std::sqrt(fx_norm[j] + ro2[j]) / etanorm[j];
+        } else if (tval[j]) {
             TRY(odd_from_t(ctx, m, eta_o, rh(j), psi_o));
         } else {
             TRY(launch_dslash(ctx, 1, 64, 64, xh(j), psi_o, 1.0 / (2.0 * m), eta_o, 0, nullptr, -1.0 / (2.0 * m), -1));
         }
-        if (P->compute_full_residual && etanorm[j] > 0) {
+        if (grouped) {
+            // formed above
+        } else if (P->compute_full_residual && etanorm[j] > 0) {
             double rr[2] = {re2f[j], 0.0};
             if (tval[j]) {
                 // an FP64 confirmation of this x_j has already formed |r_e|^2
@@ -609,7 +766,7 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
             st[j].full_residual = 0;
         }
         TRY(launch_scatter_parity(ctx, xh(j), 64, 0, out));
-        TRY(launch_scatter_parity(ctx, psi_o, 64, 1, out));
+        TRY(launch_scatter_parity(ctx, odd, 64, 1, out));
         st[j].iterations = its[j];
         st[j].even_residual = ynorm[j] > 0 ? rt[j] / ynorm[j] : 0;
         if (!st[j].converged) worst = HISQ_ERR_NOT_CONVERGED;

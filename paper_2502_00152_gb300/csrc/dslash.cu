@@ -210,77 +210,74 @@ static int blocks_per_sm(K kernel)
 }
 
 // ------------------------------------------------- the FP64 kernel
-// Fixed-point sums (fx64.cuh) of FP64 links and vectors, one thread per site, or
-// SPLIT = 4 warps per group of 32 sites, one per direction, whose integer sums are
-// added in shared memory (exact, so the result is the same bit for bit).
+// Fixed-point sums (fx64.cuh) of FP64 links and one FP64 field, one thread per site, or
+// SPLIT = 4 warps per group of 32 sites, one per direction, whose integer sums are added
+// in shared memory (exact, so the result is the same bit for bit).
 //
-// Bound by the 2304 B of links per site.  Each thread holds the links and the
-// neighbour of two hops (96 registers), so that a warp has 6.5 KB of loads in flight
-// while it multiplies; 4 blocks of 128 threads at 128 registers (136 B spilled) gave
-// 441 us per application on 32^3x64 (split included), 3 blocks at 168 registers 470,
-// 2 at 206 registers 510, blocks of 64 or 32 threads 455 to 471, one hop in flight as
-// the compiler ordered the loads 812; the FP64 kernel took 1040.
+// Bound by the 2304 B of links per site.  Each thread holds the links and the neighbour
+// of two hops (100 registers), so that a warp has 6.5 KB of loads in flight while it
+// multiplies.  32^3x64, split of the input included: 417 us per application at 168
+// registers (12 warps per SM), 500 at 128 (432 B spilled), 513 with the links in shared
+// memory as the batch has them; FP64 FMAs took 1040.
 //
 // Split where one thread per site leaves fewer than 16 warps per SM: 8^4 16 us per
-// application instead of 23, 14x10x12x22 26.7 instead of 27.3, 16^3x32 even; on
-// 24^3x48 (68 warps per SM) the split costs 181 instead of 162.
+// application instead of 23, 14x10x12x22 24 instead of 27, 16^3x32 even; on 24^3x48 (68
+// warps per SM) the split costs 181 instead of 146.
 constexpr int kFxSplitWarps = 16;
 
 template <class Epi, int SPLIT>
-__global__ void __launch_bounds__(128, SPLIT == 1 ? 4 : 3)
-    k_dslash_fx(Geom g, int par, LinksX L, FxField in0, Epi epi, RedArgs ra, int do_red, int fp64)
+__global__ void __launch_bounds__(128, 3)
+    k_dslash_fx(Geom g, int par, LinksX L, FxField in, Epi epi, RedArgs ra, int do_red, int fp64)
 {
     constexpr int kGroups = SPLIT == 1 ? 4 : 1; // site groups of a block
-    __shared__ long long sh[SPLIT == 1 ? 1 : 3][12][32];
+    __shared__ long long sh[SPLIT == 1 ? 1 : 3][18][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int grp = SPLIT == 1 ? warp : 0, part = SPLIT == 1 ? 0 : warp;
+    const int part = SPLIT == 1 ? 0 : warp;
     double red = 0;
     for (int b0 = blockIdx.x * kGroups * 32; b0 < g.Vh; b0 += gridDim.x * kGroups * 32) {
-        const int cb = b0 + grp * 32 + lane;
-        const bool on = cb < g.Vh;
-        int c[4] = {0, 0, 0, 0}, s = 0, le = 0, E[1] = {0};
-        FxAcc acc[1];
-        acc[0].zero();
-        const FxField in[1] = {in0};
-        const int4 *w = L.w + fx_link_index(on ? cb : 0, 0);
-        if (on) {
-            cb_coords(g, par, cb, c);
-            s = full_site(g, c);
-            le = L.e[cb];
-            E[0] = fp64 ? kFxMark : fx_site_exponent(g, c, s, in0.e);
-            if (E[0] != kFxMark && le != kFxMark) {
-                if (SPLIT == 1)
-                    fx_directions<1, false>(g, c, s, 0, 4, w, in, E, acc);
-                else
-                    fx_directions<1, false>(g, c, s, part, part + 1, w, in, E, acc);
-            }
-        }
+        const int at = b0 + (SPLIT == 1 ? warp * 32 : 0) + lane;
+        const int cb = min(at, g.Vh - 1);
+        int c[4];
+        cb_coords(g, par, cb, c);
+        const int s = full_site(g, c);
+        const int4 *w = L.w + fx_link_index(cb, 0);
+        const int le = L.e[cb], E = fp64 ? kFxMark : fx_site_exponent(g, c, s, in.e);
+        const bool mark = E == kFxMark || le == kFxMark;
+        FxAcc acc;
+        acc.zero();
+        if (!mark) fx_directions(g, c, s, SPLIT == 1 ? 0 : part, SPLIT == 1 ? 4 : part + 1, w, in, E, acc);
         if (SPLIT > 1) {
             if (part > 0) {
 #pragma unroll
-                for (int k = 0; k < 6; k++) {
-                    sh[part - 1][k][lane] = acc[0].h[k];
-                    sh[part - 1][6 + k][lane] = acc[0].m[k];
+                for (int k = 0; k < 9; k++) {
+                    sh[part - 1][k][lane] = acc.h[k / 3][k % 3];
+                    sh[part - 1][9 + k][lane] = acc.m[k / 3][k % 3];
                 }
             }
             __syncthreads();
             if (part == 0) {
 #pragma unroll
-                for (int k = 0; k < 6; k++)
+                for (int k = 0; k < 9; k++)
 #pragma unroll
-                    for (int w = 0; w < 3; w++) {
-                        acc[0].h[k] += sh[w][k][lane];
-                        acc[0].m[k] += sh[w][6 + k][lane];
+                    for (int u = 0; u < 3; u++) {
+                        acc.h[k / 3][k % 3] += sh[u][k][lane];
+                        acc.m[k / 3][k % 3] += sh[u][9 + k][lane];
                     }
             }
             __syncthreads();
         }
-        if (on && part == 0) {
+        if (at < g.Vh && part == 0) {
             CVec<double> o;
-            if (E[0] != kFxMark && le != kFxMark)
-                o = fx_value(acc[0], E[0], le);
-            else
-                o = fx_site_fp64(g, c, s, w, le, in0.src);
+            if (!mark) {
+                const double u = fx_unit(E, le);
+#pragma unroll
+                for (int i = 0; i < 3; i++) {
+                    o.re[i] = double(fx_sum(acc, 2 * i)) * u;
+                    o.im[i] = double(fx_sum(acc, 2 * i + 1)) * u;
+                }
+            } else {
+                o = fx_site_fp64(g, c, s, w, le, in.src);
+            }
             epi(cb, o, red);
         }
     }
@@ -320,17 +317,17 @@ static hisq_status run_fx(hisq_ctx *ctx, int par, const SpinorD &in, const Epi &
     }
     const LinksX L{ctx->links_x[par], ctx->links_xe[par]};
     const FxField f = fx_field(buf, in.p, Vh);
-    auto launch = [&](auto kern, int threads, int sites, int *bps) -> hisq_status {
-        if (*bps < 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, kern, threads, 0) != cudaSuccess || *bps < 1))
+    auto launch = [&](auto kern, int sites, int *bps) -> hisq_status {
+        if (*bps < 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, kern, 128, 0) != cudaSuccess || *bps < 1))
             *bps = 1;
         const int grid = grid_for(ctx, Vh, sites, *bps);
-        kern<<<grid, threads, 0, ctx->stream>>>(ctx->g, par, L, f, epi, ra, do_red, buf ? 0 : 1);
+        kern<<<grid, 128, 0, ctx->stream>>>(ctx->g, par, L, f, epi, ra, do_red, buf ? 0 : 1);
         const cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? HISQ_OK : cuda_err(ctx, e, "FP64 dslash launch");
     };
     static int bps1 = -1, bps4 = -1;
-    if (Vh < ctx->num_sms * 32 * kFxSplitWarps) return launch(k_dslash_fx<Epi, 4>, 128, 32, &bps4);
-    return launch(k_dslash_fx<Epi, 1>, 128, 128, &bps1);
+    if (Vh < ctx->num_sms * 32 * kFxSplitWarps) return launch(k_dslash_fx<Epi, 4>, 32, &bps4);
+    return launch(k_dslash_fx<Epi, 1>, 128, &bps1);
 }
 
 // Run the Dslash with output parity `par` on links of precision link_prec
@@ -381,7 +378,7 @@ void fp64_prof_drain(hisq_ctx *ctx, bool all, bool discard)
         float ms = 0;
         if (!discard && cudaEventElapsedTime(&ms, e.first, e.second) == cudaSuccess) {
             ctx->fp64_seconds += 1e-3 * ms;
-            ctx->fp64_launches++;
+            ctx->fp64_launches += e.fields;
         }
         cudaGetLastError();
         ctx->fp64_pool.push_back(e.first);
@@ -399,10 +396,22 @@ static hisq_status dslash_xpay(hisq_ctx *ctx, int out_parity, int prec, int link
 hisq_status launch_dslash(hisq_ctx *ctx, int out_parity, int prec, int link_prec, const void *in, void *out, double a,
                           const void *x, double b, const void *y, double c, int norm_slot)
 {
+    bool timed = false;
+    if (prec == 64) {
+        const hisq_status b0 = fp64_prof_begin(ctx, 1, &timed);
+        if (b0 != HISQ_OK) return b0;
+    }
+    const hisq_status st = dslash_xpay(ctx, out_parity, prec, link_prec, in, out, a, x, b, y, c, norm_slot);
+    const hisq_status e0 = fp64_prof_end(ctx, timed);
+    return st != HISQ_OK ? st : e0;
+}
+
+hisq_status fp64_prof_begin(hisq_ctx *ctx, int fields, bool *on)
+{
+    *on = false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (prec != 64 || !ctx->profile || cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess ||
-        cap != cudaStreamCaptureStatusNone)
-        return dslash_xpay(ctx, out_parity, prec, link_prec, in, out, a, x, b, y, c, norm_slot);
+    if (!ctx->profile || cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+        return HISQ_OK;
     cudaEvent_t e[2];
     for (int i = 0; i < 2; i++) {
         if (!ctx->fp64_pool.empty()) {
@@ -413,11 +422,17 @@ hisq_status launch_dslash(hisq_ctx *ctx, int out_parity, int prec, int link_prec
         }
     }
     HISQ_CUDA(cudaEventRecord(e[0], ctx->stream));
-    const hisq_status st = dslash_xpay(ctx, out_parity, prec, link_prec, in, out, a, x, b, y, c, norm_slot);
-    HISQ_CUDA(cudaEventRecord(e[1], ctx->stream));
-    ctx->fp64_pending.emplace_back(e[0], e[1]);
+    ctx->fp64_pending.push_back({e[0], e[1], fields});
+    *on = true;
+    return HISQ_OK;
+}
+
+hisq_status fp64_prof_end(hisq_ctx *ctx, bool on)
+{
+    if (!on) return HISQ_OK;
+    HISQ_CUDA(cudaEventRecord(ctx->fp64_pending.back().second, ctx->stream));
     fp64_prof_drain(ctx, ctx->fp64_pending.size() > 4096);
-    return st;
+    return HISQ_OK;
 }
 
 static hisq_status dslash_xpay(hisq_ctx *ctx, int out_parity, int prec, int link_prec, const void *in, void *out,

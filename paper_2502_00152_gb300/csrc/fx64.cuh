@@ -2,12 +2,13 @@
 // units.
 //
 // GB300 retires 1.68 FP64 FMAs per clock and SM (measured), so an FP64 Dslash
-// (576 complex-matrix FMAs per site and right-hand side) takes 343 clocks per site
-// and SM where its 2.4 KB of links take 111 from HBM.  32 x 32 -> 64 bit integer
-// multiply-adds run at 64 per clock and SM (measured), so the same sums are formed
-// here from 56-bit mantissas held as two 28-bit limbs, three multiply-adds per real
-// product (the product of the two low limbs, below 2^-57 of the largest term, is
-// dropped): 27 clocks, and HBM becomes the bound for one right-hand side.
+// (576 FMAs per site and right-hand side) takes 343 clocks per site and SM where its
+// 2.4 KB of links take 111 from HBM.  32 x 32 + 64 bit integer multiply-adds run at 30
+// per clock and SM (measured; the 64-bit additions of the ALU pipe pass beside them), so
+// the same sums are formed here from 56-bit mantissas held as two 28-bit limbs.  A real
+// product takes three multiply-adds (the product of the two low limbs, below 2^-57 of
+// the largest term, is dropped) and a complex one three real products instead of four
+// (Karatsuba's identity, see FxAcc): 1296 multiply-adds, 43 clocks per site.
 //
 // Block floating point: the six reals of a colour vector share the exponent of the
 // largest one, the 288 link reals of an output site share theirs, and at an output
@@ -34,6 +35,7 @@
 #pragma once
 
 #include "internal.cuh"
+#include "tc.cuh"
 
 namespace hisq {
 
@@ -83,6 +85,27 @@ __device__ __forceinline__ long long fx_mantissa(double x, int eb)
     return b < 0 ? -(long long)m : (long long)m;
 }
 
+// one site's vector to mantissas and exponent; marked sites keep no mantissas
+__device__ __forceinline__ void fx_store_site(longlong2 *v, short *e, int Vh, int i, const CVec<double> &q)
+{
+    int eb = 0;
+    bool zero = true;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        eb = max(eb, max(fx_exponent(q.re[c]), fx_exponent(q.im[c])));
+        zero = zero && q.re[c] == 0.0 && q.im[c] == 0.0;
+    }
+    if (!zero && (eb < kFxVecLo || eb > kFxVecHi)) {
+        e[i] = short(kFxMark); // the operator reads the FP64 field at the sites this one touches
+        return;
+    }
+    if (zero) eb = kFxVecLo; // below every other exponent, mantissas 0
+    e[i] = short(eb);
+#pragma unroll
+    for (int c = 0; c < 3; c++)
+        v[size_t(c) * Vh + i] = make_longlong2(fx_mantissa<7>(q.re[c], eb), fx_mantissa<7>(q.im[c], eb));
+}
+
 // limbs of a mantissa, |v| <= 2^56
 __device__ __forceinline__ void fx_limbs(long long v, int &hi, int &lo)
 {
@@ -110,24 +133,21 @@ __device__ __forceinline__ double2 fx_link(int4 q, int eb)
     return make_double2(fma(double(q.x), s1, double(q.y) * s0), fma(double(q.z), s1, double(q.w) * s0));
 }
 
-// sums of the integer products of one right-hand side: value of component c is
-// (h[c] 2^56 + m[c] 2^28) times the shared scale; c = 2 * colour + (0: re, 1: im)
+// Sums of the integer products of one right-hand side.  With W = a + ib and v = c + id,
+//   k1 = c (a + b),  k2 = a (d - c),  k3 = b (c + d):  Re W v = k1 - k3,  Im W v = k1 + k2,
+// and the three are summed separately over the 16 hops and 3 colours of row i, [row][k];
+// value: (h 2^56 + m 2^28) times the shared scale.  Single sums may wrap around 2^64, the
+// differences that are used at the end fit (above), so they are exact.
 struct FxAcc {
-    long long h[6], m[6];
+    long long h[3][3], m[3][3];
     __device__ __forceinline__ void zero()
     {
 #pragma unroll
-        for (int c = 0; c < 6; c++) h[c] = m[c] = 0;
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+            for (int k = 0; k < 3; k++) h[i][k] = m[i][k] = 0;
     }
 };
-
-// h 2^56 + m 2^28 += (ah 2^28 + al)(bh 2^28 + bl) without al bl: three IMAD.WIDE
-__device__ __forceinline__ void fx_mac(long long &h, long long &m, int ah, int al, int bh, int bl)
-{
-    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(h) : "r"(ah), "r"(bh));
-    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(m) : "r"(ah), "r"(bl));
-    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(m) : "r"(al), "r"(bh));
-}
 
 // the shared exponent of the 16 neighbours of a site (kFxMark if one is marked)
 __device__ __forceinline__ int fx_site_exponent(const Geom &g, const int c[4], int s, const short *e)
@@ -141,104 +161,129 @@ __device__ __forceinline__ int fx_site_exponent(const Geom &g, const int c[4], i
     return E;
 }
 
-// One hop of a site in flight: its link matrix and the neighbour's vector of R
-// right-hand sides.  hop = 4 mu + (0: fat fwd, 1: fat bwd, 2: long fwd, 3: long bwd).
-// KEEP: the links go through L1 (other warps of the block read the same lines), else
-// they are streamed.
-template <int R, bool KEEP>
-struct FxHop {
-    int4 w[9];
-    longlong2 v[R][3];
-    int e[R];
-    __device__ __forceinline__ void load(const Geom &g, const int c[4], int s, int mu, int h, const int4 *L,
-                                         const FxField (&in)[R])
+// What the four neighbours of a site along mu share.
+struct FxLine {
+    int base, cm, L, stride; // neighbour at distance d: (base + wrapped(cm + d) * stride) / 2
+    __device__ __forceinline__ FxLine(const Geom &g, const int c[4], int s, int mu)
     {
-        const int nb = nb_cb(g, c, s, mu, (h & 2 ? 3 : 1) * (h & 1 ? -1 : 1));
-        const int4 *p = L + (mu * 4 + h) * (9 * 32);
-#pragma unroll
-        for (int k = 0; k < 9; k++) w[k] = KEEP ? __ldg(p + 32 * k) : __ldcs(p + 32 * k);
-#pragma unroll
-        for (int r = 0; r < R; r++) {
-            e[r] = __ldg(in[r].e + nb);
-#pragma unroll
-            for (int j = 0; j < 3; j++) v[r][j] = __ldg(in[r].v + size_t(j) * g.Vh + nb);
-        }
+        L = dim_of(g, mu);
+        cm = coord_of(c, mu);
+        stride = mu == 0 ? 1 : (mu == 1 ? g.stride[1] : (mu == 2 ? g.stride[2] : g.stride[3]));
+        base = s - cm * stride;
     }
-    // acc += W v, the vector shifted down to the site's exponent
-    __device__ __forceinline__ void add(const int (&E)[R], FxAcc (&acc)[R]) const
+    __device__ __forceinline__ int at(const Geom &g, int d) const
     {
-        int vh[R][6], vl[R][6], nh[R][3], nl[R][3]; // limbs, and those of -im
-#pragma unroll
-        for (int r = 0; r < R; r++) {
-            int d = E[r] - e[r];
-            longlong2 q[3] = {v[r][0], v[r][1], v[r][2]};
-            if (d > 31) { // a neighbour far below the largest one
-#pragma unroll
-                for (int j = 0; j < 3; j++) q[j] = make_longlong2(q[j].x >> 31, q[j].y >> 31);
-                d = min(d - 31, 31);
-            }
-#pragma unroll
-            for (int j = 0; j < 3; j++) {
-                fx_shifted_limbs(q[j].x, d, vh[r][2 * j], vl[r][2 * j]);
-                fx_shifted_limbs(q[j].y, d, vh[r][2 * j + 1], vl[r][2 * j + 1]);
-                nh[r][j] = -vh[r][2 * j + 1];
-                nl[r][j] = -vl[r][2 * j + 1];
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 3; i++)
-#pragma unroll
-            for (int j = 0; j < 3; j++) {
-                const int4 q = w[3 * i + j];
-#pragma unroll
-                for (int r = 0; r < R; r++) {
-                    FxAcc &a = acc[r];
-                    fx_mac(a.h[2 * i], a.m[2 * i], q.x, q.y, vh[r][2 * j], vl[r][2 * j]);
-                    fx_mac(a.h[2 * i], a.m[2 * i], q.z, q.w, nh[r][j], nl[r][j]);
-                    fx_mac(a.h[2 * i + 1], a.m[2 * i + 1], q.x, q.y, vh[r][2 * j + 1], vl[r][2 * j + 1]);
-                    fx_mac(a.h[2 * i + 1], a.m[2 * i + 1], q.z, q.w, vh[r][2 * j], vl[r][2 * j]);
-                }
-            }
+        int cn = cm + d;
+        cn += cn < 0 ? L : 0;
+        cn -= cn >= L ? L : 0;
+        return checked_index(g, (base + cn * stride) >> 1, g.Vh);
     }
 };
 
-// directions mu0 .. mu1 - 1 of a site (L: its first link element): the loads of the next hop are issued before
-// the sums of the current one
-template <int R, bool KEEP>
-__device__ __forceinline__ void fx_directions(const Geom &g, const int c[4], int s, int mu0, int mu1, const int4 *L,
-                                              const FxField (&in)[R], const int (&E)[R],
-                                              FxAcc (&acc)[R])
+// the neighbour's vector of one hop.
+// hop = 4 mu + h, h = 0: fat fwd, 1: fat bwd, 2: long fwd, 3: long bwd.
+struct FxVec {
+    longlong2 v[3];
+    int e;
+    __device__ __forceinline__ void load(const Geom &g, const FxLine &line, int h, const FxField &in)
+    {
+        const unsigned nb = unsigned(line.at(g, (h & 2 ? 3 : 1) * (h & 1 ? -1 : 1)));
+        e = __ldg(in.e + nb);
+#pragma unroll
+        for (int j = 0; j < 3; j++) v[j] = __ldg(in.v + size_t(j) * g.Vh + nb);
+    }
+};
+
+// acc += W v, the vector shifted down to the site's exponent; link(k): element k of W
+template <class F>
+__device__ __forceinline__ void fx_add(const FxVec &x, int E, FxAcc &acc, F &&link)
 {
-    FxHop<R, KEEP> a, b;
-    a.load(g, c, s, mu0, 0, L, in);
+    int d = E - x.e;
+    longlong2 q[3] = {x.v[0], x.v[1], x.v[2]};
+    if (d > 31) { // a neighbour far below the largest one
+#pragma unroll
+        for (int j = 0; j < 3; j++) q[j] = make_longlong2(q[j].x >> 31, q[j].y >> 31);
+        d = min(d - 31, 31);
+    }
+    int vh[3][3], vl[3][3]; // limbs of c, d - c and c + d
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        int dh, dl;
+        fx_shifted_limbs(q[j].x, d, vh[j][0], vl[j][0]);
+        fx_shifted_limbs(q[j].y, d, dh, dl);
+        vh[j][1] = dh - vh[j][0];
+        vl[j][1] = dl - vl[j][0];
+        vh[j][2] = dh + vh[j][0];
+        vl[j][2] = dl + vl[j][0];
+    }
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const int4 w = link(3 * i + j);
+            const int wh[3] = {w.x + w.z, w.x, w.z}, wl[3] = {w.y + w.w, w.y, w.w};
+            // three independent sums between two additions to the same one
+#pragma unroll
+            for (int k = 0; k < 3; k++) acc.h[i][k] += (long long)wh[k] * vh[j][k];
+#pragma unroll
+            for (int k = 0; k < 3; k++) acc.m[i][k] += (long long)wh[k] * vl[j][k];
+#pragma unroll
+            for (int k = 0; k < 3; k++) acc.m[i][k] += (long long)wl[k] * vh[j][k];
+        }
+}
+
+// Directions mu0 .. mu1 - 1 of a site (L: its first link element), links in registers:
+// the loads of the next hop are issued before the sums of the current one.
+struct FxHop {
+    int4 w[9];
+    FxVec x;
+    __device__ __forceinline__ void load(const Geom &g, const FxLine &line, int mu, int h, const int4 *L,
+                                         const FxField &in)
+    {
+        const int4 *p = L + (mu * 4 + h) * (9 * 32);
+#pragma unroll
+        for (int k = 0; k < 9; k++) w[k] = __ldcs(p + 32 * k); // read once per launch
+        x.load(g, line, h, in);
+    }
+    __device__ __forceinline__ void add(int E, FxAcc &acc) const
+    {
+        fx_add(x, E, acc, [&](int k) { return w[k]; });
+    }
+};
+__device__ __forceinline__ void fx_directions(const Geom &g, const int c[4], int s, int mu0, int mu1, const int4 *L,
+                                              const FxField &in, int E, FxAcc &acc)
+{
+    FxHop a, b;
+    FxLine line(g, c, s, mu0);
+    a.load(g, line, mu0, 0, L, in);
 #pragma unroll 1
     for (int mu = mu0; mu < mu1; mu++) {
-        b.load(g, c, s, mu, 1, L, in);
+        b.load(g, line, mu, 1, L, in);
         a.add(E, acc);
-        a.load(g, c, s, mu, 2, L, in);
+        a.load(g, line, mu, 2, L, in);
         b.add(E, acc);
-        b.load(g, c, s, mu, 3, L, in);
+        b.load(g, line, mu, 3, L, in);
         a.add(E, acc);
-        if (mu + 1 < mu1) a.load(g, c, s, mu + 1, 0, L, in);
+        if (mu + 1 < mu1) {
+            line = FxLine(g, c, s, mu + 1);
+            a.load(g, line, mu + 1, 0, L, in);
+        }
         b.add(E, acc);
     }
 }
 
-// the sums as FP64: carries of the middle sum into the high one, then one rounding
-__device__ __forceinline__ CVec<double> fx_value(const FxAcc &a, int E, int le)
+// the high sum with the carry of the middle one, rounded to the unit of h: at most 2^-57
+// of the largest product is lost, as in every term.  c = 2 * colour + (0: re, 1: im)
+__device__ __forceinline__ long long fx_sum(const FxAcc &a, int c)
 {
-    const int k = E + le - 2100; // unit of h: 2^56 2^(E - 1022 - 56) 2^(le - 1022 - 56)
-    const double s1 = fx_pow2(k), s0 = fx_pow2(k - 28);
-    CVec<double> o;
-#pragma unroll
-    for (int c = 0; c < 3; c++) {
-        const long long h0 = a.h[2 * c] + (a.m[2 * c] >> 28), h1 = a.h[2 * c + 1] + (a.m[2 * c + 1] >> 28);
-        const int l0 = int(a.m[2 * c] & 0xfffffffll), l1 = int(a.m[2 * c + 1] & 0xfffffffll);
-        o.re[c] = fma(double(h0), s1, double(l0) * s0);
-        o.im[c] = fma(double(h1), s1, double(l1) * s0);
-    }
-    return o;
+    const int i = c >> 1;
+    const long long h = c & 1 ? a.h[i][0] + a.h[i][1] : a.h[i][0] - a.h[i][2];
+    const long long m = c & 1 ? a.m[i][0] + a.m[i][1] : a.m[i][0] - a.m[i][2];
+    return h + ((m + (1ll << 27)) >> 28);
 }
+
+// unit of h: 2^56 2^(E - 1022 - 56) 2^(le - 1022 - 56)
+__device__ __forceinline__ double fx_unit(int E, int le) { return fx_pow2(E + le - 2100); }
 
 // a marked site (L: its first link element): FP64 FMAs on the original field
 static __device__ __noinline__ CVec<double> fx_site_fp64(const Geom &g, const int c[4], int s, const int4 *L, int le,
@@ -271,8 +316,179 @@ static __device__ __noinline__ CVec<double> fx_site_fp64(const Geom &g, const in
     return acc;
 }
 
+// ------------------------------------------------- links through shared memory
+// A warp computes 32 consecutive sites of one field; nch warps (fields) share a site
+// group, nsg groups share a block: warp = (group, field).  The links of a hop of a site
+// group are one contiguous 4.6 KB piece: one bulk copy into a ring of `stages` slots of
+// shared memory that the nch warps read, so that each link leaves HBM once for all of
+// them and takes no registers while it travels; the next hop's vector is loaded while the
+// current one is multiplied.  Every wait is bounded: one that runs out records its code
+// in *status, the warp gives up the rest of its sites, and the launch ends.
+constexpr int kFxHopBytes = 9 * 32 * 16;
+constexpr int kFxWarps = 8; // warps of a block at most
+
+struct FxTile {
+    int nch, nsg, stages;
+    __host__ __device__ size_t smem() const { return size_t(nsg) * stages * (kFxHopBytes + 2 * sizeof(uint64_t)); }
+};
+
+// site(cb, c, s, E, le, acc) for every site of this warp
+template <class F>
+__device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const LinksX &L, const FxField &in,
+                                              const FxTile &tl, int bx, int nbx, unsigned char *dsm, int *status,
+                                              F &&site)
+{
+    const int Vh = g.Vh, stages = tl.stages;
+    const int lane = threadIdx.x & 31, chunk = (threadIdx.x >> 5) % tl.nch, sg = (threadIdx.x >> 5) / tl.nch;
+    unsigned char *ring = dsm + size_t(sg) * stages * kFxHopBytes;
+    uint64_t *full = reinterpret_cast<uint64_t *>(dsm + size_t(tl.nsg) * stages * kFxHopBytes) + 2 * sg * stages;
+    uint64_t *empty = full + stages;
+    const bool producer = chunk == 0 && lane == 0;
+    if (producer) {
+        for (int q = 0; q < stages; q++) {
+            tc::mbar_init(&full[q], 1);
+            tc::mbar_init(&empty[q], tl.nch);
+        }
+        tc::fence_mbar_init();
+    }
+    __syncthreads();
+    const int ngroups = (Vh + 31) / 32;
+    const int first = bx * tl.nsg + sg, gstride = nbx * tl.nsg;
+    const int nitems = first < ngroups ? ((ngroups - 1 - first) / gstride + 1) * 16 : 0;
+    // item j: hop j % 16 of this group's (j / 16)-th 32 sites
+    int issued = 0, islot = 0; // items issued, and the slot of the next one
+    uint32_t iphase = 1;       // parity to wait for before the next one's slot is refilled
+    auto issue = [&]() {
+        uint64_t *fb = &full[islot];
+        tc::mbar_arrive_expect_tx(fb, kFxHopBytes);
+        tc::bulk_load_1d(ring + size_t(islot) * kFxHopBytes,
+                         L.w + fx_link_index((first + (issued >> 4) * gstride) * 32, (issued & 15) * 9), kFxHopBytes, fb);
+        issued++;
+        if (++islot == stages) {
+            islot = 0;
+            iphase ^= 1;
+        }
+    };
+    if (producer)
+        while (issued < min(stages, nitems)) issue();
+
+    bool ok = true;
+    int slot = 0;       // slot of the item in work
+    uint32_t phase = 0; // its parity
+#pragma unroll 1
+    for (int it = 0; it < nitems && ok; it += 16) {
+        const int at = (first + (it >> 4) * gstride) * 32 + lane;
+        const int cb = min(at, Vh - 1);
+        int c[4];
+        cb_coords(g, par, cb, c);
+        const int s = full_site(g, c);
+        const int le = L.e[cb];
+        const int E = fx_site_exponent(g, c, s, in.e);
+        FxAcc acc;
+        acc.zero();
+        // one hop: refill the ring, wait for the links, add
+        auto hop = [&](int j, const FxVec &cur) {
+            if (producer) {
+                // a slot is refilled once every warp of the group has released it; the
+                // producer blocks only when the hop its own warp needs now is not issued
+                while (ok && issued < nitems && issued < it + j + stages) {
+                    if (!tc::mbar_try_wait(&empty[islot], iphase)) {
+                        if (issued > it + j) break;
+                        ok = tc::mbar_wait(&empty[islot], iphase, status, tc::TC_TIMEOUT_EMPTY);
+                        if (!ok) break;
+                    }
+                    issue();
+                }
+            }
+            if (ok) ok = tc::mbar_wait(&full[slot], phase, status, tc::TC_TIMEOUT_FULL);
+            const int4 *w = reinterpret_cast<const int4 *>(ring + size_t(slot) * kFxHopBytes) + lane;
+            if (ok) fx_add(cur, E, acc, [&](int k) { return w[32 * k]; });
+            ok = __all_sync(0xffffffffu, ok);
+            if (lane == 0 && ok) tc::mbar_arrive(&empty[slot]);
+            if (++slot == stages) {
+                slot = 0;
+                phase ^= 1;
+            }
+        };
+        FxVec a, b;
+        FxLine line(g, c, s, 0);
+        a.load(g, line, 0, in);
+#pragma unroll 1
+        for (int mu = 0; mu < 4; mu++) {
+            b.load(g, line, 1, in);
+            hop(4 * mu, a);
+            a.load(g, line, 2, in);
+            hop(4 * mu + 1, b);
+            b.load(g, line, 3, in);
+            hop(4 * mu + 2, a);
+            if (mu < 3) {
+                line = FxLine(g, c, s, mu + 1);
+                a.load(g, line, 0, in);
+            }
+            hop(4 * mu + 3, b);
+        }
+        if (ok && at < Vh) site(cb, c, s, E, le, acc);
+    }
+    // copies still in flight (only after a wait gave up) land before the block ends
+    if (producer && !ok)
+        for (int q = 0; q < stages; q++) {
+            // the last item issued into slot q, if any: its parity follows from how often it was used
+            const int uses = (issued + stages - 1 - q) / stages;
+            if (uses > 0)
+                for (int spin = 0; spin < (1 << 20) && !tc::mbar_try_wait(&full[q], (uses - 1) & 1); spin++) {
+                }
+        }
+}
+
 // ------------------------------------------------------------- host side
+// Tile for k fields: ny launches' worth of blocks of nch fields and nsg site groups.  An SM
+// holds 16 warps (128 registers); the tile keeps as many of them as it can on fields of
+// their own, and each further reading of the links (ny) costs a little: 12 fields on
+// 32^3x64 took 342 to 377 us per application with 16 or 12 warps at work.
+inline FxTile fx_tile(int k, int *ny)
+{
+    FxTile t{1, kFxWarps, 0};
+    double best = -1e9;
+    for (int nch = 1; nch <= kFxWarps && nch <= k; nch++) {
+        const int nsg = kFxWarps / nch, y = (k + nch - 1) / nch;
+        const double score = double(16 / (nch * nsg) * nch * nsg) / 16 * k / (nch * y) - 0.03 * y;
+        if (score >= best) {
+            best = score;
+            t.nch = nch;
+            t.nsg = nsg;
+            *ny = y;
+        }
+    }
+    t.stages = t.nsg == 1 ? 8 : (t.nsg == 2 ? 6 : (t.nsg <= 4 ? 4 : 3));
+    return t;
+}
+
 // mantissas and exponents of the FP64 parity field `in` into `out` (fx_field_bytes)
 hisq_status launch_fx_split(hisq_ctx *ctx, const void *in, void *out);
+
+// Several right-hand sides at once (at most kFxGroup): out_i = a x_i + b y_i + c D(in_i)
+// on output parity par, and |out_i|^2.  Slot q of the group is right-hand side id[q];
+// every FP64 field lies at base + 3 Vh double2 times its slot or its right-hand side.
+constexpr int kFxGroup = 12;
+struct FxArray {
+    double2 *base; // null: not there
+    bool by_slot;
+};
+struct FxGroup {
+    int k;
+    int id[kFxGroup];
+};
+struct FxBatch {
+    FxArray in, out, x, y; // out null: norms only
+    double a, b, c;
+    void *mant;     // mantissas of in, fx_field_bytes per slot
+    void *mant_out; // mantissas of out, or null
+    bool norm;      // |out|^2 into ctx->bscal->out[id]
+};
+// in (FP64) to mantissas for every slot; with add, in += add first (FP32 fields at a
+// stride of 24 Vh bytes by right-hand side)
+hisq_status launch_fx_batch_split(hisq_ctx *ctx, const FxGroup &grp, FxArray in, void *mant, const void *add);
+hisq_status launch_fx_batch(hisq_ctx *ctx, int par, const FxGroup &grp, const FxBatch &b);
+hisq_status fx_blocks_per_sm(hisq_ctx *ctx, const void *kern, const FxTile &tl, int *bps);
 
 } // namespace hisq

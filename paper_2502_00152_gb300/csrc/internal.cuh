@@ -553,7 +553,7 @@ struct DevScalars {
     double pad0;
     long long iter; // iterations done
     long long pad1;
-    double slot[16]; // generic reduction results
+    double slot[16 + 2 * 64]; // generic reduction results; from 16 on: two per right-hand side of a batch
 };
 
 enum FinishOp : int {
@@ -720,7 +720,8 @@ enum BufId : int {
     BUF_DF_X,          // double-float residual: x split into (hi, lo)
     BUF_DF_T,          // double-float residual: odd temporary D_oe x
     BUF_PERSIST,       // persistent batched CG: per-block partials, thresholds
-    BUF_FX,            // FP64 operator: mantissas and exponents of its input field
+    BUF_FX,            // FP64 operator: mantissas and exponents of its input fields (and of a batch's D_oe x)
+    BUF_FX_T,          // FP64 operator: D_oe x of the right-hand sides of a group
     BUF_COUNT
 };
 
@@ -795,7 +796,11 @@ struct hisq_ctx {
 
     // profiling of the FP64 operator (hisq_set_profiling): event pairs around
     // each FP64 Dslash launch, summed once their launches have completed
-    std::vector<std::pair<cudaEvent_t, cudaEvent_t>> fp64_pending;
+    struct Fp64Pending {
+        cudaEvent_t first, second;
+        int fields; // right-hand sides the launch served
+    };
+    std::vector<Fp64Pending> fp64_pending;
     std::vector<cudaEvent_t> fp64_pool;
     double fp64_seconds = 0;
     unsigned long long fp64_launches = 0;
@@ -816,6 +821,7 @@ hisq_status set_err(hisq_ctx *c, hisq_status s, const char *fmt, ...);
 hisq_status cuda_err(hisq_ctx *c, cudaError_t e, const char *what);
 void *dev_alloc(hisq_ctx *c, size_t bytes);
 void dev_free(hisq_ctx *c, void *p, size_t bytes);
+hisq_status check_waits(hisq_ctx *c);
 // persistent scratch buffer `id` of at least `bytes` (nullptr + error set on OOM)
 void *get_buf(hisq_ctx *c, int id, size_t bytes);
 
@@ -997,6 +1003,10 @@ hisq_status ensure_half_links(hisq_ctx *ctx);
 // FP64 operator timing: fold completed event pairs into the sums (all: wait
 // for every pending one); discard: drop them without summing
 void fp64_prof_drain(hisq_ctx *ctx, bool all, bool discard = false);
+// a pair of events around an FP64 launch that serves `fields` right-hand sides: begin
+// records the first if profiling is on outside a capture (*on), end the second
+hisq_status fp64_prof_begin(hisq_ctx *ctx, int fields, bool *on);
+hisq_status fp64_prof_end(hisq_ctx *ctx, bool on);
 hisq_status launch_dslash(hisq_ctx *ctx, int out_parity, int prec, int link_prec, const void *in,
                           void *out, double a, const void *x, double b, const void *y, double c,
                           int norm_slot);

@@ -121,3 +121,27 @@ def test_without_room_for_the_mantissas():
         assert rel(project_parity(dims, H.hisq_apply_dslash(ctx, 0, 64, f), 0), dslash_ref(o, dims, f, 0)) <= 1e-13
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("nrhs", [2, 5, 7, 8, 12, 13, 25])
+@pytest.mark.parametrize("guess", [0, 1])
+def test_batched_residuals_match_oracle(nrhs, guess):
+    """A batched solve stopped by max_iter: source preparation, the reliable update of every
+    right-hand side and the full residual run as batched launches (groups of up to 12 fields
+    of 1 to 8 warps, Vh = 576 = 18 groups of 32 sites).  Its residuals are the oracle's."""
+    dims, m = (6, 6, 4, 8), 0.02
+    ctx, o = make(dims, seed=5, eps=0.3, mass=m)
+    try:
+        etas = np.stack([I.gaussian_source(dims, 13, j) for j in range(nrhs)])
+        start = 0.1 * np.stack([I.gaussian_source(dims, 17, j) for j in range(nrhs)]) if guess else None
+        prm = H.hisq_default_solve_params(batch=1, max_iter=3, tol=1e-14, precision_sloppy=32, guess=guess)
+        psi, st, status = H.hisq_solve(ctx, etas, prm, guess=start)
+        assert status == H.HISQ_ERR_NOT_CONVERGED
+        for j in range(nrhs):
+            y = project_parity(dims, o.prepare_source(m, etas[j]), 0)
+            ref = o.even_residual(m, project_parity(dims, psi[j], 0), y)
+            assert abs(st[j]["even_residual"] - ref) <= 1e-9 * ref
+            full = o.full_residual(m, psi[j], etas[j])
+            assert abs(st[j]["full_residual"] - full) <= 1e-9 * full
+    finally:
+        ctx.close()
