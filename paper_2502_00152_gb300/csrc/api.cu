@@ -321,13 +321,13 @@ hisq_status hisq_load_links(hisq_ctx *ctx, const double *fat, const double *lng,
         ctx->links_x[p] = nullptr;
         dev_free(ctx, ctx->links_xe[p], size_t(Vh) * 2);
         ctx->links_xe[p] = nullptr;
-        dev_free(ctx, ctx->links_f[p], size_t(Vh) * (ctx->long_recon == 18 ? 8 : 4) * 9 * 16);
+        dev_free(ctx, ctx->links_f[p], link_sites(Vh) * (ctx->long_recon == 18 ? 8 : 4) * 9 * 16);
         ctx->links_f[p] = nullptr;
-        dev_free(ctx, ctx->links_f12[p], size_t(Vh) * long_f32_bytes_per_site(ctx->long_recon));
+        dev_free(ctx, ctx->links_f12[p], link_sites(Vh) * long_f32_bytes_per_site(ctx->long_recon));
         ctx->links_f12[p] = nullptr;
-        dev_free(ctx, ctx->links_h[p], size_t(Vh) * (ctx->long_recon == 18 ? 8 : 4) * 9 * 8);
+        dev_free(ctx, ctx->links_h[p], link_sites(Vh) * (ctx->long_recon == 18 ? 8 : 4) * 9 * 8);
         ctx->links_h[p] = nullptr;
-        dev_free(ctx, ctx->links_h12[p], size_t(Vh) * 4 * 6 * 8);
+        dev_free(ctx, ctx->links_h12[p], link_sites(Vh) * 4 * 6 * 8);
         ctx->links_h12[p] = nullptr;
         dev_free(ctx, ctx->links_df[p], size_t(Vh) * 16 * 9 * 16);
         ctx->links_df[p] = nullptr;
@@ -336,8 +336,8 @@ hisq_status hisq_load_links(hisq_ctx *ctx, const double *fat, const double *lng,
     for (int p = 0; p < 2; p++) {
         ctx->links_x[p] = (int4 *)dev_alloc(ctx, links_x_bytes(Vh));
         ctx->links_xe[p] = (short *)dev_alloc(ctx, size_t(Vh) * 2);
-        ctx->links_f[p] = (float4 *)dev_alloc(ctx, size_t(Vh) * (long_recon == 18 ? 8 : 4) * 9 * 16);
-        if (long_recon != 18) ctx->links_f12[p] = (float4 *)dev_alloc(ctx, size_t(Vh) * long_f32_bytes_per_site(long_recon));
+        ctx->links_f[p] = (float4 *)dev_alloc(ctx, link_sites(Vh) * (long_recon == 18 ? 8 : 4) * 9 * 16);
+        if (long_recon != 18) ctx->links_f12[p] = (float4 *)dev_alloc(ctx, link_sites(Vh) * long_f32_bytes_per_site(long_recon));
         if (!ctx->links_x[p] || !ctx->links_xe[p] || !ctx->links_f[p] || (long_recon != 18 && !ctx->links_f12[p])) return HISQ_ERR_OOM;
         // FP16 links are built from the FP32 ones on first use (ensure_half_links)
     }

@@ -88,13 +88,13 @@ struct LinksFv {
     typedef float real;
     __device__ __forceinline__ void load(int mu, int kind, int i, CMat<float> &f, CMat<float> &b) const
     {
-        const float4 *q = base + size_t((mu * nk + kind) * 9) * Vh + i;
+        const float4 *q = base + link_index(i, (mu * nk + kind) * 9, nk * 36);
 #pragma unroll
         for (int k = 0; k < 9; k++) {
-            float4 a = __ldcs(q + size_t(k) * Vh);
+            const float4 a = __ldcs(q + 32 * k);
             f.re[k] = a.x;
-            f.im[k] = a.y;
-            b.re[k] = a.z;
+            b.re[k] = a.y;
+            f.im[k] = a.z;
             b.im[k] = a.w;
         }
     }
@@ -106,7 +106,7 @@ __device__ __forceinline__ float2 h2f(unsigned u)
     return __half22float2(h);
 }
 
-// FP16: uint2 = (fwd_k, bwd_k) as two half2, [mu][kind][k<9][Vh]
+// FP16: uint2 = (fwd_k, bwd_k) as two half2
 struct LinksHv {
     const uint2 *base;
     int Vh;
@@ -114,10 +114,10 @@ struct LinksHv {
     typedef float real;
     __device__ __forceinline__ void load(int mu, int kind, int i, CMat<float> &f, CMat<float> &b) const
     {
-        const uint2 *q = base + size_t((mu * nk + kind) * 9) * Vh + i;
+        const uint2 *q = base + link_index(i, (mu * nk + kind) * 9, nk * 36);
 #pragma unroll
         for (int k = 0; k < 9; k++) {
-            uint2 a = __ldcs(q + size_t(k) * Vh);
+            const uint2 a = __ldcs(q + 32 * k);
             float2 x = h2f(a.x), y = h2f(a.y);
             f.re[k] = x.x;
             f.im[k] = x.y;
@@ -133,10 +133,10 @@ struct LinksH12 {
     int Vh;
     __device__ __forceinline__ void load(int mu, int i, CMat<float> &f, CMat<float> &b) const
     {
-        const uint2 *q = base + size_t(mu * 6) * Vh + i;
+        const uint2 *q = base + link_index(i, mu * 6, 24);
 #pragma unroll
         for (int k = 0; k < 6; k++) {
-            uint2 a = __ldcs(q + size_t(k) * Vh);
+            const uint2 a = __ldcs(q + 32 * k);
             float2 x = h2f(a.x), y = h2f(a.y);
             f.re[k] = x.x;
             f.im[k] = x.y;

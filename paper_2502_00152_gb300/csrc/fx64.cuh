@@ -161,31 +161,12 @@ __device__ __forceinline__ int fx_site_exponent(const Geom &g, const int c[4], i
     return E;
 }
 
-// What the four neighbours of a site along mu share.
-struct FxLine {
-    int base, cm, L, stride; // neighbour at distance d: (base + wrapped(cm + d) * stride) / 2
-    __device__ __forceinline__ FxLine(const Geom &g, const int c[4], int s, int mu)
-    {
-        L = dim_of(g, mu);
-        cm = coord_of(c, mu);
-        stride = mu == 0 ? 1 : (mu == 1 ? g.stride[1] : (mu == 2 ? g.stride[2] : g.stride[3]));
-        base = s - cm * stride;
-    }
-    __device__ __forceinline__ int at(const Geom &g, int d) const
-    {
-        int cn = cm + d;
-        cn += cn < 0 ? L : 0;
-        cn -= cn >= L ? L : 0;
-        return checked_index(g, (base + cn * stride) >> 1, g.Vh);
-    }
-};
-
 // the neighbour's vector of one hop.
 // hop = 4 mu + h, h = 0: fat fwd, 1: fat bwd, 2: long fwd, 3: long bwd.
 struct FxVec {
     longlong2 v[3];
     int e;
-    __device__ __forceinline__ void load(const Geom &g, const FxLine &line, int h, const FxField &in)
+    __device__ __forceinline__ void load(const Geom &g, const SiteLine &line, int h, const FxField &in)
     {
         const unsigned nb = unsigned(line.at(g, (h & 2 ? 3 : 1) * (h & 1 ? -1 : 1)));
         e = __ldg(in.e + nb);
@@ -237,7 +218,7 @@ __device__ __forceinline__ void fx_add(const FxVec &x, int E, FxAcc &acc, F &&li
 struct FxHop {
     int4 w[9];
     FxVec x;
-    __device__ __forceinline__ void load(const Geom &g, const FxLine &line, int mu, int h, const int4 *L,
+    __device__ __forceinline__ void load(const Geom &g, const SiteLine &line, int mu, int h, const int4 *L,
                                          const FxField &in)
     {
         const int4 *p = L + (mu * 4 + h) * (9 * 32);
@@ -254,7 +235,7 @@ __device__ __forceinline__ void fx_directions(const Geom &g, const int c[4], int
                                               const FxField &in, int E, FxAcc &acc)
 {
     FxHop a, b;
-    FxLine line(g, c, s, mu0);
+    SiteLine line(g, c, s, mu0);
     a.load(g, line, mu0, 0, L, in);
 #pragma unroll 1
     for (int mu = mu0; mu < mu1; mu++) {
@@ -265,7 +246,7 @@ __device__ __forceinline__ void fx_directions(const Geom &g, const int c[4], int
         b.load(g, line, mu, 3, L, in);
         a.add(E, acc);
         if (mu + 1 < mu1) {
-            line = FxLine(g, c, s, mu + 1);
+            line = SiteLine(g, c, s, mu + 1);
             a.load(g, line, mu + 1, 0, L, in);
         }
         b.add(E, acc);
@@ -411,7 +392,7 @@ __device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const Link
             }
         };
         FxVec a, b;
-        FxLine line(g, c, s, 0);
+        SiteLine line(g, c, s, 0);
         a.load(g, line, 0, in);
 #pragma unroll 1
         for (int mu = 0; mu < 4; mu++) {
@@ -422,7 +403,7 @@ __device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const Link
             b.load(g, line, 3, in);
             hop(4 * mu + 2, a);
             if (mu < 3) {
-                line = FxLine(g, c, s, mu + 1);
+                line = SiteLine(g, c, s, mu + 1);
                 a.load(g, line, 0, in);
             }
             hop(4 * mu + 3, b);

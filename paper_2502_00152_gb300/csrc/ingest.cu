@@ -68,8 +68,8 @@ __device__ __forceinline__ void atomic_max_nonneg(float *addr, float v)
 
 struct IngestOut {
     double2 *d;    // FP64, fx_link_index, for this parity
-    float4 *f;     // FP32 [mu][nk][k][Vh]
-    float4 *f12;   // FP32 compressed long: recon 12 [mu][6][Vh], recon 8 [mu][4][Vh], or null
+    float4 *f;     // FP32 rows (mu * nk + kind) * 9 + k
+    float4 *f12;   // FP32 compressed long rows: recon 12 mu * 6 + k, recon 8 mu * 4 + q, or null
     int nk;
 };
 
@@ -125,27 +125,26 @@ __global__ void k_ingest(Geom g, int par, const double2 *__restrict__ fat, const
                 const double dev = fmax(su3_deviation(Sf), su3_deviation(Sb));
                 atomic_max_nonneg(max_dev, isfinite(dev) ? float(dev) : 1e30f);
                 if (recon == 12) {
-                    float4 *q = o.f12 + size_t(mu * 6) * Vh + cb;
+                    float4 *q = o.f12 + link_index(cb, mu * 6, 24);
 #pragma unroll
                     for (int k = 0; k < 6; k++)
-                        __stcs(q + size_t(k) * Vh,
-                               make_float4(float(Sf[k].x), float(Sf[k].y), float(Sb[k].x), float(Sb[k].y)));
+                        __stcs(q + 32 * k, make_float4(float(Sf[k].x), float(Sb[k].x), float(Sf[k].y), float(Sb[k].y)));
                 } else { // recon 8: (a2, a3), (b1, arg a1, arg c1) of fwd, then of bwd
-                    float4 *q = o.f12 + size_t(mu * 4) * Vh + cb;
+                    float4 *q = o.f12 + link_index(cb, mu * 4, 16);
                     const double2 *S2[2] = {Sf, Sb};
                     for (int fb = 0; fb < 2; fb++) {
                         const double2 *S = S2[fb];
-                        __stcs(q + size_t(2 * fb) * Vh, make_float4(float(S[1].x), float(S[1].y), float(S[2].x), float(S[2].y)));
-                        __stcs(q + size_t(2 * fb + 1) * Vh, make_float4(float(S[3].x), float(S[3].y), float(atan2(S[0].y, S[0].x)),
+                        __stcs(q + 64 * fb, make_float4(float(S[1].x), float(S[1].y), float(S[2].x), float(S[2].y)));
+                        __stcs(q + 64 * fb + 32, make_float4(float(S[3].x), float(S[3].y), float(atan2(S[0].y, S[0].x)),
                                                                         float(atan2(S[6].y, S[6].x))));
                     }
                 }
             } else {
-                float4 *q = o.f + size_t((mu * o.nk + kind) * 9) * Vh + cb;
+                float4 *q = o.f + link_index(cb, (mu * o.nk + kind) * 9, o.nk * 36);
 #pragma unroll
                 for (int k = 0; k < 9; k++)
-                    __stcs(q + size_t(k) * Vh, make_float4(float(sf * Mf[k].x), float(sf * Mf[k].y),
-                                                           float(sbk * Mb[k].x), float(sbk * Mb[k].y)));
+                    __stcs(q + 32 * k, make_float4(float(sf * Mf[k].x), float(sbk * Mb[k].x), float(sf * Mf[k].y),
+                                                   float(sbk * Mb[k].y)));
             }
         }
     }
@@ -193,7 +192,7 @@ __global__ void k_links_to_half(size_t n, const float4 *__restrict__ f, uint2 *_
 {
     for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
         const float4 a = f[i];
-        const __half2 x = __floats2half2_rn(a.x, a.y), y = __floats2half2_rn(a.z, a.w);
+        const __half2 x = __floats2half2_rn(a.x, a.z), y = __floats2half2_rn(a.y, a.w);
         h[i] = make_uint2(*reinterpret_cast<const unsigned *>(&x), *reinterpret_cast<const unsigned *>(&y));
     }
 }
@@ -204,7 +203,7 @@ hisq_status ensure_half_links(hisq_ctx *ctx)
 {
     if (ctx->links_h[0]) return HISQ_OK;
     if (ctx->long_recon == 8) return set_err(ctx, HISQ_ERR_INVALID_ARG, "FP16 links need long_recon 18 or 12");
-    const size_t Vh = size_t(ctx->g.Vh);
+    const size_t Vh = link_sites(ctx->g.Vh);
     const bool r12 = ctx->long_recon == 12;
     const size_t nf = Vh * (r12 ? 4 : 8) * 9, n12 = Vh * 4 * 6;
     for (int p = 0; p < 2; p++) {

@@ -191,6 +191,25 @@ __device__ __forceinline__ int nb_cb(const Geom &g, const int c[4], int s, int m
     return checked_index(g, (s + (cn - cm) * stride_of(g, mu)) >> 1, g.Vh);
 }
 
+// What the four neighbours of a site along mu share.
+struct SiteLine {
+    int base, cm, L, stride; // neighbour at distance d: (base + wrapped(cm + d) * stride) / 2
+    __device__ __forceinline__ SiteLine(const Geom &g, const int c[4], int s, int mu)
+    {
+        L = dim_of(g, mu);
+        cm = coord_of(c, mu);
+        stride = mu == 0 ? 1 : (mu == 1 ? g.stride[1] : (mu == 2 ? g.stride[2] : g.stride[3]));
+        base = s - cm * stride;
+    }
+    __device__ __forceinline__ int at(const Geom &g, int d) const
+    {
+        int cn = cm + d;
+        cn += cn < 0 ? L : 0;
+        cn -= cn >= L ? L : 0;
+        return checked_index(g, (base + cn * stride) >> 1, g.Vh);
+    }
+};
+
 __device__ __forceinline__ int full_site(const Geom &g, const int c[4])
 {
     return c[0] + g.X * (c[1] + g.Y * (c[2] + g.Z * c[3]));
@@ -429,45 +448,37 @@ __device__ __forceinline__ CVec<To> cvt(const CVec<From> &v)
 //
 // FP64 (recon 18): [p][group of 32 sites][mu][kind][fwd,bwd][k=0..8][32], 16 B per complex
 //   element: 56-bit mantissas under one exponent per output site (fx64.cuh)
-// FP32 (recon 18): float4  [p][mu][kind][k=0..8][Vh], float4 = (fwd_k, bwd_k)
-// FP32 long links with recon 12: float4 [p][mu][k=0..5][Vh] holding rows 0,1
-//   of the SU(3) factor S of fwd and bwd; W = sign * long_scale * S, with
+// The FP32 and FP16 arrays are stored by groups of 32 output sites, rows x 32 sites each
+// (link_index):
+// FP32 (recon 18): float4, row (mu * 2 + kind) * 9 + k; float4 = (Re fwd, Re bwd, Im fwd,
+//   Im bwd) of element k
+// FP32 long links with recon 12: fat rows mu * 9 + k; long float4 rows mu * 6 + k holding
+//   rows 0,1 of the SU(3) factor S of fwd and bwd; W = sign * long_scale * S, with
 //   sign = +-eta_mu(x) * (boundary sign) recomputed from the coordinates.
-// FP32 long links with recon 8: float4 [p][mu][q=0..3][Vh]: q = 0, 1 for fwd,
+// FP32 long links with recon 8: float4 rows mu * 4 + q: q = 0, 1 for fwd,
 //   2, 3 for bwd, each pair (a2, a3) and (b1, arg a1, arg c1) of the SU(3)
 //   factor (a = row 0, b = row 1, c = row 2); the rest follows from unitarity.
-// FP16 (recon 18): uint2 [p][mu][kind][k=0..8][Vh], uint2 = (fwd_k, bwd_k) as
-//   two half2; FP16 long links with recon 12: uint2 [p][mu][k=0..5][Vh].
-struct LinksF {
-    const float4 *base; // parity offset applied
-    int Vh;
-    typedef float real;
-    __device__ __forceinline__ void load(int mu, int kind, int i, CMat<float> &f, CMat<float> &b) const
-    {
-        const float4 *q = base + size_t((mu * 2 + kind) * 9) * Vh + i;
-#pragma unroll
-        for (int k = 0; k < 9; k++) {
-            float4 a = __ldcs(q + size_t(k) * Vh);
-            f.re[k] = a.x;
-            f.im[k] = a.y;
-            b.re[k] = a.z;
-            b.im[k] = a.w;
-        }
-    }
-};
+// FP16: the rows of the FP32 arrays as uint2 = (fwd_k, bwd_k), two half2.
+// Rows of a gathered link array are stored by groups of 32 output sites: element `row`
+// of `rows` of site i.  The rows of a direction of a group are contiguous (one bulk
+// copy), and a thread reads them at constant offsets from one address.
+__host__ __device__ __forceinline__ size_t link_index(int i, int row, int rows)
+{
+    return (size_t(i >> 5) * rows + row) * 32 + (i & 31);
+}
 
 struct LinksF12 { // long links only
     const float4 *base; // parity offset applied
     int Vh;
     __device__ __forceinline__ void load(int mu, int i, CMat<float> &f, CMat<float> &b) const
     {
-        const float4 *q = base + size_t(mu * 6) * Vh + i;
+        const float4 *q = base + link_index(i, mu * 6, 24);
 #pragma unroll
         for (int k = 0; k < 6; k++) {
-            float4 a = __ldcs(q + size_t(k) * Vh);
+            const float4 a = __ldcs(q + 32 * k);
             f.re[k] = a.x;
-            f.im[k] = a.y;
-            b.re[k] = a.z;
+            b.re[k] = a.y;
+            f.im[k] = a.z;
             b.im[k] = a.w;
         }
         su3_third_row(f);
@@ -527,8 +538,8 @@ struct LinksF8 { // long links only, 8 reals per SU(3) factor
     int Vh;
     __device__ __forceinline__ void load(int mu, int i, CMat<float> &f, CMat<float> &b) const
     {
-        const float4 *q = base + size_t(mu * 4) * Vh + i;
-        const float4 f0 = __ldcs(q), f1 = __ldcs(q + Vh), b0 = __ldcs(q + 2 * size_t(Vh)), b1 = __ldcs(q + 3 * size_t(Vh));
+        const float4 *q = base + link_index(i, mu * 4, 16);
+        const float4 f0 = __ldcs(q), f1 = __ldcs(q + 32), b0 = __ldcs(q + 64), b1 = __ldcs(q + 96);
         su3_from8(f0, f1, f);
         su3_from8(b0, b1, b);
     }
@@ -536,6 +547,9 @@ struct LinksF8 { // long links only, 8 reals per SU(3) factor
 
 // bytes of the FP64 links of one parity (whole groups of 32 sites)
 inline size_t links_x_bytes(int Vh) { return size_t((Vh + 31) / 32) * 32 * 144 * 16; }
+
+// sites of the FP32 and FP16 link arrays (whole groups)
+inline size_t link_sites(int Vh) { return size_t((Vh + 31) / 32) * 32; }
 
 // floats of compressed FP32 long links per output site and parity (0: none)
 inline size_t long_f32_bytes_per_site(int recon) { return recon == 12 ? 4 * 6 * 16 : (recon == 8 ? 4 * 4 * 16 : 0); }

@@ -13,6 +13,7 @@
 #include <functional>
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <utility>
 
 #include "internal.cuh"
@@ -65,11 +66,14 @@ struct MrhsTile {
 
 // per-slot sums of R values per thread into partials[block][slot] (lanes by a
 // fixed shuffle tree, site groups in order) and, in the last block, the sums
-// over blocks in block order followed by the batch finish operation
+// over blocks (a warp per slot: lanes over the blocks, then a fixed shuffle tree;
+// one thread per slot took up to 10 us over 304 blocks) followed by the batch
+// finish operation.  The slots of a block start at first (one of gridDim.y parts).
 template <int R>
-__device__ __forceinline__ void batch_reduce(double (&v)[R], const MrhsTile &tl, int kact, const BatchRed &br)
+__device__ __forceinline__ void batch_reduce(double (&v)[R], const MrhsTile &tl, int kact, const BatchRed &br,
+                                             int first = 0)
 {
-    __shared__ double sh[8][kMaxBatch]; // [site group][slot]
+    __shared__ double sh[16][kMaxBatch]; // [site group][slot of the block]
     __shared__ bool am_last;
     const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -84,21 +88,24 @@ __device__ __forceinline__ void batch_reduce(double (&v)[R], const MrhsTile &tl,
         }
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < kact; q += blockDim.x) {
+    for (int q = threadIdx.x; q < tl.nch * R && first + q < kact; q += blockDim.x) {
         double s = 0;
         for (int w = 0; w < tl.nsg; w++) s += sh[w][q];
-        br.partials[size_t(blockIdx.x) * kMaxBatch + q] = s;
+        br.partials[size_t(blockIdx.x) * kMaxBatch + first + q] = s;
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) am_last = (atomicAdd(br.ticket, 1u) == gridDim.x - 1);
+    if (threadIdx.x == 0) am_last = (atomicAdd(br.ticket, 1u) == gridDim.x * gridDim.y - 1);
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-    for (int q = threadIdx.x; q < kact; q += blockDim.x) {
+    BatchScalars *B = br.scal;
+    for (int q = threadIdx.x >> 5; q < kact; q += blockDim.x >> 5) {
         double s = 0;
-        for (int b = 0; b < (int)gridDim.x; b++) s += ((volatile double *)br.partials)[size_t(b) * kMaxBatch + q];
-        BatchScalars *B = br.scal;
+        for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(br.partials + size_t(b) * kMaxBatch + q);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane) continue;
         const int j = B->idx[q];
         switch (br.op) {
         case BFIN_STORE: B->out[j] = s; break;
@@ -126,10 +133,33 @@ __device__ __forceinline__ void batch_reduce(double (&v)[R], const MrhsTile &tl,
 }
 
 // ------------------------------------------------------------- epilogues
+// operator(): one right-hand side at a site.  all(): R of them, every load before the
+// first store, and prefetch(): their fields into L2 (used by the ring kernel, whose
+// epilogue data come from HBM).
+__device__ __forceinline__ void prefetch_l2(const void *p)
+{
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+__device__ __forceinline__ void prefetch_site(const SpinorH &f, int cb) { prefetch_l2(f.p + cb); }
+__device__ __forceinline__ void prefetch_site(const SpinorF &f, int cb)
+{
+    prefetch_l2(f.a + cb);
+    prefetch_l2(f.b + cb);
+}
+
 // tmp_j = acc, |tmp_j|^2
 template <class S>
 struct BEpiStore {
     BatchF<S> out;
+    __device__ __forceinline__ void prefetch(int, int) const {}
+    template <int R>
+    __device__ __forceinline__ void all(int cb, const int (&jj)[R], const bool (&on)[R], const CVec<float> (&acc)[R],
+                                        double (&red)[R]) const
+    {
+#pragma unroll
+        for (int u = 0; u < R; u++)
+            if (on[u]) (*this)(cb, jj[u], acc[u], red[u]);
+    }
     template <typename R>
     __device__ __forceinline__ void operator()(int cb, int j, const CVec<R> &acc, double &red) const
     {
@@ -145,6 +175,43 @@ struct BEpiCG {
     BatchF<SX> x;
     const double *alpha; // alpha[j] by right-hand side (global or shared memory)
     const double *m4;    // 4 m^2
+    __device__ __forceinline__ void prefetch(int cb, int j) const
+    {
+        prefetch_site(p.at(j), cb);
+        prefetch_site(r.at(j), cb);
+        prefetch_site(x.at(j), cb);
+    }
+    template <int R>
+    __device__ __forceinline__ void all(int cb, const int (&jj)[R], const bool (&on)[R], const CVec<float> (&acc)[R],
+                                        double (&red)[R]) const
+    {
+        CVec<float> pv[R], rv[R];
+        CVec<typename SX::real> xv[R];
+        float al[R];
+        const float m4v = float(*m4);
+#pragma unroll
+        for (int u = 0; u < R; u++) {
+            pv[u] = p.at(jj[u]).load(cb);
+            rv[u] = r.at(jj[u]).load(cb);
+            xv[u] = x.at(jj[u]).load(cb);
+            al[u] = float(alpha[jj[u]]);
+        }
+#pragma unroll
+        for (int u = 0; u < R; u++) {
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                const float apr = fmaf(m4v, pv[u].re[i], -acc[u].re[i]), api = fmaf(m4v, pv[u].im[i], -acc[u].im[i]);
+                rv[u].re[i] = fmaf(-al[u], apr, rv[u].re[i]);
+                rv[u].im[i] = fmaf(-al[u], api, rv[u].im[i]);
+                xv[u].re[i] = fmaf(al[u], pv[u].re[i], xv[u].re[i]);
+                xv[u].im[i] = fmaf(al[u], pv[u].im[i], xv[u].im[i]);
+            }
+            if (!on[u]) continue;
+            x.at(jj[u]).store(cb, xv[u]);
+            r.at(jj[u]).store(cb, rv[u]);
+            red[u] += double(rv[u].norm2());
+        }
+    }
     template <typename R>
     __device__ __forceinline__ void operator()(int cb, int j, const CVec<R> &acc, double &red) const
     {
@@ -176,6 +243,19 @@ struct BEpiLin {
     BatchF<SpinorF> out, x, y;
     float a, b, c;
     bool hx, hy;
+    __device__ __forceinline__ void prefetch(int cb, int j) const
+    {
+        if (hx) prefetch_site(x.at(j), cb);
+        if (hy) prefetch_site(y.at(j), cb);
+    }
+    template <int R>
+    __device__ __forceinline__ void all(int cb, const int (&jj)[R], const bool (&on)[R], const CVec<float> (&acc)[R],
+                                        double (&red)[R]) const
+    {
+#pragma unroll
+        for (int u = 0; u < R; u++)
+            if (on[u]) (*this)(cb, jj[u], acc[u], red[u]);
+    }
     template <typename R>
     __device__ __forceinline__ void operator()(int cb, int j, const CVec<R> &acc, double &) const
     {
@@ -206,23 +286,18 @@ struct BEpiLin {
 };
 
 // ------------------------------------------------------------- the kernel
-__device__ __forceinline__ void prefetch_l2(const void *p)
-{
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
 __device__ __forceinline__ void prefetch_long(const LinksF12 &L, int mu, int i)
 {
     if (!L.base) return;
-    const float4 *q = L.base + size_t(mu * 6) * L.Vh + i;
+    const float4 *q = L.base + link_index(i, mu * 6, 24);
 #pragma unroll
-    for (int k = 0; k < 6; k++) prefetch_l2(q + size_t(k) * L.Vh);
+    for (int k = 0; k < 6; k++) prefetch_l2(q + 32 * k);
 }
 __device__ __forceinline__ void prefetch_long(const LinksF8 &L, int mu, int i)
 {
-    const float4 *q = L.base + size_t(mu * 4) * L.Vh + i;
+    const float4 *q = L.base + link_index(i, mu * 4, 16);
 #pragma unroll
-    for (int k = 0; k < 4; k++) prefetch_l2(q + size_t(k) * L.Vh);
+    for (int k = 0; k < 4; k++) prefetch_l2(q + 32 * k);
 }
 
 // gathered FP32 links of the batched kernels: fat (and, with 18-real long
@@ -234,19 +309,19 @@ struct LinksFvB {
     typedef float real;
     __device__ __forceinline__ void prefetch(int mu, int i) const
     {
-        const float4 *q = base + size_t((mu * nk) * 9) * Vh + i;
+        const float4 *q = base + link_index(i, mu * nk * 9, nk * 36);
 #pragma unroll
-        for (int k = 0; k < 9; k++) prefetch_l2(q + size_t(k) * Vh);
+        for (int k = 0; k < 9; k++) prefetch_l2(q + 32 * k);
     }
     __device__ __forceinline__ void load(int mu, int kind, int i, CMat<float> &f, CMat<float> &b) const
     {
-        const float4 *q = base + size_t((mu * nk + kind) * 9) * Vh + i;
+        const float4 *q = base + link_index(i, (mu * nk + kind) * 9, nk * 36);
 #pragma unroll
         for (int k = 0; k < 9; k++) {
-            float4 a = __ldg(q + size_t(k) * Vh); // shared by the lanes of one site
+            const float4 a = __ldg(q + 32 * k); // shared by the warps of a site group
             f.re[k] = a.x;
-            f.im[k] = a.y;
-            b.re[k] = a.z;
+            b.re[k] = a.y;
+            f.im[k] = a.z;
             b.im[k] = a.w;
         }
     }
@@ -381,23 +456,16 @@ __device__ __forceinline__ void pupd_sites(int Vh, const BatchF<S> &r, const Bat
     }
 }
 
-// p_j = r_j + beta_j p_j, |p_j|^2
-template <int R, class S>
-__global__ void __launch_bounds__(512, 1)
+// p_j = r_j + beta_j p_j, |p_j|^2, one field per warp (blockIdx.y: parts of the fields)
+template <class S>
+__global__ void __launch_bounds__(256)
     k_p_update_mrhs(int Vh, BatchF<S> r, BatchF<S> p, const BatchScalars *scal, MrhsTile tl, BatchRed br)
 {
-    const int kact = scal->kact;
-    int jj[R];
-#pragma unroll
-    for (int u = 0; u < R; u++) {
-        const int q = tl.chunk() * R + u;
-        jj[u] = q < kact ? scal->idx[q] : -1;
-    }
-    double red[R];
-#pragma unroll
-    for (int u = 0; u < R; u++) red[u] = 0;
-    pupd_sites<R, S>(Vh, r, p, scal->beta, jj, tl, red);
-    batch_reduce<R>(red, tl, kact, br);
+    const int kact = scal->kact, first = blockIdx.y * tl.nch, q = first + tl.chunk();
+    const int jj[1] = {q < kact ? scal->idx[q] : -1};
+    double red[1] = {0};
+    pupd_sites<1, S>(Vh, r, p, scal->beta, jj, tl, red);
+    batch_reduce<1>(red, tl, kact, br, first);
 }
 
 // ------------------------------------------------- persistent batched CG
@@ -815,10 +883,283 @@ __global__ void __launch_bounds__(512, 1)
     batch_reduce<R>(red, tl, kact, br);
 }
 
+// ------------------------------------------------- links through a ring
+// The batched operator: a thread computes one site for R right-hand sides, the lanes of a
+// warp 32 consecutive sites of the same fields, the nch warps of a site group the fields.
+//  - The links of a direction of a site group are contiguous (9 fat rows, 6 or 9 long
+//    rows of 512 B): one or two bulk copies into a ring of shared memory that all warps of
+//    the group read, so each link leaves HBM once per launch and no register or load slot
+//    is held while it travels.
+//  - The neighbours of the next (direction, kind) are loaded while the current ones are
+//    multiplied; the fields of the epilogue are brought to L2 two directions ahead and
+//    loaded for all R right-hand sides before the first store.
+//  - Of 12-real long links the sign, c3 and the vector's own scale are one factor, applied
+//    to the neighbour.
+// Bound by instruction issue (65 %: 1165 instructions per site and right-hand side, 576 of
+// them the FMAs) and the FMA pipe (52 %).  12 right-hand sides, FP16 vectors, 32^3x64:
+// D_oe 622 -> 554 us, fused update 714 -> 616 us (R = 4, 12 warps per SM) against the
+// register kernel below; R = 3 with 16 warps 611, R = 2 729.  Packed FMAs (fwd, bwd) with
+// R = 3 took 705: the pairs cost a third more registers and a move per unpacked value.
+// Every wait is bounded: one that runs out records its code in *status, the warp gives up
+// the rest of its sites (the reduction still runs) and the launch ends.
+// a neighbour as it is stored, and unpacked (times sc, if used)
+template <class S>
+struct RawVec;
+template <>
+struct RawVec<SpinorH> {
+    uint4 u;
+    __device__ __forceinline__ void load(const char *base, int, unsigned i)
+    {
+        u = __ldg(reinterpret_cast<const uint4 *>(base) + i);
+    }
+};
+template <>
+struct RawVec<SpinorF> {
+    float4 a;
+    float2 b;
+    __device__ __forceinline__ void load(const char *base, int Vh, unsigned i)
+    {
+        a = __ldg(reinterpret_cast<const float4 *>(base) + i);
+        b = __ldg(reinterpret_cast<const float2 *>(base + size_t(Vh) * 16) + i);
+    }
+};
+__device__ __forceinline__ CVec<float> unpack(const RawVec<SpinorH> &r, float sc, bool use)
+{
+    const float s = use ? __uint_as_float(r.u.w) * sc : __uint_as_float(r.u.w);
+    const unsigned h[3] = {r.u.x, r.u.y, r.u.z};
+    CVec<float> v;
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&h[c]));
+        v.re[c] = f.x * s;
+        v.im[c] = f.y * s;
+    }
+    return v;
+}
+__device__ __forceinline__ CVec<float> unpack(const RawVec<SpinorF> &r, float sc, bool use)
+{
+    CVec<float> v;
+    v.re[0] = r.a.x;
+    v.im[0] = r.a.y;
+    v.re[1] = r.a.z;
+    v.im[1] = r.a.w;
+    v.re[2] = r.b.x;
+    v.im[2] = r.b.y;
+    if (use) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            v.re[c] *= sc;
+            v.im[c] *= sc;
+        }
+    }
+    return v;
+}
+
+struct RingTile {
+    int nch, nsg, stages;
+    __host__ __device__ size_t smem(int rows) const { return size_t(nsg) * stages * (rows * 512 + 2 * sizeof(uint64_t)); }
+};
+
+template <int R, class S, bool R12, class Epi, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1)
+    k_dslash_ring(Geom g, int par, const float4 *__restrict__ fat, const float4 *__restrict__ lng, float c3,
+                  BatchF<S> in, const BatchScalars *scal, RingTile rt, Epi epi, BatchRed br, int *status)
+{
+    constexpr int ROWS = R12 ? 15 : 18;
+    constexpr int STAGE = ROWS * 512;
+    extern __shared__ __align__(128) unsigned char dsm[];
+    const int Vh = g.Vh, stages = rt.stages;
+    const MrhsTile tl{rt.nch, rt.nsg};
+    const int lane = threadIdx.x & 31, chunk = tl.chunk(), sg = tl.group();
+    unsigned char *ring = dsm + size_t(sg) * stages * STAGE;
+    uint64_t *full = reinterpret_cast<uint64_t *>(dsm + size_t(rt.nsg) * stages * STAGE) + 2 * sg * stages;
+    uint64_t *empty = full + stages;
+    const bool producer = chunk == 0 && lane == 0;
+    if (producer) {
+        for (int q = 0; q < stages; q++) {
+            tc::mbar_init(&full[q], 1);
+            tc::mbar_init(&empty[q], rt.nch);
+        }
+        tc::fence_mbar_init();
+    }
+    __syncthreads();
+
+    // slots past the last one gather its field again and skip the epilogue
+    const int kact = scal->kact;
+    const int first_slot = blockIdx.y * rt.nch * R;
+    const char *src[R];
+    int jj[R];
+    bool on[R];
+    double red[R];
+#pragma unroll
+    for (int u = 0; u < R; u++) {
+        on[u] = first_slot + chunk * R + u < kact;
+        jj[u] = scal->idx[min(first_slot + chunk * R + u, kact - 1)];
+        src[u] = in.base + in.stride * jj[u];
+        red[u] = 0;
+    }
+    const int ngroups = (Vh + 31) / 32;
+    const int first = blockIdx.x * rt.nsg + sg, gstride = gridDim.x * rt.nsg;
+    const int nitems = first < ngroups ? ((ngroups - 1 - first) / gstride + 1) * 4 : 0;
+    // item j: direction j % 4 of this group's (j / 4)-th 32 sites
+    int issued = 0, islot = 0; // items issued, slot of the next one
+    uint32_t iphase = 1;       // parity to wait for before that slot is refilled
+    auto issue = [&]() {
+        uint64_t *fb = &full[islot];
+        unsigned char *st = ring + size_t(islot) * STAGE;
+        const int cb0 = (first + (issued >> 2) * gstride) * 32, mu = issued & 3;
+        tc::mbar_arrive_expect_tx(fb, STAGE);
+        if (R12) {
+            tc::bulk_load_1d(st, fat + link_index(cb0, mu * 9, 36), 9 * 512, fb);
+            tc::bulk_load_1d(st + 9 * 512, lng + link_index(cb0, mu * 6, 24), 6 * 512, fb);
+        } else {
+            tc::bulk_load_1d(st, fat + link_index(cb0, mu * 18, 72), 18 * 512, fb);
+        }
+        issued++;
+        if (++islot == stages) {
+            islot = 0;
+            iphase ^= 1;
+        }
+    };
+    if (producer)
+        while (issued < min(stages, nitems)) issue();
+
+    bool ok = true;
+    int slot = 0;       // slot of the item in work
+    uint32_t phase = 0; // its parity
+#pragma unroll 1
+    for (int it = 0; it < nitems && ok; it += 4) {
+        const int at = (first + (it >> 2) * gstride) * 32 + lane;
+        const int cb = min(at, Vh - 1);
+        int c[4];
+        cb_coords(g, par, cb, c);
+        const int s = full_site(g, c);
+        CVec<float> acc[R];
+#pragma unroll
+        for (int u = 0; u < R; u++) acc[u].zero();
+        RawVec<S> vf[R], vb[R]; // the neighbours of the (direction, kind) in work, then of the next
+        auto gather = [&](const SiteLine &line, int n) {
+            const unsigned f = unsigned(line.at(g, n)), b = unsigned(line.at(g, -n));
+#pragma unroll
+            for (int u = 0; u < R; u++) {
+                vf[u].load(src[u], Vh, f);
+                vb[u].load(src[u], Vh, b);
+            }
+        };
+        SiteLine line(g, c, s, 0);
+        gather(line, 1);
+#pragma unroll 1
+        for (int mu = 0; mu < 4; mu++) {
+            if (producer) {
+                // a slot is refilled once every warp of the group has released it; the producer
+                // blocks only when the item its own warp needs now is not issued
+                while (ok && issued < nitems && issued < it + mu + stages) {
+                    if (!tc::mbar_try_wait(&empty[islot], iphase)) {
+                        if (issued > it + mu) break;
+                        ok = tc::mbar_wait(&empty[islot], iphase, status, tc::TC_TIMEOUT_EMPTY);
+                        if (!ok) break;
+                    }
+                    issue();
+                }
+            }
+            if (ok) ok = tc::mbar_wait(&full[slot], phase, status, tc::TC_TIMEOUT_FULL);
+            const float4 *w = reinterpret_cast<const float4 *>(ring + size_t(slot) * STAGE) + lane;
+            CVec<float> xf[R], xb[R];
+            // one link element of both hops on column j into row i of every right-hand side
+            auto mac = [&](int i, int j, float4 e) {
+#pragma unroll
+                for (int u = 0; u < R; u++) {
+                    acc[u].re[i] = fmaf(e.x, xf[u].re[j], acc[u].re[i]);
+                    acc[u].im[i] = fmaf(e.x, xf[u].im[j], acc[u].im[i]);
+                    acc[u].re[i] = fmaf(-e.z, xf[u].im[j], acc[u].re[i]);
+                    acc[u].im[i] = fmaf(e.z, xf[u].re[j], acc[u].im[i]);
+                    acc[u].re[i] = fmaf(e.y, xb[u].re[j], acc[u].re[i]);
+                    acc[u].im[i] = fmaf(e.y, xb[u].im[j], acc[u].im[i]);
+                    acc[u].re[i] = fmaf(-e.w, xb[u].im[j], acc[u].re[i]);
+                    acc[u].im[i] = fmaf(e.w, xb[u].re[j], acc[u].im[i]);
+                }
+            };
+            if (mu == 2) {
+#pragma unroll
+                for (int u = 0; u < R; u++) epi.prefetch(cb, jj[u]);
+            }
+            // fat hops
+#pragma unroll
+            for (int u = 0; u < R; u++) {
+                xf[u] = unpack(vf[u], 0, false);
+                xb[u] = unpack(vb[u], 0, false);
+            }
+            gather(line, 3);
+#pragma unroll
+            for (int k = 0; k < 9; k++) mac(k / 3, k % 3, w[32 * k]);
+            // long hops; of 12-real ones rows 0 and 1 of the SU(3) factors are stored, and the
+            // hop's sign and c3 go into the vectors
+            float sf = 1.f, sb = 1.f;
+            if (R12) {
+                const float eta = stag_phase(mu, c);
+                sf = eta * c3;
+                sb = -eta * c3;
+                if (mu == 3 && g.t_antiperiodic) {
+                    if (c[3] + 3 >= g.T) sf = -sf;
+                    if (c[3] < 3) sb = -sb;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < R; u++) {
+                xf[u] = unpack(vf[u], sf, R12);
+                xb[u] = unpack(vb[u], sb, R12);
+            }
+            if (mu < 3) {
+                line = SiteLine(g, c, s, mu + 1);
+                gather(line, 1);
+            }
+            if constexpr (R12) {
+                float4 e[6];
+#pragma unroll
+                for (int k = 0; k < 6; k++) {
+                    e[k] = w[32 * (9 + k)];
+                    mac(k / 3, k % 3, e[k]);
+                }
+#pragma unroll
+                for (int j = 0; j < 3; j++) {
+                    // row 2 = conj(a x b): (a x b)_j = a_{j+1} b_{j+2} - a_{j+2} b_{j+1}
+                    const int j1 = (j + 1) % 3, j2 = (j + 2) % 3;
+                    const float4 a1 = e[j1], a2 = e[j2], b1 = e[3 + j1], b2 = e[3 + j2];
+                    float4 t;
+                    t.x = fmaf(a1.x, b2.x, fmaf(-a1.z, b2.z, fmaf(-a2.x, b1.x, a2.z * b1.z)));
+                    t.y = fmaf(a1.y, b2.y, fmaf(-a1.w, b2.w, fmaf(-a2.y, b1.y, a2.w * b1.w)));
+                    t.z = fmaf(a2.x, b1.z, fmaf(a2.z, b1.x, fmaf(-a1.x, b2.z, -a1.z * b2.x)));
+                    t.w = fmaf(a2.y, b1.w, fmaf(a2.w, b1.y, fmaf(-a1.y, b2.w, -a1.w * b2.y)));
+                    mac(2, j, t);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 9; k++) mac(k / 3, k % 3, w[32 * (9 + k)]);
+            }
+            ok = __all_sync(0xffffffffu, ok);
+            if (lane == 0 && ok) tc::mbar_arrive(&empty[slot]);
+            if (++slot == stages) {
+                slot = 0;
+                phase ^= 1;
+            }
+        }
+        if (ok && at < Vh) epi.all(cb, jj, on, acc, red);
+    }
+    // copies still in flight (only after a wait gave up) land before the block ends
+    if (producer && !ok)
+        for (int q = 0; q < stages; q++) {
+            const int uses = (issued + stages - 1 - q) / stages;
+            if (uses > 0)
+                for (int spin = 0; spin < (1 << 20) && !tc::mbar_try_wait(&full[q], (uses - 1) & 1); spin++) {
+                }
+        }
+    batch_reduce<R>(red, tl, kact, br, first_slot);
+}
+
 // ------------------------------------------------- the TMA-fed batched kernel
 // The same operator with the links of each (site group, direction) copied into
 // shared memory by the bulk-copy engine (one elected thread per site group
-// issues 15 copies of 512 B: the 9 fat rows and the 6 stored long rows of 32
+// issues two copies: the 9 fat rows and the 6 stored long rows of 32
 // consecutive sites) into a ring of `stages` slots guarded by mbarriers.  The
 // warps then read each link element from shared memory once per R right-hand
 // sides, so no link load is held in registers while the DRAM latency elapses:
@@ -873,14 +1214,11 @@ __global__ void __launch_bounds__(256, MINB)
     auto issue = [&](int j) {
         const int mu = j & 3;
         const int cb0 = (first + (j >> 2) * gstride) * 32;
-        const uint32_t rb = uint32_t(min(32, Vh - cb0)) * 16u;
         uint64_t *fb = &full[j % stages];
         unsigned char *st = ring + size_t(j % stages) * kTmaStageBytes;
-        tc::mbar_arrive_expect_tx(fb, kTmaRows * rb);
-#pragma unroll 1
-        for (int k = 0; k < 9; k++) tc::bulk_load_1d(st + k * 512, fat + size_t(mu * 9 + k) * Vh + cb0, rb, fb);
-#pragma unroll 1
-        for (int k = 0; k < 6; k++) tc::bulk_load_1d(st + (9 + k) * 512, lng + size_t(mu * 6 + k) * Vh + cb0, rb, fb);
+        tc::mbar_arrive_expect_tx(fb, kTmaStageBytes);
+        tc::bulk_load_1d(st, fat + link_index(cb0, mu * 9, 36), 9 * 512, fb);
+        tc::bulk_load_1d(st + 9 * 512, lng + link_index(cb0, mu * 6, 24), 6 * 512, fb);
     };
     int issued = 0;
     if (producer)
@@ -936,13 +1274,13 @@ __global__ void __launch_bounds__(256, MINB)
             break;
         }
         const float4 *rows = reinterpret_cast<const float4 *>(ring + size_t(it % stages) * kTmaStageBytes) + lane;
-        // fat links: forward (x, y of each row element) and backward (z, w)
+        // fat links: forward (x, z of each row element) and backward (y, w)
 #pragma unroll
         for (int d = 0; d < 2; d++) {
 #pragma unroll
             for (int k = 0; k < 9; k++) {
-                const float2 w = d == 0 ? *reinterpret_cast<const float2 *>(rows + 32 * k)
-                                        : *(reinterpret_cast<const float2 *>(rows + 32 * k) + 1);
+                const float *e = reinterpret_cast<const float *>(rows + 32 * k);
+                const float2 w = make_float2(e[d], e[2 + d]);
                 const int i = k / 3, j = k % 3;
 #pragma unroll
                 for (int u = 0; u < R; u++) {
@@ -965,8 +1303,8 @@ __global__ void __launch_bounds__(256, MINB)
             float ar[6], ai[6]; // rows 0 and 1: (a0, a1, a2, b0, b1, b2)
 #pragma unroll
             for (int k = 0; k < 6; k++) {
-                const float2 w = d == 0 ? *reinterpret_cast<const float2 *>(rows + 32 * (9 + k))
-                                        : *(reinterpret_cast<const float2 *>(rows + 32 * (9 + k)) + 1);
+                const float *e = reinterpret_cast<const float *>(rows + 32 * (9 + k));
+                const float2 w = make_float2(e[d], e[2 + d]);
                 ar[k] = sc * w.x;
                 ai[k] = sc * w.y;
                 const int i = k / 3, j = k % 3;
@@ -1019,6 +1357,7 @@ struct MrhsShape {
     int rc;  // k_dslash_mrhs: 0 with the L2 link prefetch, 1 without; k_dslash_mrhs_tma: blocks per SM
     int tma; // 1: the TMA-fed kernel (FP32 links with 12-real long links only)
     int x2;  // 1: the packed-pair kernel (R even)
+    int ring; // 1: k_dslash_ring (18- or 12-real long links): rc = parts of the right-hand sides
 };
 constexpr int kTmaStages = 4;
 
@@ -1048,6 +1387,7 @@ static int mrhs_candidates(int kact, MrhsShape *out, bool tma_ok, bool all)
                     out[n].rc = pf;
                     out[n].tma = 0;
                     out[n].x2 = x2;
+                    out[n].ring = 0;
                     n++;
                 }
             }
@@ -1062,14 +1402,45 @@ static int mrhs_candidates(int kact, MrhsShape *out, bool tma_ok, bool all)
             out[n].rc = minb;
             out[n].tma = 1;
             out[n].x2 = 0;
+            out[n].ring = 0;
             n++;
         }
     return n;
 }
 
-static unsigned long long mrhs_key(const hisq_ctx *ctx, int kact, int prec)
+// threads of a k_dslash_ring block at most, by right-hand sides per thread: 128 registers
+// per thread, 168 for R = 4
+constexpr int ring_max_threads(int R) { return R == 4 ? 384 : 512; }
+constexpr int kRingSmem = 104 * 1024; // ring slots of the resident blocks of an SM at most (beyond two per
+                                      // site group): the rest of the 256 KB is L1 for the gathers
+
+// Candidates of k_dslash_ring: R, and how the 16 or 12 warps of an SM are dealt to
+// fields and site groups (1 to 4 blocks).  A site group's links serve nch warps; with more
+// fields than a block has warps they come in rc equal parts.
+static int ring_candidates(int kact, MrhsShape *out)
 {
-    return (1ull << 40) | (unsigned long long)kact | ((unsigned long long)prec << 8) |
+    int n = 0;
+    for (int R : {3, 2, 4}) {
+        if (R > 2 && kact < R) continue;
+        const int wmax = ring_max_threads(R) / 32, chunks = (kact + R - 1) / R;
+        for (int blocks : {1, 2, 4}) {
+            const int w = wmax / blocks; // warps of a block
+            const int parts = (chunks + w - 1) / w, nch = (chunks + parts - 1) / parts, nsg = std::min(w / nch, 8 / blocks);
+            if (nsg < 1 || (blocks > 1 && chunks > w)) continue;
+            out[n].R = R;
+            out[n].tile = MrhsTile{nch, nsg};
+            out[n].rc = parts;
+            out[n].tma = out[n].x2 = 0;
+            out[n].ring = 1;
+            n++;
+        }
+    }
+    return n;
+}
+
+static unsigned long long mrhs_key(const hisq_ctx *ctx, int kact, int prec, bool ring)
+{
+    return (ring ? 2ull << 40 : 1ull << 40) | (unsigned long long)kact | ((unsigned long long)prec << 8) |
            ((unsigned long long)ctx->long_recon << 16);
 }
 
@@ -1187,10 +1558,57 @@ static hisq_status run_mrhs_tma(hisq_ctx *ctx, int par, const BatchF<S> &in, con
     return launch(k_dslash_mrhs_tma<R, S, Epi, 2>);
 }
 
+template <int R, class S, class Epi>
+static hisq_status run_mrhs_ring(hisq_ctx *ctx, int par, const BatchF<S> &in, const MrhsShape &sh, const Epi &epi,
+                                 BatchRed br)
+{
+    const int Vh = ctx->g.Vh;
+    const int threads = 32 * sh.tile.nch * sh.tile.nsg;
+    const int rows = ctx->long_recon == 12 ? 15 : 18;
+    auto launch = [&](auto kern) -> hisq_status {
+        // ring slots: what the blocks that fit by their threads leave each other, 2 to 6
+        const int by_threads = std::max(1, ring_max_threads(R) / threads);
+        RingTile rt{sh.tile.nch, sh.tile.nsg, 0};
+        rt.stages = std::min(6, std::max(2, kRingSmem / (by_threads * sh.tile.nsg * (rows * 512 + 16))));
+        const size_t smem = rt.smem(rows);
+        static std::mutex mu;
+        static std::map<std::tuple<int, const void *, int, size_t>, int> bps_cache; // -> blocks per SM
+        int bps = 1;
+        {
+            std::lock_guard<std::mutex> lock(mu);
+            int &n = bps_cache[std::make_tuple(ctx->device, reinterpret_cast<const void *>(kern), threads, smem)];
+            if (n == 0) {
+                HISQ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess || n < 1) {
+                    cudaGetLastError();
+                    n = 1;
+                }
+            }
+            bps = n;
+        }
+        // all parts resident together, so that they sweep the sites in step
+        const int gx = std::min(grid_for(ctx, long(Vh), 32 * rt.nsg, bps), std::max(1, ctx->num_sms * bps / sh.rc));
+        kern<<<dim3(gx, sh.rc), threads, smem, ctx->stream>>>(ctx->g, par, ctx->links_f[par], ctx->links_f12[par],
+                                                             float(ctx->long_scale), in, ctx->bscal, rt, epi, br,
+                                                             ctx->wait_status_d);
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? HISQ_OK : cuda_err(ctx, e, "batched dslash (ring) launch");
+    };
+    if (ctx->long_recon == 12) return launch(k_dslash_ring<R, S, true, Epi, ring_max_threads(R)>);
+    return launch(k_dslash_ring<R, S, false, Epi, ring_max_threads(R)>);
+}
+
 template <class S, class Epi>
 static hisq_status run_shape(hisq_ctx *ctx, int par, const BatchF<S> &in, const MrhsShape &sh, const Epi &epi,
                              BatchRed br)
 {
+    if (sh.ring) {
+        switch (sh.R) {
+        case 2: return run_mrhs_ring<2>(ctx, par, in, sh, epi, br);
+        case 3: return run_mrhs_ring<3>(ctx, par, in, sh, epi, br);
+        default: return run_mrhs_ring<4>(ctx, par, in, sh, epi, br);
+        }
+    }
     if (sh.x2) {
         if (sh.R == 4) return run_mrhs_x2<2>(ctx, par, in, sh.tile, sh.rc, epi, br);
         return run_mrhs_x2<1>(ctx, par, in, sh.tile, sh.rc, epi, br);
@@ -1212,11 +1630,21 @@ static hisq_status run_shape(hisq_ctx *ctx, int par, const BatchF<S> &in, const 
 // the shape for this batch: tuned on an idempotent launch (may_tune), else
 // the one tuned before, else the default
 static hisq_status mrhs_shape(hisq_ctx *ctx, int kact, int prec, MrhsShape *sh, bool may_tune,
-                              const std::function<hisq_status(const MrhsShape &)> &launch)
+                              const std::function<hisq_status(const MrhsShape &)> &launch, bool allow_ring = true)
 {
     MrhsShape cand[kMaxMrhsCandidates];
     const bool forced = ctx->mrhs_force_kind != 0;
-    const int n = mrhs_candidates(kact, cand, ctx->long_recon == 12, forced);
+    // FP16 vectors: the ring kernel where its link formats are used, else the register
+    // kernel; FP32 vectors: whichever is faster (their gathers need twice the registers in
+    // flight), the register kernel until it has been timed
+    const bool ring = allow_ring && !forced && ctx->long_recon != 8;
+    int n = 0;
+    if (ring && prec == 16) {
+        n = ring_candidates(kact, cand);
+    } else {
+        n = mrhs_candidates(kact, cand, ctx->long_recon == 12, forced);
+        if (ring) n += ring_candidates(kact, cand + n);
+    }
     int idx = 0;
     if (forced) {
         // a launch shape chosen by the caller (hisq_set_batched_kernel)
@@ -1231,7 +1659,7 @@ static hisq_status mrhs_shape(hisq_ctx *ctx, int kact, int prec, MrhsShape *sh, 
                        "for %d right-hand sides and these links",
                        ctx->mrhs_force_kind, ctx->mrhs_force_R, ctx->mrhs_force_budget, kact);
     }
-    const unsigned long long key = mrhs_key(ctx, kact, prec);
+    const unsigned long long key = mrhs_key(ctx, kact, prec, ring);
     if (may_tune) {
         hisq_status st = autotune(ctx, key, n, 0, [&](int i) { return launch(cand[i]); }, &idx);
         if (st != HISQ_OK) return st;
@@ -1365,14 +1793,23 @@ hisq_status launch_bcg_persistent(hisq_ctx *ctx, int prec, int link_prec, void *
         return set_err(ctx, HISQ_ERR_INVALID_ARG, "persistent batched CG: FP32 links with 18- or 12-real long links");
     if (prec != 32 && prec != 16) return set_err(ctx, HISQ_ERR_INVALID_ARG, "persistent batched CG: sloppy 32 or 16");
     if (kact < 1 || kact > kMaxBatch || max_iters < 1) return set_err(ctx, HISQ_ERR_INVALID_ARG, "persistent batched CG");
-    // the shape the autotuner picks for this batch (tuned on an ordinary D_oe
-    // launch the first time, which leaves nothing the persistent kernel reads)
-    if (!ctx->tuned.count(mrhs_key(ctx, kact, prec))) {
-        hisq_status st = launch_mrhs_dslash_tt(ctx, prec, link_prec, p, tmp, kact);
-        if (st != HISQ_OK) return st;
-    }
+    // the register-kernel shape the autotuner picks for this batch (tuned on ordinary D_oe
+    // launches the first time, which leave nothing the persistent kernel reads)
     MrhsShape sh;
-    hisq_status st = mrhs_shape(ctx, kact, prec, &sh, false, nullptr);
+    BatchRed br = batch_red(ctx, BFIN_ALPHA);
+    hisq_status st =
+        prec == 16 ? mrhs_shape(ctx, kact, prec, &sh, true,
+                                [&](const MrhsShape &c) {
+                                    return run_shape(ctx, 1, batchf<SpinorH>(p, Vh, 16), c,
+                                                     BEpiStore<SpinorH>{batchf<SpinorH>(tmp, Vh, 16)}, br);
+                                },
+                                false)
+                   : mrhs_shape(ctx, kact, prec, &sh, true,
+                                [&](const MrhsShape &c) {
+                                    return run_shape(ctx, 1, batchf<SpinorF>(p, Vh, 32), c,
+                                                     BEpiStore<SpinorF>{batchf<SpinorF>(tmp, Vh, 32)}, br);
+                                },
+                                false);
     if (st != HISQ_OK) return st;
     if (sh.tma || sh.x2) return set_err(ctx, HISQ_ERR_INVALID_ARG, "persistent batched CG: register-kernel shapes only");
     const MrhsTile tl = sh.tile;
@@ -1455,16 +1892,19 @@ hisq_status launch_bcg_persistent(hisq_ctx *ctx, int prec, int link_prec, void *
     return prec == 16 ? by_r(SpinorH{}) : by_r(SpinorF{});
 }
 
-// (3) p_j = r_j + beta_j p_j, pp_j (the shape of the batch's Dslash)
-template <int R, class S>
-static hisq_status run_p_update(hisq_ctx *ctx, void *r, void *p, const MrhsTile &tl, int prec)
+// (3) p_j = r_j + beta_j p_j, pp_j: one field per warp, blocks of 8 warps
+template <class S>
+static hisq_status run_p_update(hisq_ctx *ctx, void *r, void *p, int kact, int prec)
 {
     const int Vh = ctx->g.Vh;
+    const int parts = (kact + 7) / 8, nch = (kact + parts - 1) / parts;
+    const MrhsTile tl{nch, 8 / nch};
     const int threads = 32 * tl.nch * tl.nsg;
-    auto kern = k_p_update_mrhs<R, S>;
-    const int grid = grid_for(ctx, long(Vh), 32 * tl.nsg, mrhs_blocks_per_sm(kern, threads));
-    kern<<<grid, threads, 0, ctx->stream>>>(Vh, batchf<S>(r, Vh, prec), batchf<S>(p, Vh, prec), ctx->bscal, tl,
-                                            batch_red(ctx, BFIN_P));
+    auto kern = k_p_update_mrhs<S>;
+    const int bps = mrhs_blocks_per_sm(kern, threads);
+    const int gx = std::min(grid_for(ctx, long(Vh), 32 * tl.nsg, bps), std::max(1, ctx->num_sms * bps / parts));
+    kern<<<dim3(gx, parts), threads, 0, ctx->stream>>>(Vh, batchf<S>(r, Vh, prec), batchf<S>(p, Vh, prec), ctx->bscal,
+                                                       tl, batch_red(ctx, BFIN_P));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_err(ctx, e, "batched p update");
     return HISQ_OK;
@@ -1473,19 +1913,9 @@ static hisq_status run_p_update(hisq_ctx *ctx, void *r, void *p, const MrhsTile 
 hisq_status launch_mrhs_p_update(hisq_ctx *ctx, int prec, void *r, void *p, int kact)
 {
     if (kact < 1 || kact > kMaxBatch) return set_err(ctx, HISQ_ERR_INVALID_ARG, "batched p update: 1..64 right-hand sides");
-    if (prec != 32 && prec != 16) return set_err(ctx, HISQ_ERR_INVALID_ARG, "batched sloppy precision must be 32 or 16");
-    MrhsShape sh;
-    hisq_status st = mrhs_shape(ctx, kact, prec, &sh, false, nullptr);
-    if (st != HISQ_OK) return st;
-    auto go = [&](auto tagS) -> hisq_status {
-        typedef decltype(tagS) S;
-        switch (sh.R) {
-        case 2: return run_p_update<2, S>(ctx, r, p, sh.tile, prec);
-        case 3: return run_p_update<3, S>(ctx, r, p, sh.tile, prec);
-        default: return run_p_update<4, S>(ctx, r, p, sh.tile, prec);
-        }
-    };
-    return prec == 32 ? go(SpinorF{}) : go(SpinorH{});
+    if (prec == 32) return run_p_update<SpinorF>(ctx, r, p, kact, prec);
+    if (prec == 16) return run_p_update<SpinorH>(ctx, r, p, kact, prec);
+    return set_err(ctx, HISQ_ERR_INVALID_ARG, "batched sloppy precision must be 32 or 16");
 }
 
 } // namespace hisq

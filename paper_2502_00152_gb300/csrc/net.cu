@@ -45,14 +45,14 @@ __device__ __forceinline__ void net_transport(const Geom &g, const float4 *links
     float2 v[3];
 #pragma unroll
     for (int i = 0; i < 3; i++) v[i] = ch[size_t(sn) * 3 + i];
-    const float4 *q = links_p + size_t((mu * nk + 0) * 9) * g.Vh + cb;
+    const float4 *q = links_p + link_index(cb, mu * nk * 9, nk * 36);
 #pragma unroll
     for (int i = 0; i < 3; i++) {
         float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
         for (int j = 0; j < 3; j++) {
-            const float4 w = __ldg(q + size_t(3 * i + j) * g.Vh);
-            const float2 m = d == 0 ? make_float2(w.x, w.y) : make_float2(w.z, w.w);
+            const float4 w = __ldg(q + 32 * (3 * i + j));
+            const float2 m = d == 0 ? make_float2(w.x, w.z) : make_float2(w.y, w.w);
             const float2 pr = cmulf(m, v[j]);
             acc.x += pr.x;
             acc.y += pr.y;
