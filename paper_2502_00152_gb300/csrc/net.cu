@@ -17,211 +17,379 @@
 // Weights: (Cout, Cin, 9) complex64; optionally rounded to BF16 when staged.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace hisq {
 
 constexpr int kNetHops = 9;
-constexpr int kNetSites = 16; // sites per block
 constexpr int kNetMaxC = 16;
 
-__device__ __forceinline__ float2 cmulf(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-
-// transports of site (parity p, cb) for input channel a and hop h -> 3 complex
-__device__ __forceinline__ void net_transport(const Geom &g, const float4 *links_p, int nk, const float2 *in, int V,
-                                              int a, int h, int p, int cb, const int c[4], int s, float2 (&t)[3])
+// two FP32 values as one operand of the packed FMA (each half an IEEE FMA)
+typedef unsigned long long pairf;
+__device__ __forceinline__ pairf pk(float a, float b)
 {
-    const float2 *ch = in + size_t(a) * V * 3;
-    if (h == 0) {
-#pragma unroll
-        for (int i = 0; i < 3; i++) t[i] = ch[size_t(s) * 3 + i];
-        return;
-    }
+    pairf d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ float2 upk(pairf a)
+{
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
+    return d;
+}
+__device__ __forceinline__ void pfma(pairf &c, pairf a, pairf b)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ pairf padd(pairf a, pairf b)
+{
+    pairf d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// coordinates of full-lattice site s
+__device__ __forceinline__ void net_coords(const Geom &g, int s, int (&c)[4])
+{
+    int r = fdiv(s >> 1, g.dX2);
+    c[0] = s - r * g.X;
+    int q = fdiv(r, g.dY);
+    c[1] = r - q * g.Y;
+    r = q;
+    q = fdiv(r, g.dZ);
+    c[2] = r - q * g.Z;
+    c[3] = q;
+}
+
+// neighbour of hop h (1 + 2 mu + d; 0: the site itself), full-lattice index
+__device__ __forceinline__ int net_neighbour(const Geom &g, const int (&c)[4], int s, int h)
+{
+    if (h == 0) return s;
     const int mu = (h - 1) >> 1, d = (h - 1) & 1;
-    int cn[4] = {c[0], c[1], c[2], c[3]};
-    const int L = dim_of(g, mu);
-    cn[mu] = d == 0 ? (c[mu] + 1 == L ? 0 : c[mu] + 1) : (c[mu] == 0 ? L - 1 : c[mu] - 1);
-    const int sn = checked_index(g, full_site(g, cn), g.V);
-    float2 v[3];
-#pragma unroll
-    for (int i = 0; i < 3; i++) v[i] = ch[size_t(sn) * 3 + i];
+    const int L = dim_of(g, mu), cm = coord_of(c, mu);
+    const int cn = d == 0 ? (cm + 1 == L ? 0 : cm + 1) : (cm == 0 ? L - 1 : cm - 1);
+    return checked_index(g, s + (cn - cm) * stride_of(g, mu), g.V);
+}
+
+// fat hop matrix of hop h > 0 at site (parity arrays, nk kinds per direction)
+__device__ __forceinline__ void net_link(const float4 *links_p, int nk, int cb, int h, CMat<float> &m)
+{
+    const int mu = (h - 1) >> 1;
+    const bool bwd = (h - 1) & 1;
     const float4 *q = links_p + link_index(cb, mu * nk * 9, nk * 36);
 #pragma unroll
-    for (int i = 0; i < 3; i++) {
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            const float4 w = __ldg(q + 32 * (3 * i + j));
-            const float2 m = d == 0 ? make_float2(w.x, w.z) : make_float2(w.y, w.w);
-            const float2 pr = cmulf(m, v[j]);
-            acc.x += pr.x;
-            acc.y += pr.y;
-        }
-        t[i] = acc;
+    for (int k = 0; k < 9; k++) {
+        const float4 w = __ldg(q + 32 * k);
+        m.re[k] = bwd ? w.y : w.x;
+        m.im[k] = bwd ? w.w : w.z;
     }
 }
 
-// stage the (possibly adjoint) weights of one layer into shared memory
-__device__ __forceinline__ void net_stage_weights(float2 *sw, const float2 *w, int cin, int cout, int adjoint, int bf16)
+__device__ __forceinline__ void net_load(const float2 *p, CVec<float> &v)
 {
-    // staged layout: [b][a][h] for the layer as applied (cout_eff x cin_eff)
-    const int co = adjoint ? cin : cout, ci = adjoint ? cout : cin;
-    for (int t = threadIdx.x; t < co * ci * kNetHops; t += blockDim.x) {
-        const int b = t / (ci * kNetHops), a = (t / kNetHops) % ci, h = t % kNetHops;
-        float2 v;
-        if (!adjoint) {
-            v = w[(size_t(b) * cin + a) * kNetHops + h];
-        } else {
-            // applied weight w'[b][a][h] from the stored w[a][b][h'] (b < cin, a < cout)
-            const int hs = h == 0 ? 0 : (1 + (((h - 1) >> 1) << 1) + (1 - ((h - 1) & 1)));
-            const float2 u = w[(size_t(a) * cin + b) * kNetHops + hs];
-            v = h == 0 ? make_float2(u.x, -u.y) : make_float2(-u.x, u.y);
-        }
-        if (bf16) {
-            v.x = __bfloat162float(__float2bfloat16_rn(v.x));
-            v.y = __bfloat162float(__float2bfloat16_rn(v.y));
-        }
-        sw[t] = v;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        const float2 a = __ldg(p + i);
+        v.re[i] = a.x;
+        v.im[i] = a.y;
     }
 }
 
-// out = layer(in) (adjoint = 0) or layer^dag(in) (adjoint = 1)
-__global__ void __launch_bounds__(256)
+// weight of output b, input a, hop h of the layer as applied (adjoint: see above)
+__device__ __forceinline__ float2 net_weight(const float2 *w, int cin, int b, int a, int h, int adjoint, int bf16)
+{
+    float2 v;
+    if (!adjoint) {
+        v = w[(size_t(b) * cin + a) * kNetHops + h];
+    } else {
+        const int hs = h == 0 ? 0 : (1 + (((h - 1) >> 1) << 1) + (1 - ((h - 1) & 1)));
+        const float2 u = w[(size_t(a) * cin + b) * kNetHops + hs];
+        v = h == 0 ? make_float2(u.x, -u.y) : make_float2(-u.x, u.y);
+    }
+    if (bf16) {
+        v.x = __bfloat162float(__float2bfloat16_rn(v.x));
+        v.y = __bfloat162float(__float2bfloat16_rn(v.y));
+    }
+    return v;
+}
+
+// out = layer(in) (adjoint = 0) or layer^dag(in) (adjoint = 1).  A thread computes one
+// site for 2 P output channels (blockIdx.y: which): for each hop its matrix, for each
+// input channel the transported vector, and for each pair of output channels 12 packed
+// FMAs with the two weights as the halves, the vector's components repeated in both.  The
+// weights are staged once per block and read as broadcasts; nothing else passes through
+// shared memory.  The sums over the input channels of a hop are formed on their own and
+// then added, which halves the rounding error of one long sum (1.9e-7 against 3.1e-7 of
+// the result at 16 x 16 channels; 2.3e-7 before).  Bound by the FMA pipe: 9 ci co 12 +
+// 8 ci 36 FMAs per site.  16 to 16 channels: 24^3x48 10.6 -> 1.0 ms, 16^3x32 2.1 -> 0.20 ms;
+// 8 channels per thread 1.43 ms.
+constexpr int kNetThreads = 128;
+
+template <int P>
+__global__ void __launch_bounds__(kNetThreads, P == 8 ? 2 : (P == 4 ? 3 : 4))
     k_net_layer(Geom g, const float4 *links0, const float4 *links1, int nk, const float2 *__restrict__ w, int cin,
                 int cout, int adjoint, int bf16, const float2 *__restrict__ in, float2 *__restrict__ out)
 {
-    extern __shared__ float2 sm[];
+    extern __shared__ float4 sw[]; // [hop][input channel][pair]: (re0, re1, im0, im1)
     const int co = adjoint ? cin : cout, ci = adjoint ? cout : cin;
-    float2 *sw = sm;                                   // co * ci * 9
-    float2 *st = sm + co * ci * kNetHops;              // kNetSites * ci * 9 * 3
-    net_stage_weights(sw, w, cin, cout, adjoint, bf16);
-    const int V = g.V;
-    const int nblk = (V + kNetSites - 1) / kNetSites;
-    for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-        __syncthreads();
-        // phase 1: transports of every (site, input channel, hop)
-        for (int t = threadIdx.x; t < kNetSites * ci * kNetHops; t += blockDim.x) {
-            const int ls = t / (ci * kNetHops), a = (t / kNetHops) % ci, h = t % kNetHops;
-            const int s = blk * kNetSites + ls;
-            float2 tr[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-            if (s < V) {
-                int c[4];
-                int r = s;
-                c[0] = r % g.X;
-                r /= g.X;
-                c[1] = r % g.Y;
-                r /= g.Y;
-                c[2] = r % g.Z;
-                c[3] = r / g.Z;
-                const int p = (c[0] + c[1] + c[2] + c[3]) & 1;
-                net_transport(g, p ? links1 : links0, nk, in, V, a, h, p, s >> 1, c, s, tr);
-            }
-#pragma unroll
-            for (int i = 0; i < 3; i++) st[size_t(t) * 3 + i] = tr[i];
+    const int b0 = blockIdx.y * 2 * P;
+    for (int t = threadIdx.x; t < kNetHops * ci * P; t += blockDim.x) {
+        const int h = t / (ci * P), a = t / P % ci, b = b0 + 2 * (t % P);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (b < co) {
+            const float2 u = net_weight(w, cin, b, a, h, adjoint, bf16);
+            v.x = u.x;
+            v.z = u.y;
         }
-        __syncthreads();
-        // phase 2: channel mixing, one (site, output channel) per thread
-        for (int t = threadIdx.x; t < kNetSites * co; t += blockDim.x) {
-            const int ls = t / co, b = t % co;
-            const int s = blk * kNetSites + ls;
-            if (s >= V) continue;
-            float2 acc[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-            const float2 *tb = st + size_t(ls) * ci * kNetHops * 3;
-            const float2 *wb = sw + size_t(b) * ci * kNetHops;
-            for (int q = 0; q < ci * kNetHops; q++) {
-                const float2 wv = wb[q];
+        if (b + 1 < co) {
+            const float2 u = net_weight(w, cin, b + 1, a, h, adjoint, bf16);
+            v.y = u.x;
+            v.w = u.y;
+        }
+        sw[t] = v;
+    }
+    __syncthreads();
+    const size_t V3 = size_t(g.V) * 3;
+    for (int s0 = blockIdx.x * kNetThreads; s0 < g.V; s0 += gridDim.x * kNetThreads) {
+        const int s = min(s0 + int(threadIdx.x), g.V - 1);
+        int c[4];
+        net_coords(g, s, c);
+        const float4 *links_p = (c[0] + c[1] + c[2] + c[3]) & 1 ? links1 : links0;
+        pairf re[P][3], im[P][3], sr[P][3], si[P][3]; // sums over the input channels of a hop, over all hops
+#pragma unroll
+        for (int p = 0; p < P; p++)
+#pragma unroll
+            for (int i = 0; i < 3; i++) sr[p][i] = si[p][i] = 0;
+#pragma unroll 1
+        for (int h = 0; h < kNetHops; h++) {
+#pragma unroll
+            for (int p = 0; p < P; p++)
+#pragma unroll
+                for (int i = 0; i < 3; i++) re[p][i] = im[p][i] = 0;
+            CMat<float> m;
+            if (h > 0) net_link(links_p, nk, s >> 1, h, m);
+            const float2 *q = in + size_t(net_neighbour(g, c, s, h)) * 3;
+            const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(sw) + h * ci * P;
+            CVec<float> nxt;
+            net_load(q, nxt);
+#pragma unroll 1
+            for (int a = 0; a < ci; a++) {
+                CVec<float> t = nxt;
+                q += V3;
+                if (a + 1 < ci) net_load(q, nxt);
+                if (h > 0) {
+                    const CVec<float> v = t;
+                    t.zero();
+                    mv_acc(t, m, v);
+                }
+                pairf tr[3], ti[3], tn[3];
 #pragma unroll
                 for (int i = 0; i < 3; i++) {
-                    const float2 pr = cmulf(wv, tb[q * 3 + i]);
-                    acc[i].x += pr.x;
-                    acc[i].y += pr.y;
+                    tr[i] = pk(t.re[i], t.re[i]);
+                    ti[i] = pk(t.im[i], t.im[i]);
+                    tn[i] = pk(-t.im[i], -t.im[i]);
                 }
+#pragma unroll
+                for (int p = 0; p < P; p++) {
+                    const ulonglong2 u = wp[p]; // x: the two real parts, y: the imaginary ones
+#pragma unroll
+                    for (int i = 0; i < 3; i++) {
+                        pfma(re[p][i], u.x, tr[i]);
+                        pfma(im[p][i], u.x, ti[i]);
+                        pfma(re[p][i], u.y, tn[i]);
+                        pfma(im[p][i], u.y, tr[i]);
+                    }
+                }
+                wp += P;
             }
 #pragma unroll
-            for (int i = 0; i < 3; i++) out[(size_t(b) * V + s) * 3 + i] = acc[i];
+            for (int p = 0; p < P; p++)
+#pragma unroll
+                for (int i = 0; i < 3; i++) {
+                    sr[p][i] = padd(sr[p][i], re[p][i]);
+                    si[p][i] = padd(si[p][i], im[p][i]);
+                }
+        }
+        if (s0 + int(threadIdx.x) < g.V) {
+#pragma unroll
+            for (int p = 0; p < P; p++) {
+                const int b = b0 + 2 * p;
+                float2 *o = out + size_t(b) * V3 + size_t(s) * 3;
+#pragma unroll
+                for (int i = 0; i < 3; i++) {
+                    const float2 r = upk(sr[p][i]), m = upk(si[p][i]);
+                    if (b < co) o[i] = make_float2(r.x, m.x);
+                    if (b + 1 < co) o[V3 + i] = make_float2(r.y, m.y);
+                }
+            }
         }
     }
 }
 
-// per-block partial weight gradients: G[b][a][h] = sum_x gout_b(x) . conj(T_h in_a(x))
-__global__ void __launch_bounds__(256)
+// Weight gradients: G[b][a][h] = sum_x gout_b(x) . conj(T_h in_a(x)).  A block takes 16
+// sites at a time: its 144 threads transport one (site, hop) each for every input channel
+// into shared memory, then each accumulates a 4 x 4 tile of (b, (a, h)) over the 48 (site,
+// colour) rows.  With fewer tiles than threads the rows are dealt to groups of threads.
+// The FP32 sum of a group of sites is added to a two-float sum (two-sum), so that the
+// total has the accuracy of an FP64 one; the partial sums of groups and blocks are added
+// in FP64 in a fixed order.  Bound by the FMA pipe and the latency of the transports'
+// loads between two barriers (three blocks per SM at 128 registers; two at 167: 1.77 ms).
+// 16 x 16 channels: 24^3x48 4.35 -> 1.51 ms.
+constexpr int kWgSites = 16, kWgThreads = kWgSites * kNetHops, kWgRows = kWgSites * 3;
+constexpr int kWgPitch = kNetMaxC * kNetHops + 4; // floats per row of a plane: 16-byte rows, few conflicts
+
+__device__ __forceinline__ void two_sum(float &hi, float &lo, float x)
+{
+    const float t = __fadd_rn(hi, x), z = __fsub_rn(t, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(x, z)));
+    hi = t;
+}
+
+__global__ void __launch_bounds__(kWgThreads, 3)
     k_net_wgrad(Geom g, const float4 *links0, const float4 *links1, int nk, int cin, int cout,
-                const float2 *__restrict__ in, const float2 *__restrict__ gout, double2 *part)
+                const float2 *__restrict__ in, const float2 *__restrict__ gout, int groups, double2 *part)
 {
-    extern __shared__ float2 sm[];
-    float2 *st = sm;                                           // kNetSites * cin * 9 * 3
-    float2 *sg = sm + size_t(kNetSites) * cin * kNetHops * 3;  // kNetSites * cout * 3
-    const int V = g.V;
-    const int ntrip = cout * cin * kNetHops;
-    constexpr int kPer = (kNetMaxC * kNetMaxC * kNetHops + 255) / 256;
-    double accr[kPer], acci[kPer];
+    extern __shared__ float4 dsm4[];
+    float *st = reinterpret_cast<float *>(dsm4);      // [re, im][row][kWgPitch]: transports, row = 3 site + colour
+    float2 *sg = reinterpret_cast<float2 *>(st + 2 * kWgRows * kWgPitch); // [row][kNetMaxC]: gout
+    const int nah = cin * kNetHops, nta = (nah + 3) / 4, ntb = (cout + 3) / 4, ntile = nta * ntb;
+    const int ls = threadIdx.x % kWgSites, h = threadIdx.x / kWgSites;
+    // this thread's tile and rows
+    const int tile = threadIdx.x % ntile, grp = threadIdx.x / ntile;
+    const bool on = grp < groups;
+    const int ta = tile % nta, tb = tile / nta;
+    float hr[16], hi[16], lr[16], li[16];
 #pragma unroll
-    for (int u = 0; u < kPer; u++) accr[u] = acci[u] = 0;
-    const int nblk = (V + kNetSites - 1) / kNetSites;
-    for (int blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
+    for (int k = 0; k < 16; k++) hr[k] = hi[k] = lr[k] = li[k] = 0.f;
+    const size_t V3 = size_t(g.V) * 3;
+    // the columns past the last (a, h) and the channels past the last b stay zero
+    for (int t = threadIdx.x; t < 2 * kWgRows * kWgPitch; t += blockDim.x) st[t] = 0.f;
+    for (int t = threadIdx.x; t < kWgRows * kNetMaxC; t += blockDim.x) sg[t] = make_float2(0.f, 0.f);
+    for (int blk = blockIdx.x; blk * kWgSites < g.V; blk += gridDim.x) {
         __syncthreads();
-        for (int t = threadIdx.x; t < kNetSites * cin * kNetHops; t += blockDim.x) {
-            const int ls = t / (cin * kNetHops), a = (t / kNetHops) % cin, h = t % kNetHops;
-            const int s = blk * kNetSites + ls;
-            float2 tr[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-            if (s < V) {
-                int c[4];
-                int r = s;
-                c[0] = r % g.X;
-                r /= g.X;
-                c[1] = r % g.Y;
-                r /= g.Y;
-                c[2] = r % g.Z;
-                c[3] = r / g.Z;
-                const int p = (c[0] + c[1] + c[2] + c[3]) & 1;
-                net_transport(g, p ? links1 : links0, nk, in, V, a, h, p, s >> 1, c, s, tr);
-            }
+        const int s = blk * kWgSites + ls;
+        const float live = s < g.V ? 1.f : 0.f;
+        {
+            const int sc = min(s, g.V - 1);
+            int c[4];
+            net_coords(g, sc, c);
+            CMat<float> m;
+            if (h > 0) net_link((c[0] + c[1] + c[2] + c[3]) & 1 ? links1 : links0, nk, sc >> 1, h, m);
+            const float2 *q = in + size_t(net_neighbour(g, c, sc, h)) * 3;
+            float *o = st + 3 * ls * kWgPitch + h;
+            for (int a0 = 0; a0 < cin; a0 += 4) {
+                CVec<float> v[4]; // four channels' loads in flight
 #pragma unroll
-            for (int i = 0; i < 3; i++) st[size_t(t) * 3 + i] = tr[i];
-        }
-        for (int t = threadIdx.x; t < kNetSites * cout * 3; t += blockDim.x) {
-            const int ls = t / (cout * 3), b = (t / 3) % cout, i = t % 3;
-            const int s = blk * kNetSites + ls;
-            sg[t] = s < V ? gout[(size_t(b) * V + s) * 3 + i] : make_float2(0.f, 0.f);
-        }
-        __syncthreads();
+                for (int k = 0; k < 4; k++) net_load(q + V3 * min(a0 + k, cin - 1), v[k]);
 #pragma unroll
-        for (int u = 0; u < kPer; u++) {
-            const int q = threadIdx.x + u * blockDim.x;
-            if (q >= ntrip) continue;
-            const int b = q / (cin * kNetHops), ah = q % (cin * kNetHops);
-            float sr = 0.f, si = 0.f;
-            for (int ls = 0; ls < kNetSites; ls++) {
+                for (int k = 0; k < 4; k++) {
+                    if (a0 + k >= cin) break;
+                    CVec<float> t = v[k];
+                    if (h > 0) {
+                        t.zero();
+                        mv_acc(t, m, v[k]);
+                    }
 #pragma unroll
-                for (int i = 0; i < 3; i++) {
-                    const float2 gv = sg[(ls * cout + b) * 3 + i];
-                    const float2 tv = st[(size_t(ls) * cin * kNetHops + ah) * 3 + i];
-                    // gv * conj(tv)
-                    sr += gv.x * tv.x + gv.y * tv.y;
-                    si += gv.y * tv.x - gv.x * tv.y;
+                    for (int i = 0; i < 3; i++) {
+                        o[i * kWgPitch + (a0 + k) * kNetHops] = live != 0.f ? t.re[i] : 0.f;
+                        o[(kWgRows + i) * kWgPitch + (a0 + k) * kNetHops] = live != 0.f ? t.im[i] : 0.f;
+                    }
                 }
             }
-            accr[u] += sr;
-            acci[u] += si;
         }
-    }
+        for (int t = threadIdx.x; t < kWgRows * cout; t += blockDim.x) {
+            const int b = t / kWgRows, r = t % kWgRows;
+            const size_t x = size_t(blk) * kWgRows + r;
+            sg[r * kNetMaxC + b] = x < V3 ? __ldg(gout + size_t(b) * V3 + x) : make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+        if (!on) continue;
+        pairf ar[4][2], ai[4][2]; // rows b, pairs of (a, h)
 #pragma unroll
-    for (int u = 0; u < kPer; u++) {
-        const int q = threadIdx.x + u * blockDim.x;
-        if (q < ntrip) part[size_t(blockIdx.x) * ntrip + q] = make_double2(accr[u], acci[u]);
+        for (int b = 0; b < 4; b++) ar[b][0] = ar[b][1] = ai[b][0] = ai[b][1] = 0;
+#pragma unroll 2
+        for (int r = grp; r < kWgRows; r += groups) {
+            const ulonglong2 tr = *reinterpret_cast<const ulonglong2 *>(st + r * kWgPitch + 4 * ta);
+            const ulonglong2 ti = *reinterpret_cast<const ulonglong2 *>(st + (kWgRows + r) * kWgPitch + 4 * ta);
+            const float4 *gp = reinterpret_cast<const float4 *>(sg + r * kNetMaxC + 4 * tb);
+            const float4 g0 = gp[0], g1 = gp[1];
+            const float gr[4] = {g0.x, g0.z, g1.x, g1.z}, gi[4] = {g0.y, g0.w, g1.y, g1.w};
+#pragma unroll
+            for (int b = 0; b < 4; b++) { // g conj(t)
+                const pairf pr = pk(gr[b], gr[b]), pi = pk(gi[b], gi[b]), pn = pk(-gr[b], -gr[b]);
+                pfma(ar[b][0], pi, ti.x);
+                pfma(ar[b][1], pi, ti.y);
+                pfma(ai[b][0], pn, ti.x);
+                pfma(ai[b][1], pn, ti.y);
+                pfma(ar[b][0], pr, tr.x);
+                pfma(ar[b][1], pr, tr.y);
+                pfma(ai[b][0], pi, tr.x);
+                pfma(ai[b][1], pi, tr.y);
+            }
+        }
+#pragma unroll
+        for (int b = 0; b < 4; b++)
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                const float2 r = upk(ar[b][k]), m = upk(ai[b][k]);
+                two_sum(hr[4 * b + 2 * k], lr[4 * b + 2 * k], r.x);
+                two_sum(hr[4 * b + 2 * k + 1], lr[4 * b + 2 * k + 1], r.y);
+                two_sum(hi[4 * b + 2 * k], li[4 * b + 2 * k], m.x);
+                two_sum(hi[4 * b + 2 * k + 1], li[4 * b + 2 * k + 1], m.y);
+            }
     }
+    // the groups' sums through shared memory, in group order
+    double2 *sd = reinterpret_cast<double2 *>(dsm4); // [group][tile][16]
+    __syncthreads();
+    if (on && grp > 0) {
+#pragma unroll
+        for (int k = 0; k < 16; k++)
+            sd[(size_t(grp - 1) * ntile + tile) * 16 + k] =
+                make_double2(double(hr[k]) + double(lr[k]), double(hi[k]) + double(li[k]));
+    }
+    __syncthreads();
+    if (!on || grp > 0) return;
+    double2 *p = part + size_t(blockIdx.x) * cout * nah;
+#pragma unroll
+    for (int b = 0; b < 4; b++)
+#pragma unroll
+        for (int a = 0; a < 4; a++) {
+            const int bb = 4 * tb + b, aa = 4 * ta + a, k = 4 * b + a;
+            if (bb >= cout || aa >= nah) continue;
+            double2 t = make_double2(double(hr[k]) + double(lr[k]), double(hi[k]) + double(li[k]));
+            for (int w = 1; w < groups; w++) {
+                const double2 o = sd[(size_t(w - 1) * ntile + tile) * 16 + k];
+                t.x += o.x;
+                t.y += o.y;
+            }
+            p[bb * nah + aa] = t;
+        }
 }
 
-__global__ void k_net_wgrad_finish(int nblocks, int ntrip, const double2 *part, float2 *gw)
+// gw[q] = sum of the nparts partial sums: 32 weights per block, each warp every eighth
+// part, the eight sums in a fixed order
+__global__ void __launch_bounds__(256) k_net_wgrad_finish(int nparts, int ntrip, const double2 *part, float2 *gw)
 {
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < ntrip; q += gridDim.x * blockDim.x) {
-        double r = 0, i = 0;
-        for (int b = 0; b < nblocks; b++) {
-            r += part[size_t(b) * ntrip + q].x;
-            i += part[size_t(b) * ntrip + q].y;
+    __shared__ double2 sh[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = blockIdx.x * 32 + lane;
+    double2 t = make_double2(0, 0);
+    if (q < ntrip)
+        for (int b = warp; b < nparts; b += 8) {
+            const double2 v = part[size_t(b) * ntrip + q];
+            t.x += v.x;
+            t.y += v.y;
         }
-        gw[q] = make_float2(float(r), float(i));
+    sh[warp][lane] = t;
+    __syncthreads();
+    if (warp > 0 || q >= ntrip) return;
+    for (int w = 1; w < 8; w++) {
+        t.x += sh[w][lane].x;
+        t.y += sh[w][lane].y;
     }
+    gw[q] = make_float2(float(t.x), float(t.y));
 }
 
 // Adam step on n real parameters (Kingma & Ba, ICLR 2015)
@@ -252,20 +420,29 @@ hisq_status hisq_net_layer(hisq_ctx *ctx, int cin, int cout, const float *w_dev,
     if (!ctx->links_loaded) return set_err(ctx, HISQ_ERR_STATE, "links not loaded");
     HISQ_CUDA(cudaSetDevice(ctx->device));
     const int co = adjoint ? cin : cout, ci = adjoint ? cout : cin;
-    const size_t smem = sizeof(float2) * (size_t(co) * ci * kNetHops + size_t(kNetSites) * ci * kNetHops * 3);
-    static bool attr = false;
-    if (!attr) {
-        HISQ_CUDA(cudaFuncSetAttribute(k_net_layer, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-        attr = true;
-    }
-    const int nblk = (ctx->g.V + kNetSites - 1) / kNetSites;
-    const int grid = std::min(nblk, ctx->num_sms * 4);
     const int nk = ctx->long_recon == 18 ? 2 : 1;
-    ctx->launches++;
-    k_net_layer<<<grid, 256, smem, ctx->stream>>>(ctx->g, ctx->links_f[0], ctx->links_f[1], nk, (const float2 *)w_dev,
-                                                  cin, cout, adjoint, w_bf16, (const float2 *)in_dev, (float2 *)out_dev);
-    HISQ_CUDA(cudaGetLastError());
-    return HISQ_OK;
+    const int nblk = (ctx->g.V + kNetThreads - 1) / kNetThreads;
+    // output channels per thread: 16, fewer where the layer has fewer or the lattice
+    // leaves fewer than four blocks per SM
+    int P = (co + 1) / 2 <= 1 ? 1 : ((co + 1) / 2 <= 2 ? 2 : ((co + 1) / 2 <= 4 ? 4 : 8));
+    while (P > 1 && nblk * ((co + 2 * P - 1) / (2 * P)) < 4 * ctx->num_sms) P /= 2;
+    auto launch = [&](auto kern, int per_sm) -> hisq_status {
+        const int ny = (co + 2 * P - 1) / (2 * P);
+        const int gx = std::min(nblk, std::max(1, ctx->num_sms * per_sm / ny));
+        const size_t smem = sizeof(float4) * kNetHops * ci * P;
+        ctx->launches++;
+        kern<<<dim3(gx, ny), kNetThreads, smem, ctx->stream>>>(ctx->g, ctx->links_f[0], ctx->links_f[1], nk,
+                                                               (const float2 *)w_dev, cin, cout, adjoint, w_bf16,
+                                                               (const float2 *)in_dev, (float2 *)out_dev);
+        HISQ_CUDA(cudaGetLastError());
+        return HISQ_OK;
+    };
+    switch (P) {
+    case 1: return launch(k_net_layer<1>, 16);
+    case 2: return launch(k_net_layer<2>, 8);
+    case 4: return launch(k_net_layer<4>, 3);
+    default: return launch(k_net_layer<8>, 2);
+    }
 }
 
 hisq_status hisq_net_wgrad(hisq_ctx *ctx, int cin, int cout, const float *in_dev, const float *gout_dev, float *gw_dev)
@@ -275,23 +452,22 @@ hisq_status hisq_net_wgrad(hisq_ctx *ctx, int cin, int cout, const float *in_dev
         return set_err(ctx, HISQ_ERR_INVALID_ARG, "network gradient: 1..16 channels, device pointers");
     if (!ctx->links_loaded) return set_err(ctx, HISQ_ERR_STATE, "links not loaded");
     HISQ_CUDA(cudaSetDevice(ctx->device));
-    const size_t smem = sizeof(float2) * (size_t(kNetSites) * cin * kNetHops * 3 + size_t(kNetSites) * cout * 3);
-    static bool attr = false;
-    if (!attr) {
-        HISQ_CUDA(cudaFuncSetAttribute(k_net_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-        attr = true;
-    }
-    const int nblk = (ctx->g.V + kNetSites - 1) / kNetSites;
-    const int grid = std::min(nblk, ctx->num_sms * 2);
+    const size_t smem = size_t(kWgRows) * (2 * kWgPitch * sizeof(float) + kNetMaxC * sizeof(float2));
+    HISQ_CUDA(cudaFuncSetAttribute(k_net_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    const int nblk = (ctx->g.V + kWgSites - 1) / kWgSites;
+    const int grid = std::min(nblk, ctx->num_sms * 3);
     const int ntrip = cin * cout * kNetHops;
+    const int ntile = ((cin * kNetHops + 3) / 4) * ((cout + 3) / 4);
+    const int groups = std::max(1, std::min(kWgThreads / ntile, 12));
     double2 *part = (double2 *)get_buf(ctx, BUF_NET_PART, sizeof(double2) * size_t(grid) * ntrip);
     if (!part) return HISQ_ERR_OOM;
     const int nk = ctx->long_recon == 18 ? 2 : 1;
     ctx->launches += 2;
-    k_net_wgrad<<<grid, 256, smem, ctx->stream>>>(ctx->g, ctx->links_f[0], ctx->links_f[1], nk, cin, cout,
-                                                  (const float2 *)in_dev, (const float2 *)gout_dev, part);
+    k_net_wgrad<<<grid, kWgThreads, smem, ctx->stream>>>(ctx->g, ctx->links_f[0], ctx->links_f[1], nk, cin, cout,
+                                                         (const float2 *)in_dev, (const float2 *)gout_dev, groups,
+                                                         part);
     HISQ_CUDA(cudaGetLastError());
-    k_net_wgrad_finish<<<(ntrip + 255) / 256, 256, 0, ctx->stream>>>(grid, ntrip, part, (float2 *)gw_dev);
+    k_net_wgrad_finish<<<(ntrip + 31) / 32, 256, 0, ctx->stream>>>(grid, ntrip, part, (float2 *)gw_dev);
     HISQ_CUDA(cudaGetLastError());
     return HISQ_OK;
 }
