@@ -149,8 +149,13 @@ struct LinksH12 {
 };
 
 // ------------------------------------------------------------- the kernel
+// At most 128 registers, two blocks per SM: the compiler then keeps enough link loads in
+// flight (left to itself it chose 80 to 92 registers and three blocks).  32^3x64, D_oe and
+// fused update, FP16 vectors and 12-real long links: 161 / 170 us, 171 / 172 without the
+// bound; FP32 vectors, 18-real: 192 / 206 us, 202 / 222 without; three blocks 164 / 173
+// and 194 / 208.
 template <class SIn, class Lk, class L12T, bool R12, class Epi>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
     k_dslash(Geom g, int par, Lk L, L12T L12, float c3, SIn in, Epi epi, RedArgs ra, int do_red)
 {
     typedef typename Lk::real R;
