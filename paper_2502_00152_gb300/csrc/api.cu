@@ -240,10 +240,11 @@ hisq_status hisq_create(const int dims[4], int t_antiperiodic, int device, void 
     if (!ctx->g.oob || cudaMemset(ctx->g.oob, 0, sizeof(int)) != cudaSuccess) return fail(HISQ_ERR_OOM);
     ctx->max_red_blocks = ctx->num_sms * 16;
     ctx->partials = (double *)dev_alloc(ctx, sizeof(double) * ctx->max_red_blocks * kMaxRedVals);
-    ctx->ticket = (unsigned int *)dev_alloc(ctx, 256);
+    ctx->ticket = (unsigned int *)dev_alloc(ctx, 256 + sizeof(unsigned int) * kMaxBatch);
+    ctx->rhs_ticket = ctx->ticket ? ctx->ticket + 64 : nullptr;
     ctx->scal = (DevScalars *)dev_alloc(ctx, sizeof(DevScalars));
     if (!ctx->partials || !ctx->ticket || !ctx->scal) return fail(HISQ_ERR_OOM);
-    if (cudaMemset(ctx->ticket, 0, 256) != cudaSuccess || cudaMemset(ctx->scal, 0, sizeof(DevScalars)) != cudaSuccess)
+    if (cudaMemset(ctx->ticket, 0, 256 + sizeof(unsigned int) * kMaxBatch) != cudaSuccess || cudaMemset(ctx->scal, 0, sizeof(DevScalars)) != cudaSuccess)
         return fail(HISQ_ERR_CUDA);
     if (cudaHostAlloc((void **)&ctx->monitor_h, sizeof(double) * ctx->monitor_len, cudaHostAllocMapped) != cudaSuccess)
         return fail(HISQ_ERR_OOM);

@@ -54,7 +54,7 @@ static bool dual_residual(const hisq_ctx *ctx) { return ctx->eig.prec == 32; }
         if (s_ != HISQ_OK) return s_;           \
     } while (0)
 
-enum { BS_Y = 0, BS_ETAE = 1, BS_ETAO = 2, BS_R = 3, BS_RE = 4, BS_RO = 5, BS_PP = 6, BS_RHS = 16 };
+enum { BS_Y = 0, BS_ETAE = 1, BS_ETAO = 2, BS_R = 3, BS_RE = 4, BS_RO = 5, BS_RHS = 16 };
 
 static hisq_status residual_hi_b(hisq_ctx *ctx, const double *b, const double *x, double *r, double *tmp_odd, int slot)
 {
@@ -83,14 +83,6 @@ static hisq_status deflate_pair_b(hisq_ctx *ctx, int n, bool df, const double *b
     TRY(launch_defl_project(ctx, n, ctx->eig.prec, ctx->eig.vecs, 64, r, c));
     TRY(launch_defl_expand2(ctx, n, ctx->eig.prec, ctx->eig.vecs, c, eps, 4.0 * ctx->mass * ctx->mass, x, r));
     return launch_norm2(ctx, 64, r, slot);
-}
-
-// copy selected fields of the batch scalars of right-hand side j to the device
-static hisq_status set_rhs_scalars(hisq_ctx *ctx, int j, double rr, double pp)
-{
-    HISQ_CUDA(cudaMemcpyAsync(&ctx->bscal->rr[j], &rr, sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-    HISQ_CUDA(cudaMemcpyAsync(&ctx->bscal->pp[j], &pp, sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
-    return HISQ_OK;
 }
 
 static hisq_status set_active(hisq_ctx *ctx, const std::vector<int> &act)
@@ -181,8 +173,6 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
     auto xh = [&](int j) { return (double *)(XH + s64 * j); };
     auto rh = [&](int j) { return (double *)(RH + s64 * j); };
     auto xs = [&](int j) { return (void *)(XS + sx * j); };
-    auto rs = [&](int j) { return (void *)(RS + ssl * j); };
-    auto pj = [&](int j) { return (void *)(PP + ssl * j); };
     // tensor-core deflation of the right-hand sides `fields` (at most 32):
     // x_j += V Lambda^-1 V^dag r_j and the matching r_j, |r_j| into rt[j]
     auto tc_group = [&](const std::vector<int> &fields, int n_defl, std::vector<double> &rt) -> hisq_status {
@@ -383,6 +373,22 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
         }
         defl_s += std::chrono::duration<double>(std::chrono::steady_clock::now() - d0).count();
     }
+    // sloppy state of right-hand side j after its residual has changed: noted, and formed
+    // for all of a round in one launch
+    BatchRestart todo;
+    todo.k = 0;
+    auto finalize = [&](int j, bool restart) {
+        todo.id[todo.k] = j;
+        todo.restart[todo.k] = restart;
+        todo.rr[todo.k] = rt[j] * rt[j];
+        todo.k++;
+        r_last[j] = rt[j];
+    };
+    auto restart_all = [&]() -> hisq_status {
+        TRY(launch_batch_restart(ctx, prec, todo, RH, RS, XS, PP));
+        todo.k = 0;
+        return HISQ_OK;
+    };
     for (int j = 0; j < k; j++) {
         if (etanorm[j] > 0) TRY(certify(j));
         r_last[j] = r_defl[j] = r_best[j] = rn_seen[j] = rt[j];
@@ -392,11 +398,9 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
             st[j].converged = 1;
             continue;
         }
-        TRY(launch_convert(ctx, rh(j), 64, rs(j), prec));
-        TRY(launch_convert(ctx, rh(j), 64, pj(j), prec));
-        TRY(launch_zero(ctx, xs(j), xprec));
-        TRY(set_rhs_scalars(ctx, j, rt[j] * rt[j], rt[j] * rt[j]));
+        finalize(j, true);
     }
+    TRY(restart_all());
     std::vector<int> act;
     for (int j = 0; j < k; j++)
         if (!done[j]) act.push_back(j);
@@ -569,21 +573,6 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
         checked = it;
         bool changed = false;
         std::vector<int> redefl;
-        // sloppy state of right-hand side j after a reliable update or a re-deflation
-        auto finalize = [&](int j, bool restart) -> hisq_status {
-            TRY(launch_convert(ctx, rh(j), 64, rs(j), prec));
-            TRY(launch_zero(ctx, xs(j), xprec));
-            double pp = rt[j] * rt[j];
-            if (restart) {
-                TRY(launch_convert(ctx, rh(j), 64, pj(j), prec));
-            } else {
-                TRY(launch_norm2(ctx, prec, pj(j), BS_PP));
-                TRY(read_slots(ctx, BS_PP, 1, &pp));
-            }
-            TRY(set_rhs_scalars(ctx, j, rt[j] * rt[j], pp));
-            r_last[j] = rt[j];
-            return HISQ_OK;
-        };
         // the double-float residuals of this round together (one pass over the links)
         std::vector<int> gdf;
         std::vector<double> r2df(k, 0.0);
@@ -629,7 +618,8 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
                 redefl.push_back(j);
                 return HISQ_OK;
             }
-            return finalize(j, restart);
+            finalize(j, restart);
+            return HISQ_OK;
         };
         // the FP64 residuals of this round by groups, the others one by one
         std::vector<int> g64;
@@ -686,15 +676,16 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
                     changed = true;
                     continue;
                 }
-                TRY(finalize(j, true));
+                finalize(j, true);
             }
         }
+        TRY(restart_all());
         if (changed) {
             act.clear();
             for (int j = 0; j < k; j++)
                 if (!done[j]) act.push_back(j);
+            TRY(set_active(ctx, act));
         }
-        TRY(set_active(ctx, act));
     }
     HISQ_CUDA(cudaStreamSynchronize(ctx->stream));
     retire(it);

@@ -619,6 +619,28 @@ struct RedArgs {
     int slot0;              // first slot for FIN_STORE
 };
 
+// Sums of N (a power of two) doubles over the lanes of a warp: each step halves the values
+// a lane carries and sends the other half to its partner, so N + 4 - log2 N additions
+// instead of 5 N (an FP64 addition of a warp takes 19 clocks of the SM's FP64 pipe).  The
+// sum of value i is left in v[0] of the lanes whose upper log2 N bits are i.
+template <int N>
+__device__ __forceinline__ void warp_sums(double (&v)[N])
+{
+    const int lane = threadIdx.x & 31;
+    int off = 16;
+#pragma unroll
+    for (int n = N / 2; n >= 1; n /= 2, off /= 2) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < n; i++) {
+            const double mine = up ? v[i + n] : v[i], other = up ? v[i] : v[i + n];
+            v[i] = mine + __shfl_xor_sync(0xffffffffu, other, off);
+        }
+    }
+#pragma unroll
+    for (; off >= 1; off /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+}
+
 // Deterministic grid reduction of NV doubles: each block writes its partial
 // sums, the last block to finish adds the partials in block order.
 template <int NV>
@@ -777,6 +799,7 @@ struct hisq_ctx {
     // reduction scratch
     double *partials = nullptr;
     unsigned int *ticket = nullptr;
+    unsigned int *rhs_ticket = nullptr; // one per right-hand side (launches with a block row per field)
     hisq::DevScalars *scal = nullptr;
     double *monitor_h = nullptr; // host-mapped
     double *monitor_d = nullptr;
@@ -1059,6 +1082,14 @@ hisq_status launch_mrhs_dslash_tt(hisq_ctx *ctx, int prec, int link_prec, void *
 hisq_status launch_mrhs_dslash_update(hisq_ctx *ctx, int prec, int link_prec, void *tmp, void *p, void *x, void *r,
                                       int kact);
 hisq_status launch_mrhs_p_update(hisq_ctx *ctx, int prec, void *r, void *p, int kact);
+// sloppy state of right-hand sides id[0..k-1] of a batch from their FP64 residuals rh
+struct BatchRestart {
+    int k;
+    int id[kMaxBatch];
+    bool restart[kMaxBatch]; // p = r (else p is kept)
+    double rr[kMaxBatch];    // |r|^2
+};
+hisq_status launch_batch_restart(hisq_ctx *ctx, int prec, const BatchRestart &b, void *rh, void *rs, void *xs, void *ps);
 // blocks of k ordinary FP32 fields (eigensolver): slots 0..k-1 active, and
 // out_j = a x_j + b y_j + c D(in_j) on output parity par (x, y nullable)
 hisq_status mrhs_set_identity(hisq_ctx *ctx, int k);

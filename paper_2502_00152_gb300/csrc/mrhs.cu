@@ -64,8 +64,8 @@ struct MrhsTile {
     __device__ __forceinline__ int group() const { return (threadIdx.x >> 5) / nch; }
 };
 
-// per-slot sums of R values per thread into partials[block][slot] (lanes by a
-// fixed shuffle tree, site groups in order) and, in the last block, the sums
+// per-slot sums of R values per thread into partials[block][slot] (warp_sums,
+// site groups in order) and, in the last block, the sums
 // over blocks (a warp per slot: lanes over the blocks, then a fixed shuffle tree;
 // one thread per slot took up to 10 us over 304 blocks) followed by the batch
 // finish operation.  The slots of a block start at first (one of gridDim.y parts).
@@ -76,16 +76,14 @@ __device__ __forceinline__ void batch_reduce(double (&v)[R], const MrhsTile &tl,
     __shared__ double sh[16][kMaxBatch]; // [site group][slot of the block]
     __shared__ bool am_last;
     const int lane = threadIdx.x & 31;
+    constexpr int N = R == 3 ? 4 : R;
+    double w4[N];
 #pragma unroll
-    for (int u = 0; u < R; u++)
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) v[u] += __shfl_down_sync(0xffffffffu, v[u], o);
-    if (lane == 0) {
-#pragma unroll
-        for (int u = 0; u < R; u++) {
-            const int q = tl.chunk() * R + u;
-            if (q < kMaxBatch) sh[tl.group()][q] = v[u];
-        }
+    for (int u = 0; u < N; u++) w4[u] = u < R ? v[u] : 0.0;
+    warp_sums<N>(w4);
+    {
+        const int u = lane / (32 / N), q = tl.chunk() * R + u;
+        if (lane % (32 / N) == 0 && u < R && q < kMaxBatch) sh[tl.group()][q] = w4[0];
     }
     __syncthreads();
     for (int q = threadIdx.x; q < tl.nch * R && first + q < kact; q += blockDim.x) {
@@ -1916,6 +1914,81 @@ hisq_status launch_mrhs_p_update(hisq_ctx *ctx, int prec, void *r, void *p, int 
     if (prec == 32) return run_p_update<SpinorF>(ctx, r, p, kact, prec);
     if (prec == 16) return run_p_update<SpinorH>(ctx, r, p, kact, prec);
     return set_err(ctx, HISQ_ERR_INVALID_ARG, "batched sloppy precision must be 32 or 16");
+}
+
+// The sloppy state of several right-hand sides after a residual, in one launch (blockIdx.y:
+// which): r_j = the FP64 residual, x_j = 0, and p_j = r_j (restart) or |p_j|^2; the batch
+// scalars rr_j = |r_j|^2 (known to the host) and pp_j.  It replaces, for each right-hand
+// side, two conversions or a norm with its readback, a memset and two copies of scalars.
+template <class S>
+__global__ void __launch_bounds__(256)
+    k_batch_restart(int Vh, BatchRestart b, BatchF<SpinorD> rh, BatchF<S> rs, BatchF<SpinorF> xs, BatchF<S> ps,
+                    BatchScalars *scal, double *partials, unsigned int *ticket)
+{
+    const int q = blockIdx.y, j = b.id[q];
+    const bool restart = b.restart[q];
+    const SpinorD r0 = rh.at(j);
+    const S r = rs.at(j), p = ps.at(j);
+    const SpinorF x = xs.at(j);
+    CVec<float> z;
+    z.zero();
+    double red = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Vh; i += gridDim.x * blockDim.x) {
+        const CVec<float> v = cvt<float>(r0.load(i));
+        r.store(i, v);
+        x.store(i, z);
+        if (restart)
+            p.store(i, v);
+        else
+            red += double(p.load(i).norm2());
+    }
+    // sums over lanes by a shuffle tree, warps in order, blocks by the field's last block
+    __shared__ double sh[8];
+    __shared__ bool am_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (!restart) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) red += __shfl_down_sync(0xffffffffu, red, o);
+        if (lane == 0) sh[warp] = red;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0;
+        if (!restart)
+            for (int w = 0; w < 8; w++) t += sh[w];
+        partials[size_t(blockIdx.x) * kMaxBatch + q] = t;
+        __threadfence();
+        am_last = atomicAdd(ticket + q, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!am_last || warp > 0) return;
+    __threadfence();
+    double t = 0;
+    for (int w = lane; w < int(gridDim.x); w += 32) t += __ldcg(partials + size_t(w) * kMaxBatch + q);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) {
+        scal->rr[j] = b.rr[q];
+        scal->pp[j] = restart ? b.rr[q] : t;
+        ticket[q] = 0u;
+        __threadfence();
+    }
+}
+
+hisq_status launch_batch_restart(hisq_ctx *ctx, int prec, const BatchRestart &b, void *rh, void *rs, void *xs, void *ps)
+{
+    if (b.k < 1) return HISQ_OK;
+    const int Vh = ctx->g.Vh;
+    auto go = [&](auto tagS) -> hisq_status {
+        typedef decltype(tagS) S;
+        const dim3 grid(std::max(1, std::min(grid_for(ctx, Vh, 256, 8), ctx->num_sms * 8 / b.k)), b.k);
+        k_batch_restart<S><<<grid, 256, 0, ctx->stream>>>(Vh, b, batchf<SpinorD>(rh, Vh, 64), batchf<S>(rs, Vh, prec),
+                                                          batchf<SpinorF>(xs, Vh, 32), batchf<S>(ps, Vh, prec),
+                                                          ctx->bscal, ctx->bpartials, ctx->rhs_ticket);
+        const cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? HISQ_OK : cuda_err(ctx, e, "batch restart launch");
+    };
+    return prec == 16 ? go(SpinorH{}) : go(SpinorF{});
 }
 
 } // namespace hisq
