@@ -3,6 +3,7 @@
 // deflation projection and expansion of Eq. 4 (x = sum_i v_i lambda_i^-1 v_i^dag b),
 // and the Ritz basis rotation of the thick-restart Lanczos eigensolver.
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -285,32 +286,47 @@ __device__ __forceinline__ SpinorE spinor_at<SpinorE>(const char *base, size_t s
     return make_spinorE(const_cast<char *>(base) + stride * i, Vh);
 }
 
-constexpr int kDeflVG = 8;        // vectors per block in the projection
-constexpr int kDeflSites = 4096;  // sites per block in the projection
+constexpr int kDeflSites = 4096; // sites per block in the projection: 16 per thread, summed in FP32
 
-// partial[i][chunk] = sum over the chunk's sites of v_i^dag b
+// vectors per block: 8, fewer where that gives fewer blocks than half the SMs (the sum of
+// a vector, and so its rounding, does not depend on it).  Projection, 8 -> chosen: 37
+// vectors of 9,240 sites 23.8 -> 10.8 us (1), 16 of 20,736 23.1 -> 10.4 (1), 200 of 4,096
+// 23.1 -> 15.4 (2; 1: 18.0); 64 of 65,536 stay at 8: 24.4 (4: 24.1, 2: 38.7).
+static int defl_vectors_per_block(const hisq_ctx *ctx, int n)
+{
+    const long chunks = (ctx->g.Vh + kDeflSites - 1) / kDeflSites;
+    for (int vg : {8, 4, 2})
+        if ((n + vg - 1) / vg * chunks >= ctx->num_sms / 2) return vg;
+    return 1;
+}
+
+// partial[i][chunk] = sum over the chunk's sites of v_i^dag b.  HBM bound: 128 FP32 vectors
+// of 331,776 sites 205 -> 165 us (6.2 TB/s) when the 16 sums of a block took warp_sums
+// (16 x 5 FP64 additions per warp before, a quarter of the kernel's time).
 // (16 vectors per block with unconditional loads was measured 1.8x slower:
 // at 128 registers it halves the resident blocks; 8 vectors fit 80 registers)
-template <class SV, class SB>
+template <class SV, class SB, int VG>
 __global__ void __launch_bounds__(256, 3)
     k_defl_project(int Vh, int n, const char *__restrict__ V0, size_t vstride, SB b, double2 *part, int nchunks)
 {
-    const int g0 = blockIdx.x * kDeflVG;
+    const int g0 = blockIdx.x * VG;
     const int chunk = blockIdx.y;
     const int cb0 = chunk * kDeflSites;
     const int cb1 = min(Vh, cb0 + kDeflSites);
-    float ar[kDeflVG], ai[kDeflVG];
+    float ar[VG], ai[VG];
 #pragma unroll
-    for (int j = 0; j < kDeflVG; j++) ar[j] = ai[j] = 0.f;
+    for (int j = 0; j < VG; j++) ar[j] = ai[j] = 0.f;
+    constexpr int kUn = VG <= 2 ? 4 : 1;
+#pragma unroll kUn
     for (int cb = cb0 + threadIdx.x; cb < cb1; cb += blockDim.x) {
         CVec<float> bv = cvt<float>(b.load(cb));
         // every vector's load is unconditional (a vector past n reads vector
         // n - 1 and is not accumulated), so all of them are in flight at once
-        CVec<float> v[kDeflVG];
+        CVec<float> v[VG];
 #pragma unroll
-        for (int j = 0; j < kDeflVG; j++) v[j] = spinor_at<SV>(V0, vstride, min(g0 + j, n - 1), Vh).load(cb);
+        for (int j = 0; j < VG; j++) v[j] = spinor_at<SV>(V0, vstride, min(g0 + j, n - 1), Vh).load(cb);
 #pragma unroll
-        for (int j = 0; j < kDeflVG; j++) {
+        for (int j = 0; j < VG; j++) {
             if (g0 + j < n) {
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
@@ -320,95 +336,119 @@ __global__ void __launch_bounds__(256, 3)
             }
         }
     }
-    // block reduction (fixed order)
-    __shared__ double sh[2 * kDeflVG][8];
+    // block reduction (fixed order): value j = re, VG + j = im of vector j
+    __shared__ double sh[2 * VG][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double t[2 * VG];
 #pragma unroll
-    for (int j = 0; j < kDeflVG; j++) {
-        double xr = ar[j], xi = ai[j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            xr += __shfl_down_sync(0xffffffffu, xr, o);
-            xi += __shfl_down_sync(0xffffffffu, xi, o);
-        }
-        if (lane == 0) {
-            sh[2 * j][warp] = xr;
-            sh[2 * j + 1][warp] = xi;
-        }
+    for (int j = 0; j < VG; j++) {
+        t[j] = ar[j];
+        t[VG + j] = ai[j];
     }
+    warp_sums<2 * VG>(t);
+    if (lane % (16 / VG) == 0) sh[lane / (16 / VG)][warp] = t[0];
     __syncthreads();
-    if (threadIdx.x < kDeflVG && g0 + threadIdx.x < n) {
+    if (threadIdx.x < VG && g0 + threadIdx.x < n) {
         const int j = threadIdx.x;
         double xr = 0, xi = 0;
         for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
-            xr += sh[2 * j][w];
-            xi += sh[2 * j + 1][w];
+            xr += sh[j][w];
+            xi += sh[VG + j][w];
         }
         part[size_t(g0 + j) * nchunks + chunk] = make_double2(xr, xi);
     }
 }
 
-// c_i = sum_chunks partial[i][chunk] (fixed order); optional d_i = c_i / lam_i
-__global__ void k_defl_finish(int n, int nchunks, const double2 *part, double2 *c, const double *lam, double shift)
+// c_i = sum_chunks partial[i][chunk], a warp per vector: lanes over the chunks, then a
+// fixed shuffle tree; with lam, c_i / (lam_i + shift)
+__global__ void __launch_bounds__(128) k_defl_finish(int n, int nchunks, const double2 *part, double2 *c,
+                                                     const double *lam, double shift)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        double xr = 0, xi = 0;
-        const double2 *q = part + size_t(i) * nchunks;
-        for (int k = 0; k < nchunks; k++) {
-            xr += q[k].x;
-            xi += q[k].y;
-        }
-        if (lam) {
-            const double l = lam[i] + shift;
-            xr /= l;
-            xi /= l;
-        }
-        c[i] = make_double2(xr, xi);
+    const int i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= n) return;
+    double xr = 0, xi = 0;
+    const double2 *q = part + size_t(i) * nchunks;
+    for (int k = lane; k < nchunks; k += 32) {
+        xr += q[k].x;
+        xi += q[k].y;
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        xr += __shfl_down_sync(0xffffffffu, xr, o);
+        xi += __shfl_down_sync(0xffffffffu, xi, o);
+    }
+    if (lane) return;
+    if (lam) {
+        const double l = lam[i] + shift;
+        xr /= l;
+        xi /= l;
+    }
+    c[i] = make_double2(xr, xi);
 }
 
 static hisq_status ensure_defl_scratch(hisq_ctx *ctx, size_t bytes, double2 **out);
 
-hisq_status launch_defl_project(hisq_ctx *ctx, int n, int vprec, const void *V, int bprec, const void *b,
-                                double *c_dev)
+// c_i = v_i^dag b (divided by lam_i + shift with lam) with the partial sums in `part`
+static hisq_status project_into(hisq_ctx *ctx, int n, int vprec, const void *V, int bprec, const void *b, double *c_dev,
+                                double2 *part, const double *lam, double shift)
 {
     const int Vh = ctx->g.Vh;
     const int nchunks = (Vh + kDeflSites - 1) / kDeflSites;
-    double2 *part = nullptr;
-    hisq_status st = ensure_defl_scratch(ctx, size_t(n) * nchunks * sizeof(double2), &part);
-    if (st != HISQ_OK) return st;
-    dim3 grid((n + kDeflVG - 1) / kDeflVG, nchunks);
+    const int vg = defl_vectors_per_block(ctx, n);
+    const dim3 grid((n + vg - 1) / vg, nchunks);
     const size_t stride = spinor_bytes(vprec, Vh);
-    if (vprec != 32 && vprec != 16 && vprec != HISQ_PREC_BF16 && vprec != HISQ_PREC_HALF_EV)
-        return set_err(ctx, HISQ_ERR_INVALID_ARG, "eigenvector precision must be 32, 16, 15 (BF16) or 14 (FP16)");
     if (bprec != 64 && bprec != 32) return set_err(ctx, HISQ_ERR_INVALID_ARG, "projected vector must be FP64 or FP32");
     void *bb = const_cast<void *>(b);
-    if (vprec == 32 && bprec == 64)
-        k_defl_project<SpinorF, SpinorD><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, make_spinorD(bb, Vh), part, nchunks);
-    else if (vprec == 32)
-        k_defl_project<SpinorF, SpinorF><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, make_spinorF(bb, Vh), part, nchunks);
-    else if (vprec == HISQ_PREC_BF16 && bprec == 64)
-        k_defl_project<SpinorB, SpinorD><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, make_spinorD(bb, Vh), part, nchunks);
-    else if (vprec == HISQ_PREC_BF16)
-        k_defl_project<SpinorB, SpinorF><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, make_spinorF(bb, Vh), part, nchunks);
-    else if (vprec == HISQ_PREC_HALF_EV && bprec == 64)
-        k_defl_project<SpinorE, SpinorD><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, make_spinorD(bb, Vh), part, nchunks);
-    else if (vprec == HISQ_PREC_HALF_EV)
-        k_defl_project<SpinorE, SpinorF><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, make_spinorF(bb, Vh), part, nchunks);
-    else if (bprec == 64)
-        k_defl_project<SpinorH, SpinorD><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, make_spinorD(bb, Vh), part, nchunks);
-    else
-        k_defl_project<SpinorH, SpinorF><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, make_spinorF(bb, Vh), part, nchunks);
+    auto launch = [&](auto tagV, auto sb, auto v) {
+        typedef decltype(tagV) SV;
+        typedef decltype(sb) SB;
+        constexpr int VG = decltype(v)::value;
+        k_defl_project<SV, SB, VG><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, sb, part, nchunks);
+    };
+    auto by_vg = [&](auto tagV, auto sb) {
+        switch (vg) {
+        case 8: launch(tagV, sb, std::integral_constant<int, 8>{}); break;
+        case 4: launch(tagV, sb, std::integral_constant<int, 4>{}); break;
+        case 2: launch(tagV, sb, std::integral_constant<int, 2>{}); break;
+        default: launch(tagV, sb, std::integral_constant<int, 1>{}); break;
+        }
+    };
+    auto go = [&](auto tagV) {
+        if (bprec == 64)
+            by_vg(tagV, make_spinorD(bb, Vh));
+        else
+            by_vg(tagV, make_spinorF(bb, Vh));
+    };
+    switch (vprec) {
+    case 32: go(SpinorF{}); break;
+    case 16: go(SpinorH{}); break;
+    case HISQ_PREC_BF16: go(SpinorB{}); break;
+    case HISQ_PREC_HALF_EV: go(SpinorE{}); break;
+    default: return set_err(ctx, HISQ_ERR_INVALID_ARG, "eigenvector precision must be 32, 16, 15 (BF16) or 14 (FP16)");
+    }
     LAUNCH_CHECK("defl_project");
     ctx->launches += 2;
-    k_defl_finish<<<(n + 127) / 128, 128, 0, ctx->stream>>>(n, nchunks, part, (double2 *)c_dev, nullptr, 0.0);
+    k_defl_finish<<<(n + 3) / 4, 128, 0, ctx->stream>>>(n, nchunks, part, (double2 *)c_dev, lam, shift);
     LAUNCH_CHECK("defl_finish");
     return HISQ_OK;
 }
 
-// x += coef * sum_i d_i v_i  (d in FP64 on the device, FP32 accumulation per site)
-template <class SV, class SX>
-__global__ void __launch_bounds__(256)
+hisq_status launch_defl_project(hisq_ctx *ctx, int n, int vprec, const void *V, int bprec, const void *b,
+                                double *c_dev, const double *lam, double shift)
+{
+    const int nchunks = (ctx->g.Vh + kDeflSites - 1) / kDeflSites;
+    double2 *part = nullptr;
+    hisq_status st = ensure_defl_scratch(ctx, size_t(n) * nchunks * sizeof(double2), &part);
+    if (st != HISQ_OK) return st;
+    return project_into(ctx, n, vprec, V, bprec, b, c_dev, part, lam, shift);
+}
+
+// x (+)= coef * sum_i d_i v_i  (d in FP64 on the device, FP32 accumulation per site)
+// HBM bound; 16 vectors' loads in flight per thread and three blocks per SM: 128 FP32
+// vectors of 331,776 sites 200 -> 151 us (6.7 TB/s), without the bound on the registers
+// 187, 8 in flight 162; 64 BF16 vectors of 65,536 sites 12.9 -> 9.9 us.
+template <class SV, class SX, bool ADD>
+__global__ void __launch_bounds__(256, 3)
     k_defl_expand(int Vh, int n, const char *__restrict__ V0, size_t vstride, const double2 *d, double coef, SX x)
 {
     extern __shared__ float2 sd[];
@@ -418,7 +458,7 @@ __global__ void __launch_bounds__(256)
     for (int cb = blockIdx.x * blockDim.x + threadIdx.x; cb < Vh; cb += gridDim.x * blockDim.x) {
         CVec<float> acc;
         acc.zero();
-#pragma unroll 4
+#pragma unroll 16
         for (int i = 0; i < n; i++) {
             CVec<float> v = spinor_at<SV>(V0, vstride, i, Vh).load(cb);
             const float2 w = sd[i];
@@ -428,8 +468,10 @@ __global__ void __launch_bounds__(256)
                 acc.im[c] = fmaf(w.x, v.im[c], fmaf(w.y, v.re[c], acc.im[c]));
             }
         }
-        auto xv = x.load(cb);
         typedef typename SX::real XR;
+        CVec<XR> xv;
+        xv.zero();
+        if (ADD) xv = x.load(cb);
 #pragma unroll
         for (int c = 0; c < 3; c++) {
             xv.re[c] += XR(acc.re[c]);
@@ -441,34 +483,36 @@ __global__ void __launch_bounds__(256)
 
 template <class SV, class SX>
 static hisq_status expand_go(hisq_ctx *ctx, int n, const void *V, size_t stride, const double *d, double coef, SX xs,
-                             size_t smem)
+                             size_t smem, bool add)
 {
-    auto k = k_defl_expand<SV, SX>;
-    int grid = grid_for(ctx, ctx->g.Vh, 256, occ(k, 256, smem));
-    k<<<grid, 256, smem, ctx->stream>>>(ctx->g.Vh, n, (const char *)V, stride, (const double2 *)d, coef, xs);
+    auto k = add ? k_defl_expand<SV, SX, true> : k_defl_expand<SV, SX, false>;
+    // small lattices: blocks of two warps, so that every SM has one
+    const int threads = ctx->g.Vh < 256 * 2 * ctx->num_sms ? 64 : 256;
+    int grid = grid_for(ctx, ctx->g.Vh, threads, occ(k, threads, smem));
+    k<<<grid, threads, smem, ctx->stream>>>(ctx->g.Vh, n, (const char *)V, stride, (const double2 *)d, coef, xs);
     LAUNCH_CHECK("defl_expand");
     return HISQ_OK;
 }
 
 hisq_status launch_defl_expand(hisq_ctx *ctx, int n, int vprec, const void *V, const double *d_dev, double coef,
-                               int xprec, void *x)
+                               int xprec, void *x, bool add)
 {
     const int Vh = ctx->g.Vh;
     if (n > 6144) return set_err(ctx, HISQ_ERR_INVALID_ARG, "at most 6144 deflation vectors");
     const size_t smem = size_t(n) * sizeof(float2);
     const size_t stride = spinor_bytes(vprec, Vh);
-    if (vprec == 32 && xprec == 64) return expand_go<SpinorF>(ctx, n, V, stride, d_dev, coef, make_spinorD(x, Vh), smem);
-    if (vprec == 32 && xprec == 32) return expand_go<SpinorF>(ctx, n, V, stride, d_dev, coef, make_spinorF(x, Vh), smem);
-    if (vprec == 16 && xprec == 64) return expand_go<SpinorH>(ctx, n, V, stride, d_dev, coef, make_spinorD(x, Vh), smem);
-    if (vprec == 16 && xprec == 32) return expand_go<SpinorH>(ctx, n, V, stride, d_dev, coef, make_spinorF(x, Vh), smem);
+    if (vprec == 32 && xprec == 64) return expand_go<SpinorF>(ctx, n, V, stride, d_dev, coef, make_spinorD(x, Vh), smem, add);
+    if (vprec == 32 && xprec == 32) return expand_go<SpinorF>(ctx, n, V, stride, d_dev, coef, make_spinorF(x, Vh), smem, add);
+    if (vprec == 16 && xprec == 64) return expand_go<SpinorH>(ctx, n, V, stride, d_dev, coef, make_spinorD(x, Vh), smem, add);
+    if (vprec == 16 && xprec == 32) return expand_go<SpinorH>(ctx, n, V, stride, d_dev, coef, make_spinorF(x, Vh), smem, add);
     if (vprec == HISQ_PREC_BF16 && xprec == 64)
-        return expand_go<SpinorB>(ctx, n, V, stride, d_dev, coef, make_spinorD(x, Vh), smem);
+        return expand_go<SpinorB>(ctx, n, V, stride, d_dev, coef, make_spinorD(x, Vh), smem, add);
     if (vprec == HISQ_PREC_BF16 && xprec == 32)
-        return expand_go<SpinorB>(ctx, n, V, stride, d_dev, coef, make_spinorF(x, Vh), smem);
+        return expand_go<SpinorB>(ctx, n, V, stride, d_dev, coef, make_spinorF(x, Vh), smem, add);
     if (vprec == HISQ_PREC_HALF_EV && xprec == 64)
-        return expand_go<SpinorE>(ctx, n, V, stride, d_dev, coef, make_spinorD(x, Vh), smem);
+        return expand_go<SpinorE>(ctx, n, V, stride, d_dev, coef, make_spinorD(x, Vh), smem, add);
     if (vprec == HISQ_PREC_HALF_EV && xprec == 32)
-        return expand_go<SpinorE>(ctx, n, V, stride, d_dev, coef, make_spinorF(x, Vh), smem);
+        return expand_go<SpinorE>(ctx, n, V, stride, d_dev, coef, make_spinorF(x, Vh), smem, add);
     return set_err(ctx, HISQ_ERR_INVALID_ARG, "bad deflation precisions");
 }
 
@@ -505,23 +549,6 @@ hisq_status launch_random_f(hisq_ctx *ctx, unsigned long long seed, void *out)
     int grid = grid_for(ctx, n, 256, occ(k_random_f, 256));
     k_random_f<<<grid, 256, 0, ctx->stream>>>(n, seed, (float *)out);
     LAUNCH_CHECK("random_f");
-    return HISQ_OK;
-}
-
-// d_i = c_i / (eps_i + shift) on the device
-__global__ void k_defl_scale(int n, double2 *c, const double *eps, double shift)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const double l = eps[i] + shift;
-        c[i] = make_double2(c[i].x / l, c[i].y / l);
-    }
-}
-
-hisq_status launch_defl_scale(hisq_ctx *ctx, int n, double *c_dev, const double *eps_dev, double shift)
-{
-    ctx->launches++;
-    k_defl_scale<<<(n + 127) / 128, 128, 0, ctx->stream>>>(n, (double2 *)c_dev, eps_dev, shift);
-    LAUNCH_CHECK("defl_scale");
     return HISQ_OK;
 }
 
@@ -630,32 +657,12 @@ namespace hisq {
 // number of site chunks of the deflation projection (partials per vector)
 int defl_project_chunks(int Vh) { return (Vh + kDeflSites - 1) / kDeflSites; }
 
-// The projection c_i = v_i^dag b with the partial sums in a buffer the caller
-// provides (at least n * defl_project_chunks(Vh) double2); b is FP64.
+// The projection with the partial sums in a buffer the caller provides (at least
+// n * defl_project_chunks(Vh) double2); b is FP64.
 hisq_status launch_defl_project_ext(hisq_ctx *ctx, int n, int vprec, const void *V, const double *b, double *c_dev,
-                                    void *part_buf)
+                                    void *part_buf, const double *lam, double shift)
 {
-    const int Vh = ctx->g.Vh;
-    const int nchunks = defl_project_chunks(Vh);
-    double2 *part = (double2 *)part_buf;
-    dim3 grid((n + kDeflVG - 1) / kDeflVG, nchunks);
-    const size_t stride = spinor_bytes(vprec, Vh);
-    SpinorD bs = make_spinorD(const_cast<double *>(b), Vh);
-    if (vprec == 32)
-        k_defl_project<SpinorF, SpinorD><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, bs, part, nchunks);
-    else if (vprec == 16)
-        k_defl_project<SpinorH, SpinorD><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, bs, part, nchunks);
-    else if (vprec == HISQ_PREC_BF16)
-        k_defl_project<SpinorB, SpinorD><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, bs, part, nchunks);
-    else if (vprec == HISQ_PREC_HALF_EV)
-        k_defl_project<SpinorE, SpinorD><<<grid, 256, 0, ctx->stream>>>(Vh, n, (const char *)V, stride, bs, part, nchunks);
-    else
-        return set_err(ctx, HISQ_ERR_INVALID_ARG, "eigenvector precision must be 32, 16, 15 (BF16) or 14 (FP16)");
-    LAUNCH_CHECK("defl_project_ext");
-    ctx->launches += 2;
-    k_defl_finish<<<(n + 127) / 128, 128, 0, ctx->stream>>>(n, nchunks, part, (double2 *)c_dev, nullptr, 0.0);
-    LAUNCH_CHECK("defl_finish_ext");
-    return HISQ_OK;
+    return project_into(ctx, n, vprec, V, 64, b, c_dev, (double2 *)part_buf, lam, shift);
 }
 
 } // namespace hisq

@@ -1062,13 +1062,12 @@ hisq_status launch_cdot(hisq_ctx *ctx, int prec, const void *x, const void *y, i
 hisq_status launch_scale_axpby_d(hisq_ctx *ctx, double a, const double *x, double b, double *y); // y = a x + b y
 
 // deflation (Eq. 4) over n stored vectors of precision vprec (32 or 16):
-// c_i = v_i^dag b (b FP64 or FP32), x += coef * sum_i d_i v_i (x FP64 or FP32)
+// c_i = v_i^dag b (b FP64 or FP32; with lam: / (lam_i + shift)), x += (add) or =
+// coef * sum_i d_i v_i (x FP64 or FP32)
 hisq_status launch_defl_project(hisq_ctx *ctx, int n, int vprec, const void *V, int bprec, const void *b,
-                                double *c_dev /* n complex, FP64 */);
+                                double *c_dev /* n complex, FP64 */, const double *lam = nullptr, double shift = 0);
 hisq_status launch_defl_expand(hisq_ctx *ctx, int n, int vprec, const void *V, const double *d_dev, double coef,
-                               int xprec, void *x);
-// d_i = c_i / (eps_i + shift) in place
-hisq_status launch_defl_scale(hisq_ctx *ctx, int n, double *c_dev, const double *eps_dev, double shift);
+                               int xprec, void *x, bool add = true);
 // FP32 field helpers for the eigensolver
 hisq_status launch_scale_f(hisq_ctx *ctx, double s, const void *in, void *out);
 hisq_status launch_random_f(hisq_ctx *ctx, unsigned long long seed, void *out);

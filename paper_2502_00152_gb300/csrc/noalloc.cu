@@ -8,7 +8,7 @@
 namespace hisq {
 int defl_project_chunks(int Vh);
 hisq_status launch_defl_project_ext(hisq_ctx *ctx, int n, int vprec, const void *V, const double *b, double *c_dev,
-                                    void *part_buf);
+                                    void *part_buf, const double *lam, double shift);
 } // namespace hisq
 
 using namespace hisq;
@@ -76,10 +76,8 @@ extern "C" hisq_status hisq_deflate_noalloc(hisq_ctx *ctx, int n, const double *
     double *c = reinterpret_cast<double *>(scratch + part_bytes);
     // every scratch byte used below is written by this call's kernels before it
     // is read; the eigenvalues come from the device copy kept with the pairs
-    st = launch_defl_project_ext(ctx, n, ctx->eig.prec, ctx->eig.vecs, b_dev, c, part);
+    st = launch_defl_project_ext(ctx, n, ctx->eig.prec, ctx->eig.vecs, b_dev, c, part, ctx->eig.eps_dev,
+                                 4.0 * ctx->mass * ctx->mass);
     if (st != HISQ_OK) return st;
-    st = launch_defl_scale(ctx, n, c, ctx->eig.eps_dev, 4.0 * ctx->mass * ctx->mass);
-    if (st != HISQ_OK) return st;
-    HISQ_CUDA(cudaMemsetAsync(x_dev, 0, spinor_bytes(64, Vh), ctx->stream));
-    return launch_defl_expand(ctx, n, ctx->eig.prec, ctx->eig.vecs, c, 1.0, 64, x_dev);
+    return launch_defl_expand(ctx, n, ctx->eig.prec, ctx->eig.vecs, c, 1.0, 64, x_dev, false);
 }

@@ -72,8 +72,7 @@ hisq_status deflate_add(hisq_ctx *ctx, int n, const double *r, double *x)
     double *eps = eig_eps_dev(ctx);
     double *c = (double *)get_buf(ctx, BUF_DEFL_C, sizeof(double) * 2 * (n > 0 ? n : 1));
     if (!eps || !c) return set_err(ctx, HISQ_ERR_OOM, "deflation buffers");
-    TRY(launch_defl_project(ctx, n, ctx->eig.prec, ctx->eig.vecs, 64, r, c));
-    TRY(launch_defl_scale(ctx, n, c, eps, 4.0 * ctx->mass * ctx->mass));
+    TRY(launch_defl_project(ctx, n, ctx->eig.prec, ctx->eig.vecs, 64, r, c, eps, 4.0 * ctx->mass * ctx->mass));
     return launch_defl_expand(ctx, n, ctx->eig.prec, ctx->eig.vecs, c, 1.0, 64, x);
 }
 
