@@ -440,14 +440,15 @@ def run_ours(a):
         }
 
     # the FP64 Dslash (reliable-update residuals, source preparation, odd
-    # reconstruction, residual checks) is FP64-ALU bound: 1146 flop per output
-    # site against GB300's nominal 1.25 TFLOP/s FP64 rate
+    # reconstruction, residual checks): 1146 flop per output site beside GB300's
+    # nominal 1.25 TFLOP/s FP64 rate; its sums run in fixed point on the integer
+    # units, so the fraction can exceed 1
     if fp64_n > 0 and fp64_s > 0:
         tf64 = flops_site * Vh * fp64_n / fp64_s / 1e12
         roof["fp64_dslash_kernel"] = {
-            "kernel": "k_dslash FP64 (reliable updates, source preparation, reconstruction, residual checks)",
+            "kernel": "k_dslash_fx FP64 (reliable updates, source preparation, reconstruction, residual checks)",
             "launches": fp64_n, "launch_us": round(fp64_s / fp64_n * 1e6, 2), "achieved_tflops": round(tf64, 3),
-            "peak": 1.25, "peak_source": "nominal GB300 dense FP64 rate", "frac": round(tf64 / 1.25, 4),
+            "peak": 1.25, "peak_source": "nominal GB300 dense FP64 rate (sums in fixed point on the integer units)", "frac": round(tf64 / 1.25, 4),
             "share_of_timed": round(fp64_s * 1e3 / elapsed_ms, 4)}
     rel_name = "FP64 reliable updates" if rel_prec == 64 else "double-float reliable updates, final residual in FP64"
     out = {

@@ -61,8 +61,9 @@ typedef enum {
     HISQ_ERR_STATE = 7          /* call order violated (e.g. solve before links)   */
 } hisq_status;
 
-/* Storage precisions.  Arithmetic is FP64 for HISQ_PREC_DOUBLE, double-float for
- * HISQ_PREC_DF64 and FP32 otherwise. */
+/* Storage precisions.  Arithmetic is FP64 for HISQ_PREC_DOUBLE (the operator's sums in
+ * fixed point: 56-bit mantissas under one exponent per site, rounded once; FP64 FMAs at
+ * sites that format cannot hold), double-float for HISQ_PREC_DF64 and FP32 otherwise. */
 typedef enum {
     HISQ_PREC_DOUBLE = 64,
     HISQ_PREC_SINGLE = 32,
@@ -221,7 +222,8 @@ hisq_status hisq_apply_dslash_batch(hisq_ctx *ctx, int out_parity, int precision
                                     double *out);
 
 /* Launch shape of the batched operator (testing and tuning; kind 0 = autotuned,
- * the default).  kind 1: one site per thread for rhs_per_thread (2..4)
+ * the default: with 16-bit vectors over the shapes of a kernel whose warps share
+ * a shared-memory ring of links, with 32-bit ones also over kind 1).  kind 1: one site per thread for rhs_per_thread (2..4)
  * right-hand sides, links loaded by each thread, with (budget 0) or without
  * (budget 1) an L2 prefetch of the next direction's links; kind 2: the same
  * work split with the links of each site group and direction bulk-copied into
