@@ -427,7 +427,7 @@ def run_ours(a):
             "unit": "TFLOP/s", "frac": None if tf is None else round(tf / peak32, 4),
             "traffic": ncu_traffic(f"mrhs{kps}_oe_s{a.sloppy}_r{a.recon}", Vh),
             "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz (nominal clock)",
-            "kernel": f"k_dslash_mrhs D_oe ({kps} RHS per launch)",
+            "kernel": f"batched D_oe, k_dslash_ring ({kps} RHS per launch)",
             "flops_per_rhs_site": flops_site,
             "launch_us": round(t_all / max(n_launch, 1) * 1e6, 2),
             "mean_rhs_per_launch": round(rhs_launch / max(n_launch, 1), 2),
@@ -674,7 +674,7 @@ def write_traffic(report: str, config: str, key: str, out: str, command: str, mr
     per_site = {}
     for r in data:
         name = r[col["Kernel Name"]]
-        if "k_dslash_mrhs" in name:
+        if "k_dslash_mrhs" in name or "k_dslash_ring" in name:
             kind = "oe" if "BEpiStore" in name else ("eo" if "BEpiCG" in name else None)
             prefix = f"mrhs{mrhs}_"
         else:
