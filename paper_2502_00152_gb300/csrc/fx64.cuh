@@ -385,7 +385,7 @@ __device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const Link
             const int4 *w = reinterpret_cast<const int4 *>(ring + size_t(slot) * kFxHopBytes) + lane;
             if (ok) fx_add(cur, E, acc, [&](int k) { return w[32 * k]; });
             ok = __all_sync(0xffffffffu, ok);
-            if (lane == 0 && ok) tc::mbar_arrive(&empty[slot]);
+            if (ok) tc::ring_release(&empty[slot]);
             if (++slot == stages) {
                 slot = 0;
                 phase ^= 1;

@@ -1135,7 +1135,7 @@ __global__ void __launch_bounds__(MAXT, 1)
                 for (int k = 0; k < 9; k++) mac(k / 3, k % 3, w[32 * (9 + k)]);
             }
             ok = __all_sync(0xffffffffu, ok);
-            if (lane == 0 && ok) tc::mbar_arrive(&empty[slot]);
+            if (ok) tc::ring_release(&empty[slot]);
             if (++slot == stages) {
                 slot = 0;
                 phase ^= 1;
@@ -1326,8 +1326,7 @@ __global__ void __launch_bounds__(256, MINB)
                 }
             }
         }
-        __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&empty[it % stages]);
+        tc::ring_release(&empty[it % stages]);
         if (mu == 3 && valid) {
 #pragma unroll
             for (int u = 0; u < R; u++)
