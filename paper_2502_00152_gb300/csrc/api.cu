@@ -67,6 +67,14 @@ void *dev_alloc(hisq_ctx *c, size_t bytes)
 {
     void *p = nullptr;
     if (bytes == 0) bytes = 16;
+    // cudaMalloc is forbidden while the stream is captured and would invalidate the capture
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (c->stream && cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
+    if (cap != cudaStreamCaptureStatusNone) {
+        c->alloc_in_capture = true; // graph_run reports it
+        set_err(c, HISQ_ERR_STATE, "allocation of %zu bytes while the stream is captured", bytes);
+        return nullptr;
+    }
     if (c->alloc_fail_after == 0) {
         set_err(c, HISQ_ERR_OOM, "allocation of %zu bytes refused (injected failure)", bytes);
         return nullptr;
@@ -102,6 +110,21 @@ void *get_buf(hisq_ctx *c, int id, size_t bytes)
     if (!p) return nullptr;
     c->bufs[id] = p;
     c->buf_cap[id] = bytes;
+    return p;
+}
+
+void *get_optional_buf(hisq_ctx *c, int id, size_t bytes)
+{
+    if (c->buf_cap[id] >= bytes && c->bufs[id]) return c->bufs[id];
+    size_t avail = 0, total = 0;
+    if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (bytes > avail / 8) return nullptr;
+    const std::string err = c->err;
+    void *p = get_buf(c, id, bytes);
+    if (!p) c->err = err;
     return p;
 }
 
@@ -425,6 +448,7 @@ hisq_status hisq_apply_dslash(hisq_ctx *ctx, int out_parity, int precision, int 
         TRY(launch_scatter_parity(ctx, b, 64, out_parity, full));
         return download_full(ctx, full, out);
     }
+    if (precision == 64) fx_reserve(ctx);
     TRY(launch_gather_parity(ctx, full, 1 - out_parity, precision, a));
     TRY(launch_dslash(ctx, out_parity, precision, link_precision, a, b, 0, nullptr, 0, nullptr, 1.0, -1));
     HISQ_CUDA(cudaMemsetAsync(full, 0, size_t(ctx->g.V) * 48, ctx->stream));
@@ -534,6 +558,7 @@ hisq_status hisq_apply_normal_op(hisq_ctx *ctx, int precision, int link_precisio
         TRY(launch_scatter_parity(ctx, b, 64, 0, full));
         return download_full(ctx, full, out);
     }
+    if (precision == 64) fx_reserve(ctx);
     TRY(launch_gather_parity(ctx, full, 0, precision, a));
     TRY(launch_dslash(ctx, 1, precision, lp, a, t, 0, nullptr, 0, nullptr, 1.0, -1));       // t = D_oe a
     TRY(launch_dslash(ctx, 0, precision, lp, t, b, m4, a, 0, nullptr, -1.0, -1));           // b = 4m^2 a - D_eo t

@@ -123,12 +123,16 @@ static FxScratch fx_scratch(hisq_ctx *ctx, int k)
         }
         n = std::min(n, std::max(have, int(std::min(size_t(kFxGroup), avail / 8 / (2 * ms + s64)))));
     }
-    if (n < 2) return f;
+    if (n < 2) {
+        fx_reserve(ctx);
+        return f;
+    }
     const std::string err = ctx->err;
     f.mant = (char *)get_buf(ctx, BUF_FX, 2 * ms * n);
     f.t = f.mant ? (double2 *)get_buf(ctx, BUF_FX_T, s64 * n) : nullptr;
     if (!f.t) {
         ctx->err = err;
+        fx_reserve(ctx); // room for one field at a time is kept, or asked for again
         return FxScratch{};
     }
     f.mant_t = f.mant + ms * n;

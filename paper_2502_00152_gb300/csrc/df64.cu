@@ -214,6 +214,13 @@ hisq_status ensure_df_links(hisq_ctx *ctx)
     return HISQ_OK;
 }
 
+hisq_status ensure_df_fields(hisq_ctx *ctx)
+{
+    const size_t sdf = spinor_bytes(HISQ_PREC_DF64, ctx->g.Vh);
+    if (!get_buf(ctx, BUF_DF_X, sdf) || !get_buf(ctx, BUF_DF_T, sdf)) return HISQ_ERR_OOM;
+    return ensure_df_links(ctx);
+}
+
 hisq_status launch_to_df64(hisq_ctx *ctx, const double *in, void *out)
 {
     return launch_split(ctx, size_t(ctx->g.Vh) * 3, (const double2 *)in, (float4 *)out);

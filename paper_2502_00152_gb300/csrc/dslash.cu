@@ -306,19 +306,19 @@ static hisq_status run_dslash(hisq_ctx *ctx, int par, const Lk &L, const L12T &L
     return HISQ_OK;
 }
 
+void fx_reserve(hisq_ctx *ctx) { get_optional_buf(ctx, BUF_FX, fx_field_bytes(ctx->g.Vh)); }
+
 // FP64: the input field to mantissas, then the fixed-point kernel.  Without room for
-// the mantissas (50 B per site) every site takes the FP64 path.
+// the mantissas (50 B per site, fx_reserve) every site takes the FP64 path; the buffer is
+// never asked for here, since the launches of an iteration are captured.
 template <class Epi>
 static hisq_status run_fx(hisq_ctx *ctx, int par, const SpinorD &in, const Epi &epi, RedArgs ra, int do_red)
 {
     const int Vh = ctx->g.Vh;
-    const std::string err = ctx->err;
-    void *buf = get_buf(ctx, BUF_FX, fx_field_bytes(Vh));
+    void *buf = ctx->buf_cap[BUF_FX] >= fx_field_bytes(Vh) ? ctx->bufs[BUF_FX] : nullptr;
     if (buf) {
         const hisq_status st = launch_fx_split(ctx, in.p, buf);
         if (st != HISQ_OK) return st;
-    } else {
-        ctx->err = err;
     }
     const LinksX L{ctx->links_x[par], ctx->links_xe[par]};
     const FxField f = fx_field(buf, in.p, Vh);

@@ -230,6 +230,7 @@ static hisq_status store_eigvecs(hisq_ctx *ctx, int n, const void *vf32, int pre
     double *td = (double *)get_buf(ctx, BUF_TMPHI, spinor_bytes(64, Vh));
     double *od = (double *)get_buf(ctx, BUF_RHI, spinor_bytes(64, Vh));
     if (!vd || !td || !od) return HISQ_ERR_OOM;
+    if (!eps_given) fx_reserve(ctx);
     std::vector<double> eps(n), res(n, 0.0);
     for (int i = 0; i < n; i++) {
         const void *vi = (const char *)vf32 + sf * i;

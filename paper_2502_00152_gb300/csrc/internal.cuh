@@ -822,6 +822,7 @@ struct hisq_ctx {
 
     // host-side failure injection: allocations left before they fail (-1: off)
     long long alloc_fail_after = -1;
+    bool alloc_in_capture = false; // an allocation was asked for while the stream was captured
     // host-side failure injection: the next tensor-core deflation issues no copy
     // and gives up its waits after a few thousand polls (one-shot)
     bool inject_wait_timeout = false;
@@ -861,6 +862,9 @@ void dev_free(hisq_ctx *c, void *p, size_t bytes);
 hisq_status check_waits(hisq_ctx *c);
 // persistent scratch buffer `id` of at least `bytes` (nullptr + error set on OOM)
 void *get_buf(hisq_ctx *c, int id, size_t bytes);
+// the same for scratch a call can do without: nullptr and no error where it would take more
+// than an eighth of the free device memory (which later, needed buffers may want) or is refused
+void *get_optional_buf(hisq_ctx *c, int id, size_t bytes);
 
 #define HISQ_CUDA(call)                                                                  \
     do {                                                                                 \
@@ -927,6 +931,9 @@ hisq_status graph_run(hisq_ctx *ctx, IterGraphs &G, int slot, long long key, F &
         hisq_status s = body(true);
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(ctx->stream, &g);
+        if (s == HISQ_OK && ctx->alloc_in_capture)
+            s = set_err(ctx, HISQ_ERR_STATE, "an iteration asked for device memory while it was captured");
+        ctx->alloc_in_capture = false;
         if (s != HISQ_OK) {
             if (g) cudaGraphDestroy(g);
             return s;
@@ -1037,6 +1044,11 @@ hisq_status launch_convert(hisq_ctx *ctx, const void *in, int prec_in, void *out
 // FP16 sloppy links, built from the FP32 gathered links on first use (ingest.cu)
 hisq_status ensure_half_links(hisq_ctx *ctx);
 
+// Scratch of the FP64 operator (prec 64), asked for once by each call that applies it,
+// after the buffers it cannot do without and before anything is captured; without it the
+// operator still runs, on FP64 FMAs
+void fx_reserve(hisq_ctx *ctx);
+
 // FP64 operator timing: fold completed event pairs into the sums (all: wait
 // for every pending one); discard: drop them without summing
 void fp64_prof_drain(hisq_ctx *ctx, bool all, bool discard = false);
@@ -1101,6 +1113,7 @@ hisq_status launch_bcg_persistent(hisq_ctx *ctx, int prec, int link_prec, void *
 
 // double-float operator (df64.cu): fields of HISQ_PREC_DF64 storage
 hisq_status ensure_df_links(hisq_ctx *ctx);
+hisq_status ensure_df_fields(hisq_ctx *ctx); // the links and the fields of one residual
 hisq_status launch_to_df64(hisq_ctx *ctx, const double *in, void *out);        // FP64 -> (hi, lo)
 hisq_status launch_dslash_df(hisq_ctx *ctx, int out_parity, const void *in, void *out); // out = D in
 // out (FP64) = a x + b y + c D in (x, y FP64, nullable); |out|^2 -> slot if >= 0

@@ -119,6 +119,20 @@ static hisq_status set_scalars(hisq_ctx *ctx, const HostScalars &h)
     return HISQ_OK;
 }
 
+// sloppy fields of a solve
+struct CgFields {
+    void *x, *r, *p, *tmp;
+};
+static hisq_status cg_fields(hisq_ctx *ctx, const hisq_solve_params *P, CgFields *f)
+{
+    const int Vh = ctx->g.Vh, prec = P->precision_sloppy;
+    f->x = get_buf(ctx, BUF_XSL, spinor_bytes(prec == 64 ? 64 : 32, Vh));
+    f->r = get_buf(ctx, BUF_RSL, spinor_bytes(prec, Vh));
+    f->p = get_buf(ctx, BUF_P, spinor_bytes(prec, Vh));
+    f->tmp = get_buf(ctx, BUF_TMP, spinor_bytes(prec, Vh));
+    return f->x && f->r && f->p && f->tmp ? HISQ_OK : HISQ_ERR_OOM;
+}
+
 // CG with reliable updates and re-deflation on one right-hand side.
 // b, x: FP64 even fields; x holds the initial guess on entry.
 // With double-float reliable updates the FP64 confirmation of a converged
@@ -138,11 +152,10 @@ static hisq_status cg_reliable(hisq_ctx *ctx, const hisq_solve_params *P, const 
     const int xprec = prec == 64 ? 64 : 32;
     double *r_hi = (double *)get_buf(ctx, BUF_RHI, spinor_bytes(64, Vh));
     double *t_hi = (double *)get_buf(ctx, BUF_TMPHI, spinor_bytes(64, Vh));
-    void *x_sl = get_buf(ctx, BUF_XSL, spinor_bytes(xprec, Vh));
-    void *r_sl = get_buf(ctx, BUF_RSL, spinor_bytes(prec, Vh));
-    void *p = get_buf(ctx, BUF_P, spinor_bytes(prec, Vh));
-    void *tmp = get_buf(ctx, BUF_TMP, spinor_bytes(prec, Vh));
-    if (!r_hi || !t_hi || !x_sl || !r_sl || !p || !tmp) return HISQ_ERR_OOM;
+    CgFields f;
+    TRY(cg_fields(ctx, P, &f));
+    void *x_sl = f.x, *r_sl = f.r, *p = f.p, *tmp = f.tmp;
+    if (!r_hi || !t_hi) return HISQ_ERR_OOM;
 
     double rt = rn0; // true residual norm, r_hi holds b - A x
     // double-float reliable updates; a residual that meets the target is
@@ -382,6 +395,13 @@ hisq_status solve_one(hisq_ctx *ctx, const hisq_solve_params *P, const double *e
     double *t_hi = (double *)get_buf(ctx, BUF_TMPHI, spinor_bytes(64, Vh));
     double *psi_o = (double *)get_buf(ctx, BUF_PSI_O, spinor_bytes(64, Vh));
     if (!eta_e || !eta_o || !y || !x || !r_hi || !t_hi || !psi_o) return HISQ_ERR_OOM;
+    CgFields f;
+    TRY(cg_fields(ctx, P, &f));
+    // needed buffers come before the optional scratch of the FP64 operator; without room for
+    // the double-float ones the solve reports it where it first needs them
+    const std::string err = ctx->err;
+    if (P->precision_reliable != HISQ_PREC_DF64 || ensure_df_fields(ctx) == HISQ_OK) fx_reserve(ctx);
+    ctx->err = err;
 
     // (a2) source preparation
     TRY(launch_gather_parity(ctx, eta, 0, 64, eta_e));

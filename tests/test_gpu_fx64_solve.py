@@ -1,0 +1,56 @@
+"""The FP64 operator inside a solve when device memory runs out: its scratch (the mantissas
+of one field, 50 B per site) is asked for once per solve, after the buffers the solve needs
+and never inside the iterations that are captured into a CUDA graph; refused, the whole
+solve runs on FP64 FMAs."""
+import numpy as np
+import pytest
+
+from gpu_common import make
+from paper_2502_00152_gb300 import hisq as H
+from paper_2502_00152_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+DIMS = (6, 4, 6, 8)
+VH = 6 * 4 * 6 * 8 // 2
+
+
+@pytest.mark.parametrize("sloppy,reliable", [(64, 64), (32, 64), (16, 48)])
+def test_solve_without_room_for_the_mantissas(sloppy, reliable):
+    """Allocations are let through one at a time until the solve lacks only its optional
+    scratch.  It then converges past the first captured iterations (the fifth on), and the
+    scratch is what the context still lacked."""
+    m = 0.02
+    ctx, o = make(DIMS, seed=5, eps=0.3, mass=m)
+    try:
+        eta = I.gaussian_source(DIMS, 13, 0)
+        prm = H.hisq_default_solve_params(batch=0, precision_sloppy=sloppy, precision_reliable=reliable)
+
+        def attempt(after):
+            H.hisq_inject_alloc_failure(ctx, after)
+            try:
+                return H.hisq_solve(ctx, eta, prm)
+            except H.HisqError as e:
+                assert e.status == H.HISQ_ERR_OOM, e
+                return None
+            finally:
+                H.hisq_inject_alloc_failure(ctx, -1)
+
+        for _ in range(40):
+            got = attempt(0)
+            if got is not None:
+                break
+            held = H.hisq_device_bytes(ctx)
+            attempt(1)
+            if H.hisq_device_bytes(ctx) == held:
+                attempt(2)  # the double-float links of both parities come together
+        psi, st, status = got
+        assert status == H.HISQ_OK and st[0]["iterations"] > 8
+        assert o.full_residual(m, psi.reshape(-1, 3), eta) <= 1e-10
+        before = H.hisq_device_bytes(ctx)
+        psi2, st2, status = H.hisq_solve(ctx, eta, prm)
+        assert status == H.HISQ_OK and o.full_residual(m, psi2.reshape(-1, 3), eta) <= 1e-10
+        assert 48 * VH <= H.hisq_device_bytes(ctx) - before <= 52 * VH + 512
+        assert np.linalg.norm(psi - psi2) <= 1e-7 * np.linalg.norm(psi)
+    finally:
+        ctx.close()
