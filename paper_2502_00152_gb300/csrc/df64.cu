@@ -233,9 +233,7 @@ static hisq_status run_df(hisq_ctx *ctx, int par, const void *in, const Epi &epi
     const hisq_status s = ensure_df_links(ctx);
     if (s != HISQ_OK) return s;
     auto kern = k_dslash_df<Epi>;
-    static int bps = -1;
-    if (bps < 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, 256, 0) != cudaSuccess || bps < 1))
-        bps = 1;
+    static const int bps = blocks_per_sm(kern, 256);
     const int grid = grid_for(ctx, ctx->g.Vh, 256, bps);
     kern<<<grid, 256, 0, ctx->stream>>>(ctx->g, par, ctx->links_df[par], (const float4 *)in, epi, ra, do_red);
     const cudaError_t e = cudaGetLastError();
@@ -381,9 +379,7 @@ static hisq_status run_df_batch(hisq_ctx *ctx, const DFGroup &grp, const float4 
     const int wpb = std::min(grp.k, kDFWarps);
     const int ny = (grp.k + wpb - 1) / wpb;
     auto go = [&](auto kern, int par, const float4 *in) -> hisq_status {
-        static int bps = -1;
-        if (bps < 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kern, 256, 0) != cudaSuccess || bps < 1))
-            bps = 1;
+        static const int bps = blocks_per_sm(kern, 256);
         // all ny field chunks resident together (blocks of fewer warps fit
         // proportionally more per SM), so that the chunks sweep the sites in
         // step and re-read each link line from L2 rather than DRAM

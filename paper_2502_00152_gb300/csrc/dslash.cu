@@ -206,14 +206,6 @@ __global__ void __launch_bounds__(256, 2)
 }
 
 // ------------------------------------------------------------- launch glue
-template <typename K>
-static int blocks_per_sm(K kernel)
-{
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, 256, 0) != cudaSuccess || n < 1) n = 1;
-    return n;
-}
-
 // ------------------------------------------------- the FP64 kernel
 // Fixed-point sums (fx64.cuh) of FP64 links and one FP64 field, one thread per site, or
 // SPLIT = 4 warps per group of 32 sites, one per direction, whose integer sums are added
@@ -297,8 +289,7 @@ static hisq_status run_dslash(hisq_ctx *ctx, int par, const Lk &L, const L12T &L
                               RedArgs ra, int do_red)
 {
     auto kern = k_dslash<SIn, Lk, L12T, R12, Epi>;
-    static int bps = -1;
-    if (bps < 0) bps = blocks_per_sm(kern);
+    static const int bps = blocks_per_sm(kern, 256);
     const int grid = grid_for(ctx, ctx->g.Vh, 256, bps);
     kern<<<grid, 256, 0, ctx->stream>>>(ctx->g, par, L, L12, float(ctx->long_scale), in, epi, ra, do_red);
     cudaError_t e = cudaGetLastError();
@@ -322,17 +313,18 @@ static hisq_status run_fx(hisq_ctx *ctx, int par, const SpinorD &in, const Epi &
     }
     const LinksX L{ctx->links_x[par], ctx->links_xe[par]};
     const FxField f = fx_field(buf, in.p, Vh);
-    auto launch = [&](auto kern, int sites, int *bps) -> hisq_status {
-        if (*bps < 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, kern, 128, 0) != cudaSuccess || *bps < 1))
-            *bps = 1;
-        const int grid = grid_for(ctx, Vh, sites, *bps);
+    auto launch = [&](auto kern, int sites, int bps) -> hisq_status {
+        const int grid = grid_for(ctx, Vh, sites, bps);
         kern<<<grid, 128, 0, ctx->stream>>>(ctx->g, par, L, f, epi, ra, do_red, buf ? 0 : 1);
         const cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? HISQ_OK : cuda_err(ctx, e, "FP64 dslash launch");
     };
-    static int bps1 = -1, bps4 = -1;
-    if (Vh < ctx->num_sms * 32 * kFxSplitWarps) return launch(k_dslash_fx<Epi, 4>, 32, &bps4);
-    return launch(k_dslash_fx<Epi, 1>, 128, &bps1);
+    if (Vh < ctx->num_sms * 32 * kFxSplitWarps) {
+        static const int bps4 = blocks_per_sm(k_dslash_fx<Epi, 4>, 128);
+        return launch(k_dslash_fx<Epi, 4>, 32, bps4);
+    }
+    static const int bps1 = blocks_per_sm(k_dslash_fx<Epi, 1>, 128);
+    return launch(k_dslash_fx<Epi, 1>, 128, bps1);
 }
 
 // Run the Dslash with output parity `par` on links of precision link_prec

@@ -884,6 +884,19 @@ inline int grid_for(const hisq_ctx *ctx, long n, int threads, int blocks_per_sm)
     return int(want);
 }
 
+// resident blocks of a kernel per SM; callers keep it in a `static const` of their own,
+// which is set once and whole when contexts of several threads meet there
+template <typename K>
+int blocks_per_sm(K kernel, int threads)
+{
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, 0) != cudaSuccess || n < 1) {
+        cudaGetLastError();
+        n = 1;
+    }
+    return n;
+}
+
 // ------------------------------------------------------- CUDA graph replay
 // The launches of one CG iteration are the same every iteration (all scalars
 // live in device memory), so they are captured once into a CUDA graph and
