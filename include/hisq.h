@@ -230,7 +230,8 @@ hisq_status hisq_apply_dslash_batch(hisq_ctx *ctx, int out_parity, int precision
  * a shared-memory ring, `budget` (2..4) blocks per SM (12-real long links only;
  * never chosen by the autotuner, slower on GB300); kind 3: as kind 1 with the
  * right-hand sides in pairs whose colour algebra runs as packed two-wide FP32
- * FMAs (rhs_per_thread 2 or 4).  A shape that does not exist for a batch size
+ * FMAs (rhs_per_thread 2 or 4); kind 4: the kernel of the default, `budget` (1, 2
+ * or 4) blocks per SM (18- or 12-real long links).  A shape that does not exist for a batch size
  * makes the batched calls fail with HISQ_ERR_INVALID_ARG. */
 hisq_status hisq_set_batched_kernel(hisq_ctx *ctx, int kind, int rhs_per_thread, int budget);
 
@@ -357,9 +358,12 @@ hisq_status hisq_inject_alloc_failure(hisq_ctx *ctx, int after);
  * producer that issues no copy and with waits that give up after a few
  * thousand polls, so the MMA warp's wait for its operands runs out while no
  * copy and no MMA is in flight; a persistent batched CG launch runs its grid
- * barriers with a zero time limit.  The call returns HISQ_ERR_TIMEOUT with a
- * message and the context stays usable.  One-shot: the next call runs
- * normally.  on = 0 cancels it. */
+ * barriers with a zero time limit.  With on = 2 it is instead the next kernel
+ * that reads links through a shared-memory ring (the batched operator or the
+ * batched FP64 operator) that gives up at its first wait, and lets its copies in
+ * flight land before it ends.  The call returns HISQ_ERR_TIMEOUT with a message
+ * and the context stays usable.  One-shot: the next call runs normally.  on = 0
+ * cancels it. */
 hisq_status hisq_inject_wait_timeout(hisq_ctx *ctx, int on);
 
 /* Bounds checking (a stand-in for a memory checker): in a library built with

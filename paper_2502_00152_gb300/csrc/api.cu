@@ -6,6 +6,7 @@
 #include <cstring>
 
 #include "internal.cuh"
+#include "tc.cuh"
 
 using namespace hisq;
 
@@ -143,6 +144,13 @@ hisq_status check_waits(hisq_ctx *ctx)
     if (code == 0) return HISQ_OK;
     *ctx->wait_status_h = 0;
     return set_err(ctx, HISQ_ERR_TIMEOUT, "operator: a pipeline wait ran out (code %d)", code);
+}
+
+uint32_t ring_spin_limit(hisq_ctx *ctx)
+{
+    if (ctx->inject_wait_timeout != 2) return tc::kSpinLimit;
+    ctx->inject_wait_timeout = 0;
+    return 0;
 }
 
 // scalar slot readback (synchronises the stream)
@@ -480,10 +488,11 @@ hisq_status hisq_inject_alloc_failure(hisq_ctx *ctx, int after)
 hisq_status hisq_set_batched_kernel(hisq_ctx *ctx, int kind, int rhs_per_thread, int budget)
 {
     if (!ctx) return HISQ_ERR_INVALID_ARG;
-    if (kind < 0 || kind > 3) return set_err(ctx, HISQ_ERR_INVALID_ARG, "kind must be 0, 1, 2 or 3");
+    if (kind < 0 || kind > 4) return set_err(ctx, HISQ_ERR_INVALID_ARG, "kind must be 0, 1, 2, 3 or 4");
     if (kind != 0 && (rhs_per_thread < 2 || rhs_per_thread > 4 || (kind == 3 && rhs_per_thread == 3)))
         return set_err(ctx, HISQ_ERR_INVALID_ARG, "rhs_per_thread must be 2, 3 or 4 (2 or 4 for kind 3)");
-    if (((kind == 1 || kind == 3) && (budget < 0 || budget > 1)) || (kind == 2 && (budget < 2 || budget > 4)))
+    if (((kind == 1 || kind == 3) && (budget < 0 || budget > 1)) || (kind == 2 && (budget < 2 || budget > 4)) ||
+        (kind == 4 && budget != 1 && budget != 2 && budget != 4))
         return set_err(ctx, HISQ_ERR_INVALID_ARG, "budget out of range for this kind");
     ctx->mrhs_force_kind = kind;
     ctx->mrhs_force_R = kind ? rhs_per_thread : 0;
@@ -524,7 +533,7 @@ hisq_status hisq_apply_dslash_batch(hisq_ctx *ctx, int out_parity, int precision
 hisq_status hisq_inject_wait_timeout(hisq_ctx *ctx, int on)
 {
     if (!ctx) return HISQ_ERR_INVALID_ARG;
-    ctx->inject_wait_timeout = on != 0;
+    ctx->inject_wait_timeout = on == 0 ? 0 : (on == 2 ? 2 : 1);
     return HISQ_OK;
 }
 

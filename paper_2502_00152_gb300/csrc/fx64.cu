@@ -128,7 +128,7 @@ hisq_status launch_fx_batch_split(hisq_ctx *ctx, const FxGroup &grp, FxArray in,
 // products per complex one, took 495.
 __global__ void __launch_bounds__(32 * kFxWarps, 2)
     k_dslash_fx_batch(Geom g, int par, LinksX L, FxGroup grp, FxBatch o, size_t ms, FxTile tl, double *partials,
-                      unsigned int *ticket, double *norms, int *status)
+                      unsigned int *ticket, double *norms, int *status, uint32_t spin_limit)
 {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ double sh[kFxWarps];
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2)
     const char *mq = (const char *)o.mant + ms * q;
     const FxField in{(const longlong2 *)mq, (const short *)(mq + size_t(Vh) * 48), nullptr};
     double red = 0;
-    fx_ring_sites(g, par, L, in, tl, blockIdx.x, gridDim.x, dsm, status,
+    fx_ring_sites(g, par, L, in, tl, blockIdx.x, gridDim.x, dsm, status, spin_limit,
                   [&](int cb, const int (&c)[4], int s, int E, int le, const FxAcc &acc) {
                       if (q0 >= grp.k) return;
                       CVec<double> v, t;
@@ -254,7 +254,7 @@ hisq_status launch_fx_batch(hisq_ctx *ctx, int par, const FxGroup &grp, const Fx
     if (st != HISQ_OK) return st;
     kern<<<grid, threads, smem, ctx->stream>>>(ctx->g, par, LinksX{ctx->links_x[par], ctx->links_xe[par]}, grp, b,
                                                fx_field_bytes(Vh), tl, ctx->bpartials, ctx->ticket + 40, ctx->bscal->out,
-                                               ctx->wait_status_d);
+                                               ctx->wait_status_d, ring_spin_limit(ctx));
     const cudaError_t err = cudaGetLastError();
     st = fp64_prof_end(ctx, timed);
     return err == cudaSuccess ? st : cuda_err(ctx, err, "FP64 dslash (batch) launch");

@@ -317,7 +317,7 @@ struct FxTile {
 template <class F>
 __device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const LinksX &L, const FxField &in,
                                               const FxTile &tl, int bx, int nbx, unsigned char *dsm, int *status,
-                                              F &&site)
+                                              uint32_t spin_limit, F &&site)
 {
     const int Vh = g.Vh, stages = tl.stages;
     const int lane = threadIdx.x & 31, chunk = (threadIdx.x >> 5) % tl.nch, sg = (threadIdx.x >> 5) / tl.nch;
@@ -375,13 +375,13 @@ __device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const Link
                 while (ok && issued < nitems && issued < it + j + stages) {
                     if (!tc::mbar_try_wait(&empty[islot], iphase)) {
                         if (issued > it + j) break;
-                        ok = tc::mbar_wait(&empty[islot], iphase, status, tc::TC_TIMEOUT_EMPTY);
+                        ok = tc::mbar_wait(&empty[islot], iphase, status, tc::TC_TIMEOUT_EMPTY, spin_limit);
                         if (!ok) break;
                     }
                     issue();
                 }
             }
-            if (ok) ok = tc::mbar_wait(&full[slot], phase, status, tc::TC_TIMEOUT_FULL);
+            if (ok) ok = tc::mbar_wait(&full[slot], phase, status, tc::TC_TIMEOUT_FULL, spin_limit);
             const int4 *w = reinterpret_cast<const int4 *>(ring + size_t(slot) * kFxHopBytes) + lane;
             if (ok) fx_add(cur, E, acc, [&](int k) { return w[32 * k]; });
             ok = __all_sync(0xffffffffu, ok);

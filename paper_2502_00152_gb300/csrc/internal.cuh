@@ -823,9 +823,11 @@ struct hisq_ctx {
     // host-side failure injection: allocations left before they fail (-1: off)
     long long alloc_fail_after = -1;
     bool alloc_in_capture = false; // an allocation was asked for while the stream was captured
-    // host-side failure injection: the next tensor-core deflation issues no copy
-    // and gives up its waits after a few thousand polls (one-shot)
-    bool inject_wait_timeout = false;
+    // host-side failure injection (one-shot), 1: the next tensor-core deflation issues no
+    // copy and gives up its waits after a few thousand polls, or the next persistent CG
+    // has no time for its barriers; 2: the next kernel with a ring of links gives up at its
+    // first wait, its copies in flight
+    int inject_wait_timeout = 0;
 
     // launch shapes chosen by the autotuner, by problem key
     std::map<unsigned long long, int> tuned;
@@ -860,6 +862,7 @@ hisq_status cuda_err(hisq_ctx *c, cudaError_t e, const char *what);
 void *dev_alloc(hisq_ctx *c, size_t bytes);
 void dev_free(hisq_ctx *c, void *p, size_t bytes);
 hisq_status check_waits(hisq_ctx *c);
+uint32_t ring_spin_limit(hisq_ctx *c); // polls of a wait of a ring kernel about to be launched
 // persistent scratch buffer `id` of at least `bytes` (nullptr + error set on OOM)
 void *get_buf(hisq_ctx *c, int id, size_t bytes);
 // the same for scratch a call can do without: nullptr and no error where it would take more

@@ -961,7 +961,8 @@ struct RingTile {
 template <int R, class S, bool R12, class Epi, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1)
     k_dslash_ring(Geom g, int par, const float4 *__restrict__ fat, const float4 *__restrict__ lng, float c3,
-                  BatchF<S> in, const BatchScalars *scal, RingTile rt, Epi epi, BatchRed br, int *status)
+                  BatchF<S> in, const BatchScalars *scal, RingTile rt, Epi epi, BatchRed br, int *status,
+                  uint32_t spin_limit)
 {
     constexpr int ROWS = R12 ? 15 : 18;
     constexpr int STAGE = ROWS * 512;
@@ -1054,13 +1055,13 @@ __global__ void __launch_bounds__(MAXT, 1)
                 while (ok && issued < nitems && issued < it + mu + stages) {
                     if (!tc::mbar_try_wait(&empty[islot], iphase)) {
                         if (issued > it + mu) break;
-                        ok = tc::mbar_wait(&empty[islot], iphase, status, tc::TC_TIMEOUT_EMPTY);
+                        ok = tc::mbar_wait(&empty[islot], iphase, status, tc::TC_TIMEOUT_EMPTY, spin_limit);
                         if (!ok) break;
                     }
                     issue();
                 }
             }
-            if (ok) ok = tc::mbar_wait(&full[slot], phase, status, tc::TC_TIMEOUT_FULL);
+            if (ok) ok = tc::mbar_wait(&full[slot], phase, status, tc::TC_TIMEOUT_FULL, spin_limit);
             const float4 *w = reinterpret_cast<const float4 *>(ring + size_t(slot) * STAGE) + lane;
             CVec<float> xf[R], xb[R];
             // one link element of both hops on column j into row i of every right-hand side
@@ -1354,7 +1355,7 @@ struct MrhsShape {
     int rc;  // k_dslash_mrhs: 0 with the L2 link prefetch, 1 without; k_dslash_mrhs_tma: blocks per SM
     int tma; // 1: the TMA-fed kernel (FP32 links with 12-real long links only)
     int x2;  // 1: the packed-pair kernel (R even)
-    int ring; // 1: k_dslash_ring (18- or 12-real long links): rc = parts of the right-hand sides
+    int ring; // k_dslash_ring (18- or 12-real long links): blocks per SM (0: not); rc = parts of the right-hand sides
 };
 constexpr int kTmaStages = 4;
 
@@ -1428,7 +1429,7 @@ static int ring_candidates(int kact, MrhsShape *out)
             out[n].tile = MrhsTile{nch, nsg};
             out[n].rc = parts;
             out[n].tma = out[n].x2 = 0;
-            out[n].ring = 1;
+            out[n].ring = blocks;
             n++;
         }
     }
@@ -1587,7 +1588,7 @@ static hisq_status run_mrhs_ring(hisq_ctx *ctx, int par, const BatchF<S> &in, co
         const int gx = std::min(grid_for(ctx, long(Vh), 32 * rt.nsg, bps), std::max(1, ctx->num_sms * bps / sh.rc));
         kern<<<dim3(gx, sh.rc), threads, smem, ctx->stream>>>(ctx->g, par, ctx->links_f[par], ctx->links_f12[par],
                                                              float(ctx->long_scale), in, ctx->bscal, rt, epi, br,
-                                                             ctx->wait_status_d);
+                                                             ctx->wait_status_d, ring_spin_limit(ctx));
         const cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? HISQ_OK : cuda_err(ctx, e, "batched dslash (ring) launch");
     };
@@ -1636,7 +1637,7 @@ static hisq_status mrhs_shape(hisq_ctx *ctx, int kact, int prec, MrhsShape *sh, 
     // flight), the register kernel until it has been timed
     const bool ring = allow_ring && !forced && ctx->long_recon != 8;
     int n = 0;
-    if (ring && prec == 16) {
+    if ((ring && prec == 16) || (ctx->mrhs_force_kind == 4 && ctx->long_recon != 8)) {
         n = ring_candidates(kact, cand);
     } else {
         n = mrhs_candidates(kact, cand, ctx->long_recon == 12, forced);
@@ -1647,7 +1648,8 @@ static hisq_status mrhs_shape(hisq_ctx *ctx, int kact, int prec, MrhsShape *sh, 
         // a launch shape chosen by the caller (hisq_set_batched_kernel)
         for (int i = 0; i < n; i++)
             if (cand[i].tma == (ctx->mrhs_force_kind == 2) && cand[i].x2 == (ctx->mrhs_force_kind == 3) &&
-                cand[i].R == ctx->mrhs_force_R && cand[i].rc == ctx->mrhs_force_budget) {
+                (cand[i].ring > 0) == (ctx->mrhs_force_kind == 4) && cand[i].R == ctx->mrhs_force_R &&
+                (cand[i].ring ? cand[i].ring : cand[i].rc) == ctx->mrhs_force_budget) {
                 *sh = cand[i];
                 return HISQ_OK;
             }
@@ -1808,7 +1810,7 @@ hisq_status launch_bcg_persistent(hisq_ctx *ctx, int prec, int link_prec, void *
                                 },
                                 false);
     if (st != HISQ_OK) return st;
-    if (sh.tma || sh.x2) return set_err(ctx, HISQ_ERR_INVALID_ARG, "persistent batched CG: register-kernel shapes only");
+    if (sh.tma || sh.x2 || sh.ring) return set_err(ctx, HISQ_ERR_INVALID_ARG, "persistent batched CG: register-kernel shapes only");
     const MrhsTile tl = sh.tile;
     const int threads = 32 * tl.nch * tl.nsg;
     const bool r12 = ctx->long_recon == 12;
@@ -1837,8 +1839,8 @@ hisq_status launch_bcg_persistent(hisq_ctx *ctx, int prec, int link_prec, void *
         HISQ_CUDA(cudaMemsetAsync(ns, 0, 2 * sizeof(unsigned long long), ctx->stream));
         // failure injection (tests): a zero wait limit, so every block that waits
         // at the first barrier gives up
-        const bool inject = ctx->inject_wait_timeout;
-        ctx->inject_wait_timeout = false;
+        const bool inject = ctx->inject_wait_timeout == 1;
+        if (inject) ctx->inject_wait_timeout = 0;
         PersistArgs pa{(double *)buf, ctx->ticket + 48, ctx->wait_status_d, lo2, hi2, max_iters, ctx->bmonitor_d,
                        ctx->bmonitor_len, phase_s ? ns : nullptr, done, its_d, inject ? 0ull : kGridWaitNs};
         BatchF<S> P = batchf<S>(p, Vh, prec), T = batchf<S>(tmp, Vh, prec), Rr = batchf<S>(r, Vh, prec);

@@ -656,8 +656,8 @@ hisq_status tc_deflate_batch(hisq_ctx *ctx, int n, int k, double *R, double *X, 
     if (!part || !C) return HISQ_ERR_OOM;
     // failure injection (tests): one call whose producers issue nothing and
     // whose waits give up after a few thousand polls
-    const bool inject = ctx->inject_wait_timeout;
-    ctx->inject_wait_timeout = false;
+    const bool inject = ctx->inject_wait_timeout == 1;
+    if (inject) ctx->inject_wait_timeout = 0;
     const uint32_t lim = inject ? 4096u : tc::kSpinLimit;
     ExpandEpi none{};
     none.spin_limit = lim;

@@ -359,7 +359,8 @@ def hisq_set_batched_kernel(ctx: Context, kind: int = 0, rhs_per_thread: int = 0
     """Launch shape of the batched operator: kind 0 autotuned; 1 register kernel
     with (budget 0) or without (1) the L2 prefetch of the next direction's links;
     2 TMA-fed kernel (budget = blocks per SM, 2..4); 3 packed-pair kernel
-    (rhs_per_thread 2 or 4, budget as kind 1)."""
+    (rhs_per_thread 2 or 4, budget as kind 1); 4 the autotuned default's ring
+    kernel (budget = blocks per SM, 1, 2 or 4)."""
     _check(ctx.handle, load_library().hisq_set_batched_kernel(ctx.handle, kind, rhs_per_thread, budget))
 
 
@@ -375,8 +376,9 @@ def hisq_apply_dslash_batch(ctx: Context, out_parity: int, precision: int, field
 
 def hisq_inject_wait_timeout(ctx: Context, on: bool = True) -> None:
     """Failure injection: the next tensor-core deflation's GEMM issues no copy and
-    its bounded waits give up quickly (HISQ_ERR_TIMEOUT); one-shot."""
-    _check(ctx.handle, load_library().hisq_inject_wait_timeout(ctx.handle, 1 if on else 0))
+    its bounded waits give up quickly (HISQ_ERR_TIMEOUT); with on = 2 the next
+    kernel with a shared-memory ring of links does.  One-shot."""
+    _check(ctx.handle, load_library().hisq_inject_wait_timeout(ctx.handle, int(on)))
 
 
 def hisq_set_profiling(ctx: Context, on: bool = True) -> None:
