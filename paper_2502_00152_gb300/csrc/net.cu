@@ -233,20 +233,13 @@ __global__ void __launch_bounds__(kNetThreads, P == 8 ? 2 : (P == 4 ? 3 : 4))
 // sites at a time: its 144 threads transport one (site, hop) each for every input channel
 // into shared memory, then each accumulates a 4 x 4 tile of (b, (a, h)) over the 48 (site,
 // colour) rows.  With fewer tiles than threads the rows are dealt to groups of threads.
-// The FP32 sum of a group of sites is added to a two-float sum (two-sum), so that the
-// total has the accuracy of an FP64 one; the partial sums of groups and blocks are added
-// in FP64 in a fixed order.  Bound by the FMA pipe and the latency of the transports'
-// loads between two barriers (three blocks per SM at 128 registers; two at 167: 1.77 ms).
-// 16 x 16 channels: 24^3x48 4.35 -> 1.51 ms.
+// The products are summed in FP32 over kWgChain rows by chains of FMAs, the chains over
+// kWgSum rows, and these sums in FP64, as the partial sums of groups and blocks are, in a
+// fixed order.  The FP64 sums of a thread stay in local memory, since their 64 registers
+// would leave an SM two blocks instead of three.
 constexpr int kWgSites = 16, kWgThreads = kWgSites * kNetHops, kWgRows = kWgSites * 3;
+constexpr int kWgChain = 48, kWgSum = 48; // rows of one chain of FMAs, and of one FP32 sum of chains
 constexpr int kWgPitch = kNetMaxC * kNetHops + 4; // floats per row of a plane: 16-byte rows, few conflicts
-
-__device__ __forceinline__ void two_sum(float &hi, float &lo, float x)
-{
-    const float t = __fadd_rn(hi, x), z = __fsub_rn(t, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(x, z)));
-    hi = t;
-}
 
 __global__ void __launch_bounds__(kWgThreads, 3)
     k_net_wgrad(Geom g, const float4 *links0, const float4 *links1, int nk, int cin, int cout,
@@ -261,9 +254,31 @@ __global__ void __launch_bounds__(kWgThreads, 3)
     const int tile = threadIdx.x % ntile, grp = threadIdx.x / ntile;
     const bool on = grp < groups;
     const int ta = tile % nta, tb = tile / nta;
-    float hr[16], hi[16], lr[16], li[16];
+    pairf ar[4][2], ai[4][2]; // FP32 sums [b][pair of (a, h)]
+    double mem[32], *sr = mem; // FP64 sums
+    asm("" : "+l"(sr));        // an address, so that they are not taken into registers
+    double *si = sr + 16;
 #pragma unroll
-    for (int k = 0; k < 16; k++) hr[k] = hi[k] = lr[k] = li[k] = 0.f;
+    for (int k = 0; k < 16; k++) {
+        sr[k] = si[k] = 0;
+        ar[k >> 2][k & 1] = ai[k >> 2][k & 1] = 0;
+    }
+    const int every = kWgSum / ((kWgRows + groups - 1) / groups); // tiles that make one FP32 sum
+    int left = every;
+    auto flush = [&]() {
+#pragma unroll
+        for (int b = 0; b < 4; b++)
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                const float2 r = upk(ar[b][k]), m = upk(ai[b][k]);
+                sr[4 * b + 2 * k] = sr[4 * b + 2 * k] + double(r.x);
+                sr[4 * b + 2 * k + 1] = sr[4 * b + 2 * k + 1] + double(r.y);
+                si[4 * b + 2 * k] = si[4 * b + 2 * k] + double(m.x);
+                si[4 * b + 2 * k + 1] = si[4 * b + 2 * k + 1] + double(m.y);
+                ar[b][k] = ai[b][k] = 0;
+            }
+        left = every;
+    };
     const size_t V3 = size_t(g.V) * 3;
     // the columns past the last (a, h) and the channels past the last b stay zero
     for (int t = threadIdx.x; t < 2 * kWgRows * kWgPitch; t += blockDim.x) st[t] = 0.f;
@@ -307,40 +322,43 @@ __global__ void __launch_bounds__(kWgThreads, 3)
         }
         __syncthreads();
         if (!on) continue;
-        pairf ar[4][2], ai[4][2]; // rows b, pairs of (a, h)
+#pragma unroll 1
+        for (int r0 = grp; r0 < kWgRows; r0 += kWgChain * groups) {
+            pairf cr[4][2], ci[4][2];
 #pragma unroll
-        for (int b = 0; b < 4; b++) ar[b][0] = ar[b][1] = ai[b][0] = ai[b][1] = 0;
+            for (int b = 0; b < 4; b++) cr[b][0] = cr[b][1] = ci[b][0] = ci[b][1] = 0;
+            const int r1 = min(kWgRows, r0 + kWgChain * groups);
 #pragma unroll 2
-        for (int r = grp; r < kWgRows; r += groups) {
-            const ulonglong2 tr = *reinterpret_cast<const ulonglong2 *>(st + r * kWgPitch + 4 * ta);
-            const ulonglong2 ti = *reinterpret_cast<const ulonglong2 *>(st + (kWgRows + r) * kWgPitch + 4 * ta);
-            const float4 *gp = reinterpret_cast<const float4 *>(sg + r * kNetMaxC + 4 * tb);
-            const float4 g0 = gp[0], g1 = gp[1];
-            const float gr[4] = {g0.x, g0.z, g1.x, g1.z}, gi[4] = {g0.y, g0.w, g1.y, g1.w};
+            for (int r = r0; r < r1; r += groups) {
+                const ulonglong2 tr = *reinterpret_cast<const ulonglong2 *>(st + r * kWgPitch + 4 * ta);
+                const ulonglong2 ti = *reinterpret_cast<const ulonglong2 *>(st + (kWgRows + r) * kWgPitch + 4 * ta);
+                const float4 *gp = reinterpret_cast<const float4 *>(sg + r * kNetMaxC + 4 * tb);
+                const float4 g0 = gp[0], g1 = gp[1];
+                const float gr[4] = {g0.x, g0.z, g1.x, g1.z}, gi[4] = {g0.y, g0.w, g1.y, g1.w};
 #pragma unroll
-            for (int b = 0; b < 4; b++) { // g conj(t)
-                const pairf pr = pk(gr[b], gr[b]), pi = pk(gi[b], gi[b]), pn = pk(-gr[b], -gr[b]);
-                pfma(ar[b][0], pi, ti.x);
-                pfma(ar[b][1], pi, ti.y);
-                pfma(ai[b][0], pn, ti.x);
-                pfma(ai[b][1], pn, ti.y);
-                pfma(ar[b][0], pr, tr.x);
-                pfma(ar[b][1], pr, tr.y);
-                pfma(ai[b][0], pi, tr.x);
-                pfma(ai[b][1], pi, tr.y);
+                for (int b = 0; b < 4; b++) { // g conj(t)
+                    const pairf pr = pk(gr[b], gr[b]), pi = pk(gi[b], gi[b]), pn = pk(-gr[b], -gr[b]);
+                    pfma(cr[b][0], pi, ti.x);
+                    pfma(cr[b][1], pi, ti.y);
+                    pfma(ci[b][0], pn, ti.x);
+                    pfma(ci[b][1], pn, ti.y);
+                    pfma(cr[b][0], pr, tr.x);
+                    pfma(cr[b][1], pr, tr.y);
+                    pfma(ci[b][0], pi, tr.x);
+                    pfma(ci[b][1], pi, tr.y);
+                }
             }
+#pragma unroll
+            for (int b = 0; b < 4; b++)
+#pragma unroll
+                for (int k = 0; k < 2; k++) {
+                    ar[b][k] = padd(ar[b][k], cr[b][k]);
+                    ai[b][k] = padd(ai[b][k], ci[b][k]);
+                }
         }
-#pragma unroll
-        for (int b = 0; b < 4; b++)
-#pragma unroll
-            for (int k = 0; k < 2; k++) {
-                const float2 r = upk(ar[b][k]), m = upk(ai[b][k]);
-                two_sum(hr[4 * b + 2 * k], lr[4 * b + 2 * k], r.x);
-                two_sum(hr[4 * b + 2 * k + 1], lr[4 * b + 2 * k + 1], r.y);
-                two_sum(hi[4 * b + 2 * k], li[4 * b + 2 * k], m.x);
-                two_sum(hi[4 * b + 2 * k + 1], li[4 * b + 2 * k + 1], m.y);
-            }
+        if (--left == 0) flush();
     }
+    flush();
     // the groups' sums through shared memory, in group order
     double2 *sd = reinterpret_cast<double2 *>(dsm4); // [group][tile][16]
     __syncthreads();
@@ -348,7 +366,7 @@ __global__ void __launch_bounds__(kWgThreads, 3)
 #pragma unroll
         for (int k = 0; k < 16; k++)
             sd[(size_t(grp - 1) * ntile + tile) * 16 + k] =
-                make_double2(double(hr[k]) + double(lr[k]), double(hi[k]) + double(li[k]));
+                make_double2(sr[k], si[k]);
     }
     __syncthreads();
     if (!on || grp > 0) return;
@@ -359,7 +377,7 @@ __global__ void __launch_bounds__(kWgThreads, 3)
         for (int a = 0; a < 4; a++) {
             const int bb = 4 * tb + b, aa = 4 * ta + a, k = 4 * b + a;
             if (bb >= cout || aa >= nah) continue;
-            double2 t = make_double2(double(hr[k]) + double(lr[k]), double(hi[k]) + double(li[k]));
+            double2 t = make_double2(sr[k], si[k]);
             for (int w = 1; w < groups; w++) {
                 const double2 o = sd[(size_t(w - 1) * ntile + tile) * 16 + k];
                 t.x += o.x;
