@@ -235,10 +235,15 @@ __global__ void __launch_bounds__(kNetThreads, P == 8 ? 2 : (P == 4 ? 3 : 4))
 // colour) rows.  With fewer tiles than threads the rows are dealt to groups of threads.
 // The products are summed in FP32 over kWgChain rows by chains of FMAs, the chains over
 // kWgSum rows, and these sums in FP64, as the partial sums of groups and blocks are, in a
-// fixed order.  The FP64 sums of a thread stay in local memory, since their 64 registers
-// would leave an SM two blocks instead of three.
+// fixed order.  Rounding, 16 x 16 channels, relative to the sums: 1.29e-7 with chains of 16
+// rows; 1.8e-7 with one of all 48 (two roundings a product); 1.44e-7 with each product
+// formed first, at half as many FP32 operations again.
+// Bound by the FMA pipe and the latency of the transports' loads between two barriers, at
+// three blocks per SM.  The FP64 sums of a thread stay in local memory, touched every
+// fourth tile: in 64 registers they left an SM two blocks.  16 x 16 channels: 24^3x48 4.35
+// -> 1.59 ms (FP64 sums after every tile 1.64, in registers 1.89), 16^3x32 0.33 ms.
 constexpr int kWgSites = 16, kWgThreads = kWgSites * kNetHops, kWgRows = kWgSites * 3;
-constexpr int kWgChain = 48, kWgSum = 48; // rows of one chain of FMAs, and of one FP32 sum of chains
+constexpr int kWgChain = 16, kWgSum = 192; // rows of one chain of FMAs, and of one FP32 sum of chains
 constexpr int kWgPitch = kNetMaxC * kNetHops + 4; // floats per row of a plane: 16-byte rows, few conflicts
 
 __global__ void __launch_bounds__(kWgThreads, 3)
