@@ -168,7 +168,7 @@ __global__ void k_split_df(size_t n, const double2 *__restrict__ in, float4 *__r
     }
 }
 
-// the double-float split of the gathered FP64 links (mantissas, fx64.cuh)
+// the double-float split of the gathered FP64 links (fx64.cuh)
 __global__ void k_split_df_links(int Vh, const int4 *__restrict__ w, const short *__restrict__ e,
                                  float4 *__restrict__ out)
 {

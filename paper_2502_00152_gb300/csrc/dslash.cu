@@ -213,9 +213,10 @@ __global__ void __launch_bounds__(256, 2)
 //
 // Bound by the 2304 B of links per site.  Each thread holds the links and the neighbour
 // of two hops (100 registers), so that a warp has 6.5 KB of loads in flight while it
-// multiplies.  32^3x64, split of the input included: 417 us per application at 168
-// registers (12 warps per SM), 500 at 128 (432 B spilled), 513 with the links in shared
-// memory as the batch has them; FP64 FMAs took 1040.
+// multiplies.  32^3x64, split of the input included: 439 us per application at 168
+// registers (12 warps per SM); FP64 FMAs took 1040.  With links cut to 56-bit limbs
+// beforehand, which saves the shift of each real but loses bits of the small ones: 417, at
+// 128 registers (432 B spilled) 500, with the links in shared memory as the batch has them 513.
 //
 // Split where one thread per site leaves fewer than 16 warps per SM: 8^4 16 us per
 // application instead of 23, 14x10x12x22 24 instead of 27, 16^3x32 even; on 24^3x48 (68

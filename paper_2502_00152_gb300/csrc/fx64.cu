@@ -37,37 +37,33 @@ hisq_status launch_fx_split(hisq_ctx *ctx, const void *in, void *out)
     return err == cudaSuccess ? HISQ_OK : cuda_err(ctx, err, "fixed-point split");
 }
 
-// The gathered FP64 links of one parity to mantissas, in place: each thread owns the
-// 144 elements of its site.  Zero matrices keep an ordinary exponent; sites whose
-// largest entry lies outside 2^+-100 stay FP64 and are marked.
+// The gathered FP64 links of one parity to the operator's form, in place: each thread owns
+// the 144 elements of its site.  Zero matrices get an ordinary exponent; sites whose
+// largest entry lies outside 2^+-100, or that have one more than 127 binary places below
+// it, stay FP64 and are marked.
 __global__ void __launch_bounds__(256) k_links_fx(int Vh, int4 *w, short *e)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Vh; i += gridDim.x * blockDim.x) {
         int4 *p = w + fx_link_index(i, 0);
-        int eb = 0;
+        int eb = 0, low = 0x7ff; // exponents of the largest and of the smallest entry that is not zero
         for (int k = 0; k < 144; k++) {
             const int4 q = p[32 * k];
-            eb = max(eb, max((q.y >> 20) & 0x7ff, (q.w >> 20) & 0x7ff));
+            for (const double x : {__hiloint2double(q.y, q.x), __hiloint2double(q.w, q.z)}) {
+                const int ex = fx_exponent(x);
+                eb = max(eb, ex);
+                if (x != 0.0) low = min(low, ex);
+            }
         }
-        if (eb < kFxLinkLo || eb > kFxLinkHi) {
-            bool zero = eb == 0;
-            for (int k = 0; k < 144 && zero; k++) {
-                const int4 q = p[32 * k];
-                zero = ((q.y | q.w) & 0x7fffffff) == 0 && (q.x | q.z) == 0;
-            }
-            if (!zero) {
-                e[i] = short(kFxMark);
-                continue;
-            }
-            eb = 1022;
+        if (low == 0x7ff && eb == 0) eb = low = 1022; // all zero
+        if (eb < kFxLinkLo || eb > kFxLinkHi || eb - low > kFxDepth) {
+            e[i] = short(kFxMark);
+            continue;
         }
         e[i] = short(eb);
         for (int k = 0; k < 144; k++) {
             const int4 q = p[32 * k];
-            int4 o;
-            fx_limbs(fx_mantissa<3>(__hiloint2double(q.y, q.x), eb), o.x, o.y);
-            fx_limbs(fx_mantissa<3>(__hiloint2double(q.w, q.z), eb), o.z, o.w);
-            p[32 * k] = o;
+            const long long re = fx_encode(__hiloint2double(q.y, q.x), eb), im = fx_encode(__hiloint2double(q.w, q.z), eb);
+            p[32 * k] = make_int4(int(re), int(re >> 32), int(im), int(im >> 32));
         }
     }
 }
@@ -123,9 +119,10 @@ hisq_status launch_fx_batch_split(hisq_ctx *ctx, const FxGroup &grp, FxArray in,
 
 // The operator for a group of fields (fx_ring_sites), blockIdx.y: fields blockIdx.y * nch ...
 // Bound by instruction issue and the multiply-add pipe together (54 % busy at 12 warps):
-// 32^3x64, per field and application: 330 us for 8 fields, 342 for 12, 352 for 2 (16 warps
-// per SM), one field at a time 417, FP64 FMAs 1040.  Two fields per thread, with four real
-// products per complex one, took 495.
+// 32^3x64, per field and application, splits included: 377 us for 12 or 5 fields, one field
+// at a time 439, FP64 FMAs 1040.  With links cut to 56-bit limbs beforehand (bits of the
+// small ones lost) 351 and 340; two fields per thread, with four real products per complex
+// one, took 495.
 __global__ void __launch_bounds__(32 * kFxWarps, 2)
     k_dslash_fx_batch(Geom g, int par, LinksX L, FxGroup grp, FxBatch o, size_t ms, FxTile tl, double *partials,
                       unsigned int *ticket, double *norms, int *status, uint32_t spin_limit)

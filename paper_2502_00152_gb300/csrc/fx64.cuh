@@ -12,9 +12,11 @@
 //
 // Block floating point: the six reals of a colour vector share the exponent of the
 // largest one, the 288 link reals of an output site share theirs, and at an output
-// site the 16 neighbour vectors are aligned to the largest of their exponents.  A
-// mantissa keeps 56 bits below the shared exponent (FP64 keeps 53 below its own), and
-// the integer sums are exact.  Measured against 113-bit sums on 8^4: relative error
+// site the 16 neighbour vectors are aligned to the largest of their exponents.  In the sums
+// a mantissa has 56 bits below the shared exponent (FP64 keeps 53 below its own), and
+// the integer sums are exact.  So an error is at most 2.3 x 96 x 2^-56 of the product of
+// the two shared powers of two: small against the site's result, but not against a component
+// that only small entries couple to.  Measured against 113-bit sums on 8^4: relative error
 // 6.4e-17 for a Gaussian field (FP64 FMAs 3.5e-16), 1.0e-16 where site vectors differ by
 // up to e^20 (3.5e-16).  The sums do not depend on the order of the terms, so a site may be
 // split over threads without changing a bit of the result.
@@ -26,7 +28,10 @@
 // hi = the upper word plus the sign bit of the lower, lo = the lower word >> 4.
 //
 // Links are stored by groups of 32 sites, [group][mu][kind][fwd,bwd][k][32] int4: the
-// 144 loads of a thread are at constant offsets from one address.
+// 144 loads of a thread are at constant offsets from one address.  A real keeps its own 53
+// bits: its signed mantissa times 2^7 in 64 bits, with the number of places it lies below
+// the site's exponent in the seven low ones, so that one shift aligns it (links of the
+// solves, of FP64 FMAs and of the double-float operator are the same values).
 //
 // Values the block format cannot hold -- Inf, NaN, and exponents so far out that a
 // product's scale would leave the FP64 range -- are marked, and a site that meets a
@@ -51,9 +56,9 @@ struct FxField {
     const double2 *src;
 };
 
-// gathered links of one output parity: int4 =
-// (re hi, re lo, im hi, im lo) per element, biased exponents [Vh]; where the exponent
-// is kFxMark the int4 holds the two FP64 values themselves
+// gathered links of one output parity: int4 = (re low, re high, im low, im high) words of an
+// element (fx_encode), biased exponents [Vh]; where the exponent is kFxMark they hold the
+// two FP64 values themselves
 struct LinksX {
     const int4 *w; // fx_link_index
     const short *e;
@@ -72,15 +77,14 @@ inline FxField fx_field(void *buf, const void *src, int Vh)
 
 __device__ __forceinline__ int fx_exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
-// round(x 2^(53 + UP - (eb - 1022))) for |x| < 2^(eb - 1022)
-template <int UP>
+// round(x 2^(60 - (eb - 1022))) for |x| < 2^(eb - 1022)
 __device__ __forceinline__ long long fx_mantissa(double x, int eb)
 {
     const long long b = __double_as_longlong(x);
     const int e = int(b >> 52) & 0x7ff;
     const int s = eb - (e > 0 ? e : 1);
     unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (e > 0 ? 1ull << 52 : 0ull);
-    m <<= UP;
+    m <<= 7;
     if (s > 0) m = s < 62 ? (m + (1ull << (s - 1))) >> s : 0ull;
     return b < 0 ? -(long long)m : (long long)m;
 }
@@ -103,14 +107,39 @@ __device__ __forceinline__ void fx_store_site(longlong2 *v, short *e, int Vh, in
     e[i] = short(eb);
 #pragma unroll
     for (int c = 0; c < 3; c++)
-        v[size_t(c) * Vh + i] = make_longlong2(fx_mantissa<7>(q.re[c], eb), fx_mantissa<7>(q.im[c], eb));
+        v[size_t(c) * Vh + i] = make_longlong2(fx_mantissa(q.re[c], eb), fx_mantissa(q.im[c], eb));
 }
 
-// limbs of a mantissa, |v| <= 2^56
-__device__ __forceinline__ void fx_limbs(long long v, int &hi, int &lo)
+// a link real under exponent eb: signed mantissa (53 bits) 2^7, and in the low seven bits
+// how far its own exponent lies below eb (at most kFxDepth); zero: 0
+constexpr int kFxDepth = 127;
+__device__ __forceinline__ long long fx_encode(double x, int eb)
 {
-    hi = int((v + (1ll << 27)) >> 28);
-    lo = int(unsigned(v) - (unsigned(hi) << 28));
+    if (x == 0.0) return 0;
+    const long long b = __double_as_longlong(x);
+    const long long m = ((b & 0xfffffffffffffll) | (1ll << 52)) << 7;
+    return (b < 0 ? -m : m) | (eb - fx_exponent(x));
+}
+__device__ __forceinline__ double fx_decode(int w0, int w1, int eb)
+{
+    const unsigned long long u = ((unsigned long long)(unsigned)w1 << 32) | unsigned(w0 & ~kFxDepth);
+    if (u == 0) return 0.0;
+    const unsigned long long m = (w1 < 0 ? 0ull - u : u) >> 7;
+    const unsigned long long e = (unsigned long long)(eb - (w0 & kFxDepth)) << 52;
+    return __longlong_as_double((long long)((m & 0xfffffffffffffull) | e | (w1 < 0 ? 1ull << 63 : 0ull)));
+}
+
+// limbs of an encoded link real shifted down to its site's exponent, |v| <= 2^60.  Below a
+// shift of 16 the count takes bits that the low limb drops, from 16 on it is shifted out.
+__device__ __forceinline__ void fx_link_limbs(int w0, int w1, int &hi, int &lo)
+{
+    long long v;
+    asm("{\n\t.reg .s64 t;\n\tmov.b64 t, {%1, %2};\n\tshr.s64 %0, t, %3;\n\t}"
+        : "=l"(v)
+        : "r"(w0), "r"(w1), "r"(w0 & kFxDepth)); // a shift past 63 places leaves the sign
+    const unsigned l = unsigned(v);
+    hi = int(v >> 32) + int(l >> 31);
+    lo = int(l) >> 4;
 }
 
 // limbs of a vector mantissa shifted down by d (0..31), |v| <= 2^60: two shifts, one
@@ -129,8 +158,7 @@ __device__ __forceinline__ double fx_pow2(int k) { return __hiloint2double((k + 
 __device__ __forceinline__ double2 fx_link(int4 q, int eb)
 {
     if (eb == kFxMark) return make_double2(__hiloint2double(q.y, q.x), __hiloint2double(q.w, q.z));
-    const double s1 = fx_pow2(eb - 1022 - 28), s0 = fx_pow2(eb - 1022 - 56);
-    return make_double2(fma(double(q.x), s1, double(q.y) * s0), fma(double(q.z), s1, double(q.w) * s0));
+    return make_double2(fx_decode(q.x, q.y, eb), fx_decode(q.z, q.w, eb));
 }
 
 // Sums of the integer products of one right-hand side.  With W = a + ib and v = c + id,
@@ -202,7 +230,11 @@ __device__ __forceinline__ void fx_add(const FxVec &x, int E, FxAcc &acc, F &&li
 #pragma unroll
         for (int j = 0; j < 3; j++) {
             const int4 w = link(3 * i + j);
-            const int wh[3] = {w.x + w.z, w.x, w.z}, wl[3] = {w.y + w.w, w.y, w.w};
+            int wh[3], wl[3]; // limbs of a + b, a, b
+            fx_link_limbs(w.x, w.y, wh[1], wl[1]);
+            fx_link_limbs(w.z, w.w, wh[2], wl[2]);
+            wh[0] = wh[1] + wh[2];
+            wl[0] = wl[1] + wl[2];
             // three independent sums between two additions to the same one
 #pragma unroll
             for (int k = 0; k < 3; k++) acc.h[i][k] += (long long)wh[k] * vh[j][k];

@@ -7,7 +7,7 @@
 //   bwd, n hops:  W = -eta_mu(x) * bc(x - n mu, n) * U_mu(x - n mu)^dag
 // with bc = -1 for a hop that wraps the time boundary of an antiperiodic
 // lattice.  They are written in FP64 (then turned into the fixed-point operator's
-// mantissas in place, fx64.cuh) and FP32 (see internal.cuh for layouts).
+// form in place, fx64.cuh) and FP32 (see internal.cuh for layouts).
 // With 12-real long links only rows 0 and 1 of S = U_long / long_scale are kept
 // (for fwd and bwd); the Dslash rebuilds row 2 and applies the sign and scale.
 #include "fx64.cuh"

@@ -447,7 +447,7 @@ __device__ __forceinline__ CVec<To> cvt(const CVec<From> &v)
 // (kind 0: fat, n = 1; kind 1: long, n = 3).
 //
 // FP64 (recon 18): [p][group of 32 sites][mu][kind][fwd,bwd][k=0..8][32], 16 B per complex
-//   element: 56-bit mantissas under one exponent per output site (fx64.cuh)
+//   element: 53-bit mantissas with their places below one exponent per output site (fx64.cuh)
 // The FP32 and FP16 arrays are stored by groups of 32 output sites, rows x 32 sites each
 // (link_index):
 // FP32 (recon 18): float4, row (mu * 2 + kind) * 9 + k; float4 = (Re fwd, Re bwd, Im fwd,
@@ -788,7 +788,7 @@ struct hisq_ctx {
     double long_scale = 1.0;
 
     // gathered links; index [parity]
-    int4 *links_x[2] = {nullptr, nullptr};     // FP64, 16 hops: mantissas as two limbs (fx64.cuh)
+    int4 *links_x[2] = {nullptr, nullptr};     // FP64, 16 hops (fx_encode, fx64.cuh)
     short *links_xe[2] = {nullptr, nullptr};   // their exponents, one per output site
     float4 *links_f[2] = {nullptr, nullptr};   // FP32: fat (+ long when recon 18)
     float4 *links_f12[2] = {nullptr, nullptr}; // FP32 long, recon 12
@@ -1138,7 +1138,7 @@ hisq_status launch_dslash_df_xpay(hisq_ctx *ctx, int out_parity, const void *in,
 // r = b - (4m^2 - D_eo D_oe) x on even fields, |r|^2 -> slot
 hisq_status launch_residual_df(hisq_ctx *ctx, const double *b, const double *x, double *r, int slot);
 
-// the gathered FP64 links of one parity to the operator's mantissas, in place (fx64.cu)
+// the gathered FP64 links of one parity to the operator's form, in place (fx64.cu)
 hisq_status launch_links_fx(hisq_ctx *ctx, int par);
 
 // link ingest (ingest.cu)
