@@ -456,9 +456,8 @@ hisq_status hisq_apply_dslash(hisq_ctx *ctx, int out_parity, int precision, int 
         TRY(launch_scatter_parity(ctx, b, 64, out_parity, full));
         return download_full(ctx, full, out);
     }
-    if (precision == 64) fx_reserve(ctx);
     TRY(launch_gather_parity(ctx, full, 1 - out_parity, precision, a));
-    TRY(launch_dslash(ctx, out_parity, precision, link_precision, a, b, 0, nullptr, 0, nullptr, 1.0, -1));
+    TRY(launch_dslash(ctx, out_parity, precision, link_precision, a, b, 0, nullptr, 0, nullptr, 1.0, -1, true));
     HISQ_CUDA(cudaMemsetAsync(full, 0, size_t(ctx->g.V) * 48, ctx->stream));
     TRY(launch_scatter_parity(ctx, b, precision, out_parity, full));
     return download_full(ctx, full, out);
@@ -567,10 +566,9 @@ hisq_status hisq_apply_normal_op(hisq_ctx *ctx, int precision, int link_precisio
         TRY(launch_scatter_parity(ctx, b, 64, 0, full));
         return download_full(ctx, full, out);
     }
-    if (precision == 64) fx_reserve(ctx);
     TRY(launch_gather_parity(ctx, full, 0, precision, a));
-    TRY(launch_dslash(ctx, 1, precision, lp, a, t, 0, nullptr, 0, nullptr, 1.0, -1));       // t = D_oe a
-    TRY(launch_dslash(ctx, 0, precision, lp, t, b, m4, a, 0, nullptr, -1.0, -1));           // b = 4m^2 a - D_eo t
+    TRY(launch_dslash(ctx, 1, precision, lp, a, t, 0, nullptr, 0, nullptr, 1.0, -1, true)); // t = D_oe a
+    TRY(launch_dslash(ctx, 0, precision, lp, t, b, m4, a, 0, nullptr, -1.0, -1, true));     // b = 4m^2 a - D_eo t
     HISQ_CUDA(cudaMemsetAsync(full, 0, size_t(ctx->g.V) * 48, ctx->stream));
     TRY(launch_scatter_parity(ctx, b, precision, 0, full));
     return download_full(ctx, full, out);

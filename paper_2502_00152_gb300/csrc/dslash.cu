@@ -148,14 +148,33 @@ struct LinksH12 {
     }
 };
 
+// FP64 for the FP64-FMA form of the operator
+struct LinksXv {
+    LinksX L;
+    typedef double real;
+    __device__ __forceinline__ void load(int mu, int kind, int i, CMat<double> &f, CMat<double> &b) const
+    {
+        const int4 *q = L.w + fx_link_index(i, (mu * 2 + kind) * 18);
+        const int eb = L.e[i];
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            const double2 x = fx_link(__ldcs(q + 32 * k), eb), y = fx_link(__ldcs(q + 32 * (9 + k)), eb);
+            f.re[k] = x.x;
+            f.im[k] = x.y;
+            b.re[k] = y.x;
+            b.im[k] = y.y;
+        }
+    }
+};
+
 // ------------------------------------------------------------- the kernel
 // At most 128 registers, two blocks per SM: the compiler then keeps enough link loads in
 // flight (left to itself it chose 80 to 92 registers and three blocks).  32^3x64, D_oe and
 // fused update, FP16 vectors and 12-real long links: 161 / 170 us, 171 / 172 without the
 // bound; FP32 vectors, 18-real: 192 / 206 us, 202 / 222 without; three blocks 164 / 173
-// and 194 / 208.
+// and 194 / 208.  FP64 sums (bound by the FP64 pipe) take what registers they need.
 template <class SIn, class Lk, class L12T, bool R12, class Epi>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, sizeof(typename Lk::real) == 8 ? 1 : 2)
     k_dslash(Geom g, int par, Lk L, L12T L12, float c3, SIn in, Epi epi, RedArgs ra, int do_red)
 {
     typedef typename Lk::real R;
@@ -329,8 +348,8 @@ static hisq_status run_fx(hisq_ctx *ctx, int par, const SpinorD &in, const Epi &
 }
 
 // Run the Dslash with output parity `par` on links of precision link_prec
-// (64, 32 or 16) in the context's long-link format.
-template <class S, class Epi>
+// (64, 32 or 16) in the context's long-link format; FMA64: FP64 on FP64 FMAs.
+template <bool FMA64 = false, class S, class Epi>
 static hisq_status run_any(hisq_ctx *ctx, int par, int link_prec, const S &in, const Epi &epi, RedArgs ra, int dored)
 {
     typedef typename S::real R;
@@ -338,7 +357,10 @@ static hisq_status run_any(hisq_ctx *ctx, int par, int link_prec, const S &in, c
     const bool r12 = ctx->long_recon == 12, r8 = ctx->long_recon == 8;
     const int nk = (r12 || r8) ? 1 : 2;
     if (link_prec == 64) {
-        if constexpr (sizeof(R) == 8) return run_fx(ctx, par, in, epi, ra, dored);
+        if constexpr (sizeof(R) == 8 && !FMA64) return run_fx(ctx, par, in, epi, ra, dored);
+        if constexpr (sizeof(R) == 8 && FMA64)
+            return run_dslash<S, LinksXv, LinksF12, false>(ctx, par, LinksXv{{ctx->links_x[par], ctx->links_xe[par]}},
+                                                           LinksF12{nullptr, Vh}, in, epi, ra, dored);
         return set_err(ctx, HISQ_ERR_INVALID_ARG, "FP64 links need FP64 vectors");
     }
     if constexpr (sizeof(R) == 4) {
@@ -386,20 +408,20 @@ void fp64_prof_drain(hisq_ctx *ctx, bool all, bool discard)
 }
 
 static hisq_status dslash_xpay(hisq_ctx *ctx, int out_parity, int prec, int link_prec, const void *in, void *out,
-                               double a, const void *x, double b, const void *y, double c, int norm_slot);
+                               double a, const void *x, double b, const void *y, double c, int norm_slot, bool fma64);
 
 // With profiling on, an FP64 launch outside stream capture is bracketed by a
 // pair of events (from a pool); the pairs are summed once they have completed,
 // so the host never waits for a launch it has just issued.
 hisq_status launch_dslash(hisq_ctx *ctx, int out_parity, int prec, int link_prec, const void *in, void *out, double a,
-                          const void *x, double b, const void *y, double c, int norm_slot)
+                          const void *x, double b, const void *y, double c, int norm_slot, bool fma64)
 {
     bool timed = false;
     if (prec == 64) {
         const hisq_status b0 = fp64_prof_begin(ctx, 1, &timed);
         if (b0 != HISQ_OK) return b0;
     }
-    const hisq_status st = dslash_xpay(ctx, out_parity, prec, link_prec, in, out, a, x, b, y, c, norm_slot);
+    const hisq_status st = dslash_xpay(ctx, out_parity, prec, link_prec, in, out, a, x, b, y, c, norm_slot, fma64);
     const hisq_status e0 = fp64_prof_end(ctx, timed);
     return st != HISQ_OK ? st : e0;
 }
@@ -434,7 +456,7 @@ hisq_status fp64_prof_end(hisq_ctx *ctx, bool on)
 }
 
 static hisq_status dslash_xpay(hisq_ctx *ctx, int out_parity, int prec, int link_prec, const void *in, void *out,
-                               double a, const void *x, double b, const void *y, double c, int norm_slot)
+                               double a, const void *x, double b, const void *y, double c, int norm_slot, bool fma64)
 {
     const int Vh = ctx->g.Vh;
     if (!ctx->links_loaded) return set_err(ctx, HISQ_ERR_STATE, "links not loaded");
@@ -446,6 +468,7 @@ static hisq_status dslash_xpay(hisq_ctx *ctx, int out_parity, int prec, int link
         typedef decltype(in_) S;
         typedef typename S::real R;
         EpiXpay<S> epi{out_, x_, y_, R(a), R(b), R(c), x != nullptr, y != nullptr, dored};
+        if (fma64) return run_any<true>(ctx, out_parity, link_prec, in_, epi, ra, dored);
         return run_any(ctx, out_parity, link_prec, in_, epi, ra, dored);
     };
     void *ii = const_cast<void *>(in);

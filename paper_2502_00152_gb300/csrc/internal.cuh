@@ -1057,6 +1057,7 @@ hisq_status launch_convert(hisq_ctx *ctx, const void *in, int prec_in, void *out
 // out = a*x + b*y + c*D(in)  on output parity `out_parity`; x, y nullable,
 // all of precision `prec`, links of precision link_prec (64 or 32).
 // If norm_slot >= 0 the squared norm of out is reduced into scal->slot[norm_slot].
+// Precision 64: fixed-point sums (fx64.cuh), or FP64 FMAs with fma64.
 // FP16 sloppy links, built from the FP32 gathered links on first use (ingest.cu)
 hisq_status ensure_half_links(hisq_ctx *ctx);
 
@@ -1074,7 +1075,7 @@ hisq_status fp64_prof_begin(hisq_ctx *ctx, int fields, bool *on);
 hisq_status fp64_prof_end(hisq_ctx *ctx, bool on);
 hisq_status launch_dslash(hisq_ctx *ctx, int out_parity, int prec, int link_prec, const void *in,
                           void *out, double a, const void *x, double b, const void *y, double c,
-                          int norm_slot);
+                          int norm_slot, bool fma64 = false);
 
 // CG iteration kernels (sloppy precision `prec`, links `link_prec`, x in xprec)
 hisq_status launch_cg_dslash_tt(hisq_ctx *ctx, int prec, int link_prec, const void *p, void *tmp);
