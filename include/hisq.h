@@ -63,11 +63,11 @@ typedef enum {
 
 /* Storage precisions.  Arithmetic is FP64 for HISQ_PREC_DOUBLE, double-float for
  * HISQ_PREC_DF64 and FP32 otherwise.  Inside a solve (and for the eigenvalues of stored
- * vectors) the FP64 operator forms its sums in fixed point: 56-bit mantissas of the links
- * and of the 16 neighbours of a site, each under one exponent per site, rounded once; FP64
- * FMAs at sites that format cannot hold.  Its error is small relative to the site's
- * largest product, but not relative to a component far below it.  hisq_apply_dslash and
- * hisq_apply_normal_op use FP64 FMAs. */
+ * vectors) the FP64 operator forms its sums in fixed point: 56-bit mantissas under an
+ * exponent per link matrix and colour vector, the 16 products of a site aligned to the
+ * largest, rounded once; FP64 FMAs at sites that format cannot hold.  Its error is below
+ * that of FP64 FMAs relative to the largest products of a site, but not relative to a
+ * component far below them.  hisq_apply_dslash and hisq_apply_normal_op use FP64 FMAs. */
 typedef enum {
     HISQ_PREC_DOUBLE = 64,
     HISQ_PREC_SINGLE = 32,

@@ -351,7 +351,7 @@ hisq_status hisq_load_links(hisq_ctx *ctx, const double *fat, const double *lng,
     for (int p = 0; p < 2; p++) {
         dev_free(ctx, ctx->links_x[p], links_x_bytes(Vh));
         ctx->links_x[p] = nullptr;
-        dev_free(ctx, ctx->links_xe[p], size_t(Vh) * 2);
+        dev_free(ctx, ctx->links_xe[p], links_xe_bytes(Vh));
         ctx->links_xe[p] = nullptr;
         dev_free(ctx, ctx->links_f[p], link_sites(Vh) * (ctx->long_recon == 18 ? 8 : 4) * 9 * 16);
         ctx->links_f[p] = nullptr;
@@ -367,7 +367,7 @@ hisq_status hisq_load_links(hisq_ctx *ctx, const double *fat, const double *lng,
     ctx->links_loaded = false;
     for (int p = 0; p < 2; p++) {
         ctx->links_x[p] = (int4 *)dev_alloc(ctx, links_x_bytes(Vh));
-        ctx->links_xe[p] = (short *)dev_alloc(ctx, size_t(Vh) * 2);
+        ctx->links_xe[p] = (unsigned *)dev_alloc(ctx, links_xe_bytes(Vh));
         ctx->links_f[p] = (float4 *)dev_alloc(ctx, link_sites(Vh) * (long_recon == 18 ? 8 : 4) * 9 * 16);
         if (long_recon != 18) ctx->links_f12[p] = (float4 *)dev_alloc(ctx, link_sites(Vh) * long_f32_bytes_per_site(long_recon));
         if (!ctx->links_x[p] || !ctx->links_xe[p] || !ctx->links_f[p] || (long_recon != 18 && !ctx->links_f12[p])) return HISQ_ERR_OOM;

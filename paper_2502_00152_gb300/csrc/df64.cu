@@ -169,13 +169,13 @@ __global__ void k_split_df(size_t n, const double2 *__restrict__ in, float4 *__r
 }
 
 // the double-float split of the gathered FP64 links (fx64.cuh)
-__global__ void k_split_df_links(int Vh, const int4 *__restrict__ w, const short *__restrict__ e,
-                                 float4 *__restrict__ out)
+__global__ void k_split_df_links(int Vh, LinksX L, float4 *__restrict__ out)
 {
     const size_t n = size_t(Vh) * 144;
     for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
-        const int cb = int(i % size_t(Vh));
-        const double2 d = fx_link(w[fx_link_index(cb, int(i / size_t(Vh)))], e[cb]);
+        const int cb = int(i % size_t(Vh)), k = int(i / size_t(Vh)), hop = k / 9;
+        const double2 d = fx_link(L.w[fx_link_index(cb, k)],
+                                  fx_hop_exponent(L.e[cb], L.dl[size_t(4) * cb + (hop >> 2)], hop & 3));
         const float2 re = split_df(d.x), im = split_df(d.y);
         out[i] = make_float4(re.x, re.y, im.x, im.y);
     }
@@ -201,7 +201,7 @@ hisq_status ensure_df_links(hisq_ctx *ctx)
     hisq_status s = (d[0] && d[1]) ? HISQ_OK : HISQ_ERR_OOM;
     for (int p = 0; p < 2 && s == HISQ_OK; p++) {
         ctx->launches++;
-        k_split_df_links<<<ctx->num_sms * 8, 256, 0, ctx->stream>>>(ctx->g.Vh, ctx->links_x[p], ctx->links_xe[p], d[p]);
+        k_split_df_links<<<ctx->num_sms * 8, 256, 0, ctx->stream>>>(ctx->g.Vh, links_fx(ctx, p), d[p]);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) s = cuda_err(ctx, e, "double-float link split");
     }

@@ -155,10 +155,11 @@ struct LinksXv {
     __device__ __forceinline__ void load(int mu, int kind, int i, CMat<double> &f, CMat<double> &b) const
     {
         const int4 *q = L.w + fx_link_index(i, (mu * 2 + kind) * 18);
-        const int eb = L.e[i];
+        const unsigned dl = __ldg(L.dl + size_t(4) * i + mu);
+        const int ef = fx_hop_exponent(L.e[i], dl, 2 * kind), eb = fx_hop_exponent(L.e[i], dl, 2 * kind + 1);
 #pragma unroll
         for (int k = 0; k < 9; k++) {
-            const double2 x = fx_link(__ldcs(q + 32 * k), eb), y = fx_link(__ldcs(q + 32 * (9 + k)), eb);
+            const double2 x = fx_link(__ldcs(q + 32 * k), ef), y = fx_link(__ldcs(q + 32 * (9 + k)), eb);
             f.re[k] = x.x;
             f.im[k] = x.y;
             b.re[k] = y.x;
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__(256, sizeof(typename Lk::real) == 8 ? 1 : 2)
 // Bound by the 2304 B of links per site.  Each thread holds the links and the neighbour
 // of two hops (100 registers), so that a warp has 6.5 KB of loads in flight while it
 // multiplies.  32^3x64, split of the input included: 439 us per application at 168
-// registers (12 warps per SM); FP64 FMAs took 1040.  With links cut to 56-bit limbs
+// registers (12 warps per SM); FP64 FMAs take 1058.  With links cut to 56-bit limbs
 // beforehand, which saves the shift of each real but loses bits of the small ones: 417, at
 // 128 registers (432 B spilled) 500, with the links in shared memory as the batch has them 513.
 //
@@ -258,11 +259,12 @@ __global__ void __launch_bounds__(128, 3)
         cb_coords(g, par, cb, c);
         const int s = full_site(g, c);
         const int4 *w = L.w + fx_link_index(cb, 0);
-        const int le = L.e[cb], E = fp64 ? kFxMark : fx_site_exponent(g, c, s, in.e);
+        const unsigned *dl = L.dl + size_t(4) * cb;
+        const int le = L.e[cb], E = fp64 ? kFxMark : fx_site_exponent(g, c, s, in.e, dl);
         const bool mark = E == kFxMark || le == kFxMark;
         FxAcc acc;
         acc.zero();
-        if (!mark) fx_directions(g, c, s, SPLIT == 1 ? 0 : part, SPLIT == 1 ? 4 : part + 1, w, in, E, acc);
+        if (!mark) fx_directions(g, c, s, SPLIT == 1 ? 0 : part, SPLIT == 1 ? 4 : part + 1, w, dl, in, E, acc);
         if (SPLIT > 1) {
             if (part > 0) {
 #pragma unroll
@@ -293,7 +295,7 @@ __global__ void __launch_bounds__(128, 3)
                     o.im[i] = double(fx_sum(acc, 2 * i + 1)) * u;
                 }
             } else {
-                o = fx_site_fp64(g, c, s, w, le, in.src);
+                o = fx_site_fp64(g, c, s, w, dl, le, in.src);
             }
             epi(cb, o, red);
         }
@@ -331,7 +333,7 @@ static hisq_status run_fx(hisq_ctx *ctx, int par, const SpinorD &in, const Epi &
         const hisq_status st = launch_fx_split(ctx, in.p, buf);
         if (st != HISQ_OK) return st;
     }
-    const LinksX L{ctx->links_x[par], ctx->links_xe[par]};
+    const LinksX L = links_fx(ctx, par);
     const FxField f = fx_field(buf, in.p, Vh);
     auto launch = [&](auto kern, int sites, int bps) -> hisq_status {
         const int grid = grid_for(ctx, Vh, sites, bps);
@@ -359,7 +361,7 @@ static hisq_status run_any(hisq_ctx *ctx, int par, int link_prec, const S &in, c
     if (link_prec == 64) {
         if constexpr (sizeof(R) == 8 && !FMA64) return run_fx(ctx, par, in, epi, ra, dored);
         if constexpr (sizeof(R) == 8 && FMA64)
-            return run_dslash<S, LinksXv, LinksF12, false>(ctx, par, LinksXv{{ctx->links_x[par], ctx->links_xe[par]}},
+            return run_dslash<S, LinksXv, LinksF12, false>(ctx, par, LinksXv{links_fx(ctx, par)},
                                                            LinksF12{nullptr, Vh}, in, epi, ra, dored);
         return set_err(ctx, HISQ_ERR_INVALID_ARG, "FP64 links need FP64 vectors");
     }

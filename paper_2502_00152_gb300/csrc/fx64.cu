@@ -41,37 +41,54 @@ hisq_status launch_fx_split(hisq_ctx *ctx, const void *in, void *out)
 // the 144 elements of its site.  Zero matrices get an ordinary exponent; sites whose
 // largest entry lies outside 2^+-100, or that have one more than 127 binary places below
 // it, stay FP64 and are marked.
-__global__ void __launch_bounds__(256) k_links_fx(int Vh, int4 *w, short *e)
+__global__ void __launch_bounds__(256) k_links_fx(int Vh, int4 *w, unsigned *dl, short *e)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Vh; i += gridDim.x * blockDim.x) {
         int4 *p = w + fx_link_index(i, 0);
-        int eb = 0, low = 0x7ff; // exponents of the largest and of the smallest entry that is not zero
-        for (int k = 0; k < 144; k++) {
-            const int4 q = p[32 * k];
-            for (const double x : {__hiloint2double(q.y, q.x), __hiloint2double(q.w, q.z)}) {
-                const int ex = fx_exponent(x);
-                eb = max(eb, ex);
-                if (x != 0.0) low = min(low, ex);
+        int eb = 0, low = 0x7ff; // exponents of the largest entry and of the smallest that is not zero
+        int hop[16];             // of the largest of each hop, 0 for a zero matrix
+        bool zero = true;
+#pragma unroll
+        for (int h = 0; h < 16; h++) {
+            hop[h] = 0;
+            for (int k = 9 * h; k < 9 * h + 9; k++) {
+                const int4 q = p[32 * k];
+                for (const double x : {__hiloint2double(q.y, q.x), __hiloint2double(q.w, q.z)}) {
+                    hop[h] = max(hop[h], fx_exponent(x));
+                    if (x != 0.0) low = min(low, fx_exponent(x));
+                    zero = zero && x == 0.0;
+                }
             }
+            eb = max(eb, hop[h]);
         }
-        if (low == 0x7ff && eb == 0) eb = low = 1022; // all zero
+        if (zero) eb = low = 1022;
         if (eb < kFxLinkLo || eb > kFxLinkHi || eb - low > kFxDepth) {
             e[i] = short(kFxMark);
+            reinterpret_cast<uint4 *>(dl)[i] = make_uint4(0, 0, 0, 0);
             continue;
         }
         e[i] = short(eb);
-        for (int k = 0; k < 144; k++) {
-            const int4 q = p[32 * k];
-            const long long re = fx_encode(__hiloint2double(q.y, q.x), eb), im = fx_encode(__hiloint2double(q.w, q.z), eb);
-            p[32 * k] = make_int4(int(re), int(re >> 32), int(im), int(im >> 32));
+        unsigned d[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int h = 0; h < 16; h++) {
+            const int depth = min(eb - hop[h], kFxDepth);
+            d[h >> 2] |= unsigned(depth) << (8 * (h & 3));
+            for (int k = 9 * h; k < 9 * h + 9; k++) {
+                const int4 q = p[32 * k];
+                const long long re = fx_encode(__hiloint2double(q.y, q.x), eb - depth);
+                const long long im = fx_encode(__hiloint2double(q.w, q.z), eb - depth);
+                p[32 * k] = make_int4(int(re), int(re >> 32), int(im), int(im >> 32));
+            }
         }
+        reinterpret_cast<uint4 *>(dl)[i] = make_uint4(d[0], d[1], d[2], d[3]);
     }
 }
 
 hisq_status launch_links_fx(hisq_ctx *ctx, int par)
 {
     const int grid = grid_for(ctx, ctx->g.Vh, 256, 8);
-    k_links_fx<<<grid, 256, 0, ctx->stream>>>(ctx->g.Vh, ctx->links_x[par], ctx->links_xe[par]);
+    k_links_fx<<<grid, 256, 0, ctx->stream>>>(ctx->g.Vh, ctx->links_x[par], ctx->links_xe[par],
+                                              (short *)(ctx->links_xe[par] + size_t(4) * ctx->g.Vh));
     const cudaError_t err = cudaGetLastError();
     return err == cudaSuccess ? HISQ_OK : cuda_err(ctx, err, "fixed-point links");
 }
@@ -119,9 +136,10 @@ hisq_status launch_fx_batch_split(hisq_ctx *ctx, const FxGroup &grp, FxArray in,
 
 // The operator for a group of fields (fx_ring_sites), blockIdx.y: fields blockIdx.y * nch ...
 // Bound by instruction issue and the multiply-add pipe together (54 % busy at 12 warps):
-// 32^3x64, per field and application, splits included: 377 us for 12 or 5 fields, one field
-// at a time 439, FP64 FMAs 1040.  With links cut to 56-bit limbs beforehand (bits of the
-// small ones lost) 351 and 340; two fields per thread, with four real products per complex
+// 32^3x64, per field and application, splits included: 386 us for 12 or 5 fields, one field
+// at a time 439, FP64 FMAs 1058.  With one exponent per site instead of one per hop 377;
+// with links cut to 56-bit limbs beforehand as well (bits of the small ones lost) 351 and
+// 340; two fields per thread, with four real products per complex
 // one, took 495.
 __global__ void __launch_bounds__(32 * kFxWarps, 2)
     k_dslash_fx_batch(Geom g, int par, LinksX L, FxGroup grp, FxBatch o, size_t ms, FxTile tl, double *partials,
@@ -151,7 +169,8 @@ __global__ void __launch_bounds__(32 * kFxWarps, 2)
                               v.im[i] = double(fx_sum(acc, 2 * i + 1));
                           }
                       } else {
-                          v = fx_site_fp64(g, c, s, L.w + fx_link_index(cb, 0), le, fx_at(o.in, grp, q, Vh));
+                          v = fx_site_fp64(g, c, s, L.w + fx_link_index(cb, 0), L.dl + size_t(4) * cb, le,
+                                             fx_at(o.in, grp, q, Vh));
                       }
                       t.zero();
                       if (o.y.base) {
@@ -249,7 +268,7 @@ hisq_status launch_fx_batch(hisq_ctx *ctx, int par, const FxGroup &grp, const Fx
     bool timed = false;
     st = fp64_prof_begin(ctx, grp.k, &timed);
     if (st != HISQ_OK) return st;
-    kern<<<grid, threads, smem, ctx->stream>>>(ctx->g, par, LinksX{ctx->links_x[par], ctx->links_xe[par]}, grp, b,
+    kern<<<grid, threads, smem, ctx->stream>>>(ctx->g, par, links_fx(ctx, par), grp, b,
                                                fx_field_bytes(Vh), tl, ctx->bpartials, ctx->ticket + 40, ctx->bscal->out,
                                                ctx->wait_status_d, ring_spin_limit(ctx));
     const cudaError_t err = cudaGetLastError();

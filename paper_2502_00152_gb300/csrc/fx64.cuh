@@ -11,14 +11,15 @@
 // (Karatsuba's identity, see FxAcc): 1296 multiply-adds, 43 clocks per site.
 //
 // Block floating point: the six reals of a colour vector share the exponent of the
-// largest one, the 288 link reals of an output site share theirs, and at an output
-// site the 16 neighbour vectors are aligned to the largest of their exponents.  In the sums
-// a mantissa has 56 bits below the shared exponent (FP64 keeps 53 below its own), and
-// the integer sums are exact.  So an error is at most 2.3 x 96 x 2^-56 of the product of
-// the two shared powers of two: small against the site's result, but not against a component
-// that only small entries couple to.  The solves use this operator, whose residuals are
-// norms over the lattice; hisq_apply_dslash and hisq_apply_normal_op, whose callers see each
-// component, run on FP64 FMAs.  Measured against 113-bit sums on 8^4: relative error
+// largest one, the 18 reals of a hop's matrix theirs, and the 16 products of an output site
+// are aligned to the largest sum of the two.  In the sums a matrix entry has 56 bits below
+// its hop's exponent, a vector entry the same less what its product is shifted down (FP64
+// keeps 53 below its own), and the integer sums are exact.  So an error is at most about
+// 2.3 x 96 x 2^-56 of the largest product of a matrix's and a vector's power of two: small
+// against the site's result, but not against a component that only small entries couple
+// to.  The solves use this operator, whose residuals are norms over the lattice;
+// hisq_apply_dslash and hisq_apply_normal_op, whose callers see each component, run on FP64
+// FMAs.  Measured against 113-bit sums on 8^4: relative error
 // 6.4e-17 for a Gaussian field (FP64 FMAs 3.5e-16), 1.0e-16 where site vectors differ by
 // up to e^20 (3.5e-16).  The sums do not depend on the order of the terms, so a site may be
 // split over threads without changing a bit of the result.
@@ -32,7 +33,7 @@
 // Links are stored by groups of 32 sites, [group][mu][kind][fwd,bwd][k][32] int4: the
 // 144 loads of a thread are at constant offsets from one address.  A real keeps its own 53
 // bits: its signed mantissa times 2^7 in 64 bits, with the number of places it lies below
-// the site's exponent in the seven low ones, so that one shift aligns it (links of the
+// its hop's exponent in the seven low ones, so that one shift aligns it (links of the
 // solves, of FP64 FMAs and of the double-float operator are the same values).
 //
 // Values the block format cannot hold -- Inf, NaN, and exponents so far out that a
@@ -59,12 +60,20 @@ struct FxField {
 };
 
 // gathered links of one output parity: int4 = (re low, re high, im low, im high) words of an
-// element (fx_encode), biased exponents [Vh]; where the exponent is kFxMark they hold the
-// two FP64 values themselves
+// element (fx_encode); of each site the biased exponent of its largest entry and, one byte
+// per hop, how far that of the hop's largest entry lies below it (fx_hop_exponent).  Where
+// the site's exponent is kFxMark the int4 hold the two FP64 values themselves.
 struct LinksX {
-    const int4 *w; // fx_link_index
-    const short *e;
+    const int4 *w;      // fx_link_index
+    const unsigned *dl; // [Vh][mu], byte h = hop of the direction: fat fwd, fat bwd, long fwd, long bwd
+    const short *e;     // [Vh]
 };
+inline LinksX links_fx(const hisq_ctx *ctx, int par)
+{
+    return LinksX{ctx->links_x[par], ctx->links_xe[par], (const short *)(ctx->links_xe[par] + size_t(4) * ctx->g.Vh)};
+}
+__device__ __forceinline__ int fx_depth(unsigned dl, int h) { return int((dl >> (8 * h)) & 255); }
+__device__ __forceinline__ int fx_hop_exponent(int le, unsigned dl, int h) { return le == kFxMark ? le : le - fx_depth(dl, h); }
 
 __host__ __device__ __forceinline__ size_t fx_link_index(int cb, int k) // element k = 9 hop + 3 row + column
 {
@@ -112,8 +121,8 @@ __device__ __forceinline__ void fx_store_site(longlong2 *v, short *e, int Vh, in
         v[size_t(c) * Vh + i] = make_longlong2(fx_mantissa(q.re[c], eb), fx_mantissa(q.im[c], eb));
 }
 
-// a link real under exponent eb: signed mantissa (53 bits) 2^7, and in the low seven bits
-// how far its own exponent lies below eb (at most kFxDepth); zero: 0
+// a link real under its hop's exponent eb: signed mantissa (53 bits) 2^7, and in the low seven
+// bits how far its own exponent lies below eb (at most kFxDepth); zero: 0
 constexpr int kFxDepth = 127;
 __device__ __forceinline__ long long fx_encode(double x, int eb)
 {
@@ -131,7 +140,7 @@ __device__ __forceinline__ double fx_decode(int w0, int w1, int eb)
     return eb == kFxMark ? __hiloint2double(w1, w0) : __hiloint2double(int(top), int(unsigned(m)));
 }
 
-// limbs of an encoded link real shifted down to its site's exponent, |v| <= 2^60.  Below a
+// limbs of an encoded link real shifted down to its hop's exponent, |v| <= 2^60.  Below a
 // shift of 16 the count takes bits that the low limb drops, from 16 on it is shifted out.
 __device__ __forceinline__ void fx_link_limbs(int w0, int w1, int &hi, int &lo)
 {
@@ -156,7 +165,7 @@ __device__ __forceinline__ void fx_shifted_limbs(long long v, int d, int &hi, in
 // 2^k, -1022 <= k <= 1023
 __device__ __forceinline__ double fx_pow2(int k) { return __hiloint2double((k + 1023) << 20, 0); }
 
-// link element (re, im) as FP64
+// link element (re, im) of a hop of exponent eb as FP64
 __device__ __forceinline__ double2 fx_link(int4 q, int eb)
 {
     return make_double2(fx_decode(q.x, q.y, eb), fx_decode(q.z, q.w, eb));
@@ -178,27 +187,30 @@ struct FxAcc {
     }
 };
 
-// the shared exponent of the 16 neighbours of a site (kFxMark if one is marked)
-__device__ __forceinline__ int fx_site_exponent(const Geom &g, const int c[4], int s, const short *e)
+// the largest exponent of a neighbour's vector less its hop's depth, which the 16 products
+// are aligned to (kFxMark if a neighbour is marked)
+__device__ __forceinline__ int fx_site_exponent(const Geom &g, const int c[4], int s, const short *e, const unsigned *dl)
 {
+    const uint4 q = __ldg(reinterpret_cast<const uint4 *>(dl));
+    const unsigned d[4] = {q.x, q.y, q.z, q.w};
     int E = 0;
 #pragma unroll
-    for (int mu = 0; mu < 4; mu++) {
-        E = max(E, max(int(__ldg(e + nb_cb(g, c, s, mu, 1))), int(__ldg(e + nb_cb(g, c, s, mu, -1)))));
-        E = max(E, max(int(__ldg(e + nb_cb(g, c, s, mu, 3))), int(__ldg(e + nb_cb(g, c, s, mu, -3)))));
-    }
-    return E;
+    for (int mu = 0; mu < 4; mu++)
+#pragma unroll
+        for (int h = 0; h < 4; h++)
+            E = max(E, int(__ldg(e + nb_cb(g, c, s, mu, (h & 2 ? 3 : 1) * (h & 1 ? -1 : 1)))) - fx_depth(d[mu], h));
+    return E > kFxVecHi ? kFxMark : E; // a mark less a depth is still above every exponent
 }
 
 // the neighbour's vector of one hop.
 // hop = 4 mu + h, h = 0: fat fwd, 1: fat bwd, 2: long fwd, 3: long bwd.
 struct FxVec {
     longlong2 v[3];
-    int e;
-    __device__ __forceinline__ void load(const Geom &g, const SiteLine &line, int h, const FxField &in)
+    int e; // less the hop's depth
+    __device__ __forceinline__ void load(const Geom &g, const SiteLine &line, int h, const FxField &in, unsigned dl)
     {
         const unsigned nb = unsigned(line.at(g, (h & 2 ? 3 : 1) * (h & 1 ? -1 : 1)));
-        e = __ldg(in.e + nb);
+        e = int(__ldg(in.e + nb)) - fx_depth(dl, h);
 #pragma unroll
         for (int j = 0; j < 3; j++) v[j] = __ldg(in.v + size_t(j) * g.Vh + nb);
     }
@@ -246,18 +258,18 @@ __device__ __forceinline__ void fx_add(const FxVec &x, int E, FxAcc &acc, F &&li
         }
 }
 
-// Directions mu0 .. mu1 - 1 of a site (L: its first link element), links in registers:
+// Directions mu0 .. mu1 - 1 of a site (L: its first link element, dl: its depths), links in registers:
 // the loads of the next hop are issued before the sums of the current one.
 struct FxHop {
     int4 w[9];
     FxVec x;
     __device__ __forceinline__ void load(const Geom &g, const SiteLine &line, int mu, int h, const int4 *L,
-                                         const FxField &in)
+                                         const FxField &in, unsigned dl)
     {
         const int4 *p = L + (mu * 4 + h) * (9 * 32);
 #pragma unroll
         for (int k = 0; k < 9; k++) w[k] = __ldcs(p + 32 * k); // read once per launch
-        x.load(g, line, h, in);
+        x.load(g, line, h, in, dl);
     }
     __device__ __forceinline__ void add(int E, FxAcc &acc) const
     {
@@ -265,22 +277,24 @@ struct FxHop {
     }
 };
 __device__ __forceinline__ void fx_directions(const Geom &g, const int c[4], int s, int mu0, int mu1, const int4 *L,
-                                              const FxField &in, int E, FxAcc &acc)
+                                              const unsigned *dl, const FxField &in, int E, FxAcc &acc)
 {
     FxHop a, b;
     SiteLine line(g, c, s, mu0);
-    a.load(g, line, mu0, 0, L, in);
+    unsigned d = __ldg(dl + mu0);
+    a.load(g, line, mu0, 0, L, in, d);
 #pragma unroll 1
     for (int mu = mu0; mu < mu1; mu++) {
-        b.load(g, line, mu, 1, L, in);
+        b.load(g, line, mu, 1, L, in, d);
         a.add(E, acc);
-        a.load(g, line, mu, 2, L, in);
+        a.load(g, line, mu, 2, L, in, d);
         b.add(E, acc);
-        b.load(g, line, mu, 3, L, in);
+        b.load(g, line, mu, 3, L, in, d);
         a.add(E, acc);
         if (mu + 1 < mu1) {
             line = SiteLine(g, c, s, mu + 1);
-            a.load(g, line, mu + 1, 0, L, in);
+            d = __ldg(dl + mu + 1);
+            a.load(g, line, mu + 1, 0, L, in, d);
         }
         b.add(E, acc);
     }
@@ -300,8 +314,8 @@ __device__ __forceinline__ long long fx_sum(const FxAcc &a, int c)
 __device__ __forceinline__ double fx_unit(int E, int le) { return fx_pow2(E + le - 2100); }
 
 // a marked site (L: its first link element): FP64 FMAs on the original field
-static __device__ __noinline__ CVec<double> fx_site_fp64(const Geom &g, const int c[4], int s, const int4 *L, int le,
-                                                         const double2 *src)
+static __device__ __noinline__ CVec<double> fx_site_fp64(const Geom &g, const int c[4], int s, const int4 *L,
+                                                         const unsigned *dl, int le, const double2 *src)
 {
     const int Vh = g.Vh;
     CVec<double> acc;
@@ -309,6 +323,7 @@ static __device__ __noinline__ CVec<double> fx_site_fp64(const Geom &g, const in
 #pragma unroll 1
     for (int h = 0; h < 16; h++) {
         const int mu = h >> 2, kind = (h >> 1) & 1, bwd = h & 1;
+        const int eh = fx_hop_exponent(le, dl[mu], h & 3);
         const int nb = nb_cb(g, c, s, mu, (kind ? 3 : 1) * (bwd ? -1 : 1));
         const int4 *w = L + h * (9 * 32);
         CVec<double> v;
@@ -321,7 +336,7 @@ static __device__ __noinline__ CVec<double> fx_site_fp64(const Geom &g, const in
         CMat<double> W;
 #pragma unroll
         for (int k = 0; k < 9; k++) {
-            const double2 q = fx_link(w[32 * k], le);
+            const double2 q = fx_link(w[32 * k], eh);
             W.re[k] = q.x;
             W.im[k] = q.y;
         }
@@ -397,7 +412,8 @@ __device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const Link
         cb_coords(g, par, cb, c);
         const int s = full_site(g, c);
         const int le = L.e[cb];
-        const int E = fx_site_exponent(g, c, s, in.e);
+        const unsigned *dl = L.dl + size_t(4) * cb;
+        const int E = fx_site_exponent(g, c, s, in.e, dl);
         FxAcc acc;
         acc.zero();
         // one hop: refill the ring, wait for the links, add
@@ -426,18 +442,20 @@ __device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const Link
         };
         FxVec a, b;
         SiteLine line(g, c, s, 0);
-        a.load(g, line, 0, in);
+        unsigned d = __ldg(dl);
+        a.load(g, line, 0, in, d);
 #pragma unroll 1
         for (int mu = 0; mu < 4; mu++) {
-            b.load(g, line, 1, in);
+            b.load(g, line, 1, in, d);
             hop(4 * mu, a);
-            a.load(g, line, 2, in);
+            a.load(g, line, 2, in, d);
             hop(4 * mu + 1, b);
-            b.load(g, line, 3, in);
+            b.load(g, line, 3, in, d);
             hop(4 * mu + 2, a);
             if (mu < 3) {
                 line = SiteLine(g, c, s, mu + 1);
-                a.load(g, line, 0, in);
+                d = __ldg(dl + mu + 1);
+                a.load(g, line, 0, in, d);
             }
             hop(4 * mu + 3, b);
         }
@@ -458,7 +476,7 @@ __device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const Link
 // Tile for k fields: ny launches' worth of blocks of nch fields and nsg site groups.  An SM
 // holds 16 warps (128 registers); the tile keeps as many of them as it can on fields of
 // their own, and each further reading of the links (ny) costs a little: 12 fields on
-// 32^3x64 took 342 to 377 us per application with 16 or 12 warps at work.
+// 32^3x64 took 10 % longer with 12 warps at work than with 16.
 inline FxTile fx_tile(int k, int *ny)
 {
     FxTile t{1, kFxWarps, 0};

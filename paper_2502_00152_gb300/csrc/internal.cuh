@@ -447,7 +447,7 @@ __device__ __forceinline__ CVec<To> cvt(const CVec<From> &v)
 // (kind 0: fat, n = 1; kind 1: long, n = 3).
 //
 // FP64 (recon 18): [p][group of 32 sites][mu][kind][fwd,bwd][k=0..8][32], 16 B per complex
-//   element: 53-bit mantissas with their places below one exponent per output site (fx64.cuh)
+//   element: 53-bit mantissas with their places below one exponent per hop (fx64.cuh)
 // The FP32 and FP16 arrays are stored by groups of 32 output sites, rows x 32 sites each
 // (link_index):
 // FP32 (recon 18): float4, row (mu * 2 + kind) * 9 + k; float4 = (Re fwd, Re bwd, Im fwd,
@@ -547,6 +547,9 @@ struct LinksF8 { // long links only, 8 reals per SU(3) factor
 
 // bytes of the FP64 links of one parity (whole groups of 32 sites)
 inline size_t links_x_bytes(int Vh) { return size_t((Vh + 31) / 32) * 32 * 144 * 16; }
+
+// and of their exponents, 18 per site
+inline size_t links_xe_bytes(int Vh) { return size_t(Vh) * 18; }
 
 // sites of the FP32 and FP16 link arrays (whole groups)
 inline size_t link_sites(int Vh) { return size_t((Vh + 31) / 32) * 32; }
@@ -789,7 +792,7 @@ struct hisq_ctx {
 
     // gathered links; index [parity]
     int4 *links_x[2] = {nullptr, nullptr};     // FP64, 16 hops (fx_encode, fx64.cuh)
-    short *links_xe[2] = {nullptr, nullptr};   // their exponents, one per output site
+    unsigned *links_xe[2] = {nullptr, nullptr}; // their exponents: [Vh][4] depths of the hops, short [Vh] of the sites
     float4 *links_f[2] = {nullptr, nullptr};   // FP32: fat (+ long when recon 18)
     float4 *links_f12[2] = {nullptr, nullptr}; // FP32 long, recon 12
     uint2 *links_h[2] = {nullptr, nullptr};    // FP16: fat (+ long when recon 18)

@@ -1,6 +1,15 @@
-"""Accuracy of the FP64 operator against sums in extended precision: hisq_apply_dslash runs
-on FP64 FMAs, so that each component is within 96 roundings of the sum of its products'
-magnitudes, however small it is beside the others of its site."""
+"""Accuracy of the two FP64 forms of the operator against sums in extended precision.
+
+hisq_apply_dslash runs on FP64 FMAs: each component is within 96 roundings of the sum of
+its products' magnitudes, however small it is beside the others of its site.
+
+A solve runs on fixed-point sums: 56 bits below the largest of the 16 hops' powers of two
+(largest matrix entry times largest vector entry).  Its operator is read out of a solve that converges
+at once: with m = 1/2, eta zero on odd sites, the field as the guess and a tolerance above
+any residual, the odd part of psi is -D_oe of the guess.
+
+6^3 x 10: four warps per site group and a ragged last group; 18 x 16^2 x 34: one thread per
+site."""
 import numpy as np
 import pytest
 
@@ -32,20 +41,25 @@ def field(dims, kind):
     if kind == "components":  # each real of its own size
         f.real *= np.ldexp(1.0, r.integers(-60, 1, f.shape))
         f.imag *= np.ldexp(1.0, r.integers(-60, 1, f.shape))
-    elif kind == "sites300":
-        f *= np.ldexp(1.0, r.integers(-300, 301, f.shape[0]))[:, None]
+    elif kind in ("sites40", "sites300"):
+        k = int(kind[5:])
+        f *= np.ldexp(1.0, r.integers(-k, k + 1, f.shape[0]))[:, None]
         f[r.random(f.shape[0]) < 0.1] = 0
+    elif kind == "tiny":  # sites below the block format's range
+        f[r.random(f.shape[0]) < 0.1] *= 1e-290
     elif kind == "point":
         f[:] = 0
         f[r.choice(f.shape[0], 20, replace=False), 1] = 1
+    elif kind == "wall":
+        f = I.z2_wall_source(dims, 5, 2, 0)
     else:
         assert kind == "gauss"
     return f
 
 
 class Extended:
-    """D at some sites of one parity: sums in extended precision and the sums of the products'
-    magnitudes"""
+    """D at some sites of one parity: sums in extended precision, the sums of the products'
+    magnitudes, and the error bound of the fixed-point form"""
 
     def __init__(self, dims, fat, lng, f, par, nsites):
         X, Y, Z, T = dims
@@ -57,6 +71,7 @@ class Extended:
         self.sites, x = p, x[:, p]
         f = project_parity(dims, f, 1 - par)
         stride = (1, X, X * Y, X * Y * Z)
+        big = lambda a: np.maximum(np.abs(a.real), np.abs(a.imag)).reshape(len(p), -1).max(1)
         mats, vecs = [], []
         for mu in range(4):
             eta = 1.0 - 2.0 * (x[:mu].sum(0) % 2)
@@ -69,20 +84,44 @@ class Extended:
                     mats.append(phase[:, None, None] * w)
                     vecs.append(f[nb])
         self.hits = np.sum([np.any(v != 0, axis=1) for v in vecs], axis=0)
+        two = lambda q: np.where(q > 0, np.ldexp(1.0, np.frexp(q)[1]), 0)[:, None]
+        A, B = [two(big(w)) for w in mats], [two(big(v)) for v in vecs]
+        P = np.max([a * b for a, b in zip(A, B)], axis=0)  # what all products are aligned to
         L = np.longdouble
         self.re, self.im = np.zeros((2, len(p), 3), L)
-        self.mag_re, self.mag_im = np.zeros((2, len(p), 3))
-        for w, v in zip(mats, vecs):
+        self.mag_re, self.mag_im, part = np.zeros((3, len(p), 3))
+        for w, v, scale in zip(mats, vecs, A):
             a, b = w.real, w.imag
             c, d = (q[:, None, :] for q in (v.real, v.imag))
             self.re += (a.astype(L) * c - b.astype(L) * d).sum(-1)
             self.im += (a.astype(L) * d + b.astype(L) * c).sum(-1)
             self.mag_re += (np.abs(a * c) + np.abs(b * d)).sum(-1)
             self.mag_im += (np.abs(a * d) + np.abs(b * c)).sum(-1)
+            part += (scale * (np.abs(c) + np.abs(d))[:, 0, :].sum(-1, keepdims=True)
+                     + P / np.where(scale > 0, scale, 1) * (np.abs(a) + np.abs(b)).sum(-1) + 3 * P / 2)
+        # a link real of a hop is cut to 2^-56 of its scale A, a neighbour's (after rounding to 2^-60
+        # of its own) to 2^-56 P / A, a product of two low limbs (below 2^-58 P) is dropped, the sum
+        # rounded to 2^-56 P and to FP64
+        self.bound_re = 1.1 * 2.0 ** -56 * part + U * np.abs(self.re)
+        self.bound_im = 1.1 * 2.0 ** -56 * part + U * np.abs(self.im)
+        # sites next to a vector outside the format (2^+-700) are summed in FP64
+        out = np.any([(big(v) > 0) & (big(v) < 2.0 ** -699) for v in vecs], axis=0)
+        self.bound_re[out], self.bound_im[out] = 97 * U * self.mag_re[out], 97 * U * self.mag_im[out]
 
     def errors(self, out):
         o = out[self.sites]
         return np.abs(o.real - self.re), np.abs(o.imag - self.im)
+
+
+def solve_operator(ctx, dims, f):
+    """D_oe f as a solve computes it"""
+    H.hisq_set_mass(ctx, 0.5)
+    eta = np.zeros((int(np.prod(dims)), 3), complex)
+    eta[0, 0] = 1
+    prm = H.hisq_default_solve_params(batch=0, guess=1, tol=1e200)
+    psi, st, status = H.hisq_solve(ctx, eta, prm, guess=project_parity(dims, f, 0))
+    assert status == H.HISQ_OK and st[0]["iterations"] == 0
+    return -project_parity(dims, psi, 1)
 
 
 def context(dims, fat, lng):
@@ -110,5 +149,36 @@ def test_applied_operator_is_accurate_in_each_component(dims, depth, kind):
                 one = ref.hits == 1
                 assert dims == LARGE or one.sum() > 50
                 assert np.array_equal(out[ref.sites][one], (ref.re + 1j * ref.im)[one].astype(complex))
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("dims", [SMALL, LARGE])
+@pytest.mark.parametrize("depth", [0, 60])
+@pytest.mark.parametrize("kind", ["gauss", "components", "sites40", "sites300", "tiny", "point", "wall"])
+def test_solve_operator_is_accurate_at_each_site(dims, depth, kind):
+    fat, lng = links(dims, depth)
+    f = field(dims, kind)
+    ctx = context(dims, fat, lng)
+    try:
+        ref = Extended(dims, fat, lng, f, 1, 3000)
+        er, ei = ref.errors(solve_operator(ctx, dims, f))
+        assert np.all(er <= ref.bound_re) and np.all(ei <= ref.bound_im)
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("kind", ["gauss", "sites40"])
+def test_solve_operator_is_no_less_accurate_than_fp64(kind):
+    """dense fields: relative to the largest product of a site, its rms error is below that of
+    FP64 FMAs"""
+    fat, lng = links(SMALL, 0)
+    f = field(SMALL, kind)
+    ctx = context(SMALL, fat, lng)
+    try:
+        ref = Extended(SMALL, fat, lng, f, 1, 3000)
+        scale = np.maximum(ref.mag_re, ref.mag_im).max(1, keepdims=True)
+        rms = lambda out: np.sqrt(np.mean([np.mean((e / scale) ** 2) for e in ref.errors(out)]))
+        assert rms(solve_operator(ctx, SMALL, f)) <= rms(H.hisq_apply_dslash(ctx, 1, 64, f))
     finally:
         ctx.close()
