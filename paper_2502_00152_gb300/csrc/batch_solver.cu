@@ -225,13 +225,13 @@ hisq_status solve_batched(hisq_ctx *ctx, const hisq_solve_params *P, const doubl
     // the target is recomputed in FP64 first, and a right-hand side whose FP64
     // residual does not confirm it stays on FP64 residuals from then on
     std::vector<char> use_df(k, P->precision_reliable == HISQ_PREC_DF64);
-    // tok[j]: t_hi holds D_oe x_j for the current x_j (left by an FP64
-    // residual); tval[j]: rh(j), no longer needed once j has finished, keeps
-    // that D_oe x_j for the odd reconstruction
+    // tok[j]: tsrc[j] (t_hi, or j's slot of its group's scratch until the next group
+    // runs) holds D_oe x_j for the current x_j, left by an FP64 residual; tval[j]: rh(j),
+    // no longer needed once j has finished, keeps that D_oe x_j for the odd reconstruction
     std::vector<char> tok(k, 0), tval(k, 0);
     // |r_e|^2 of the full residual left by the FP64 confirmation of j (-1: none)
     std::vector<double> re2f(k, -1.0);
-    std::vector<const double *> tsrc(k, t_hi); // where the D_oe x_j of tok[j] lies
+    std::vector<const double *> tsrc(k, t_hi);
     auto keep_t = [&](int j) -> hisq_status {
         if (!tok[j]) return HISQ_OK;
         HISQ_CUDA(cudaMemcpyAsync(rh(j), tsrc[j], s64, cudaMemcpyDeviceToDevice, ctx->stream));

@@ -1,11 +1,13 @@
-"""The FP64 operator inside a solve when device memory runs out: its scratch (the mantissas
+"""The FP64 operator inside a solve.  When device memory runs out: its scratch (the mantissas
 of one field, 50 B per site) is asked for once per solve, after the buffers the solve needs
 and never inside the iterations that are captured into a CUDA graph; refused, the whole
-solve runs on FP64 FMAs."""
+solve runs on FP64 FMAs.  For a batch on a half-volume that is not whole groups of 32 sites:
+its residuals are the oracle's."""
 import numpy as np
 import pytest
 
 from gpu_common import make
+from oracle.oracle import project_parity
 from paper_2502_00152_gb300 import hisq as H
 from paper_2502_00152_gb300 import inputs as I
 
@@ -52,5 +54,27 @@ def test_solve_without_room_for_the_mantissas(sloppy, reliable):
         assert status == H.HISQ_OK and o.full_residual(m, psi2.reshape(-1, 3), eta) <= 1e-10
         assert 48 * VH <= H.hisq_device_bytes(ctx) - before <= 52 * VH + 512
         assert np.linalg.norm(psi - psi2) <= 1e-7 * np.linalg.norm(psi)
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("nrhs", [2, 3, 5, 8, 12, 13, 17])
+def test_batched_residuals_on_a_ragged_volume(nrhs):
+    """6^3 x 10: 33 groups of 32 sites and one of 24.  Source preparation, the reliable update
+    and the full residual of fields of sizes from 1 to 1e4, in groups of up to 12 with a
+    remainder; two FP64 evaluations of a residual of order 1 agree to far better than 1e-9."""
+    dims, m = (6, 6, 6, 10), 0.02
+    ctx, o = make(dims, seed=5, eps=0.3, mass=m)
+    try:
+        etas = np.stack([I.gaussian_source(dims, 13, j) * 10.0 ** (j % 5) for j in range(nrhs)])
+        prm = H.hisq_default_solve_params(batch=1, max_iter=3, tol=1e-14, precision_sloppy=32)
+        psi, st, status = H.hisq_solve(ctx, etas, prm)
+        assert status == H.HISQ_ERR_NOT_CONVERGED
+        for j in range(nrhs):
+            y = project_parity(dims, o.prepare_source(m, etas[j]), 0)
+            ref = o.even_residual(m, project_parity(dims, psi[j], 0), y)
+            assert abs(st[j]["even_residual"] - ref) <= 1e-9 * ref
+            full = o.full_residual(m, psi[j], etas[j])
+            assert abs(st[j]["full_residual"] - full) <= 1e-9 * full
     finally:
         ctx.close()
