@@ -56,7 +56,7 @@ def dslash_source_hash() -> str:
     kernels; a stored ncu traffic figure is valid only for the hash it was
     taken on."""
     h = hashlib.sha256()
-    for name in ("dslash.cu", "mrhs.cu", "internal.cuh"):
+    for name in ("dslash.cu", "mrhs.cu", "internal.cuh", "fx64.cuh", "tc.cuh"):
         with open(os.path.join(CSRC, name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
