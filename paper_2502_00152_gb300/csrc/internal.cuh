@@ -945,6 +945,7 @@ hisq_status graph_run(hisq_ctx *ctx, IterGraphs &G, int slot, long long key, F &
     }
     if (!G.exec[slot]) {
         const unsigned long long l0 = ctx->launches;
+        ctx->alloc_in_capture = false; // one refused in a capture of the caller's is not this one's
         cudaError_t e = cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_err(ctx, e, "graph capture begin");
         hisq_status s = body(true);

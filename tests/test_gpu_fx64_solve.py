@@ -5,9 +5,10 @@ solve runs on FP64 FMAs.  For a batch on a half-volume that is not whole groups 
 its residuals are the oracle's."""
 import numpy as np
 import pytest
+import torch
 
 from gpu_common import make
-from oracle.oracle import project_parity
+from oracle.oracle import Oracle, project_parity
 from paper_2502_00152_gb300 import hisq as H
 from paper_2502_00152_gb300 import inputs as I
 
@@ -54,6 +55,37 @@ def test_solve_without_room_for_the_mantissas(sloppy, reliable):
         assert status == H.HISQ_OK and o.full_residual(m, psi2.reshape(-1, 3), eta) <= 1e-10
         assert 48 * VH <= H.hisq_device_bytes(ctx) - before <= 52 * VH + 512
         assert np.linalg.norm(psi - psi2) <= 1e-7 * np.linalg.norm(psi)
+    finally:
+        ctx.close()
+
+
+def test_allocation_in_a_callers_capture_does_not_outlast_it():
+    """A call that needs memory while its caller captures the stream is refused with a message
+    and leaves the capture usable; a later solve captures its own iterations as usual."""
+    m = 0.02
+    fat, lng = I.hisq_links(DIMS, 5, 0.3)
+    o = Oracle(DIMS, fat, lng, t_antiperiodic=True)
+    s = torch.cuda.Stream()
+    ctx = H.hisq_create(DIMS, True, 0, s.cuda_stream)
+    try:
+        H.hisq_load_links(ctx, fat, lng)
+        H.hisq_set_mass(ctx, m)
+        x = torch.zeros(2, 2 * VH, 3, dtype=torch.complex64, device="cuda")
+        gw = torch.zeros(2, 2, 9, dtype=torch.complex64, device="cuda")
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(s):
+            g.capture_begin()
+            try:
+                with pytest.raises(H.HisqError) as e:
+                    H.hisq_net_wgrad(ctx, x, x, gw)  # its partial sums have no buffer yet
+            finally:
+                g.capture_end()
+        assert "captured" in str(e.value)
+        eta = I.gaussian_source(DIMS, 13, 0)
+        psi, st, status = H.hisq_solve(ctx, eta, H.hisq_default_solve_params(batch=0, precision_sloppy=64))
+        assert status == H.HISQ_OK and st[0]["iterations"] > 8
+        assert o.full_residual(m, psi, eta) <= 1e-10
     finally:
         ctx.close()
 
