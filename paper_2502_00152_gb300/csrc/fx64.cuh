@@ -434,8 +434,7 @@ __device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const Link
             if (ok) ok = tc::mbar_wait(&full[slot], phase, status, tc::TC_TIMEOUT_FULL, spin_limit);
             const int4 *w = reinterpret_cast<const int4 *>(ring + size_t(slot) * kFxHopBytes) + lane;
             if (ok) fx_add(cur, E, acc, [&](int k) { return w[32 * k]; });
-            ok = __all_sync(0xffffffffu, ok);
-            if (ok) tc::ring_release(&empty[slot]);
+            tc::ring_release(&empty[slot], ok);
             if (++slot == stages) {
                 slot = 0;
                 phase ^= 1;
@@ -460,6 +459,7 @@ __device__ __forceinline__ void fx_ring_sites(const Geom &g, int par, const Link
             }
             hop(4 * mu + 3, b);
         }
+        ok = __all_sync(0xffffffffu, ok); // the lanes leave the loop together
         if (ok && at < Vh) site(cb, c, s, E, le, acc);
     }
     // copies still in flight (only after a wait gave up) land before the block ends

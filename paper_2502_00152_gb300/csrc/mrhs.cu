@@ -895,8 +895,9 @@ __global__ void __launch_bounds__(512, 1)
 //    to the neighbour.
 // Bound by instruction issue (65 %: 1165 instructions per site and right-hand side, 576 of
 // them the FMAs) and the FMA pipe (52 %).  12 right-hand sides, FP16 vectors, 32^3x64:
-// D_oe 622 -> 554 us, fused update 714 -> 616 us (R = 4, 12 warps per SM) against the
-// register kernel below; R = 3 with 16 warps 611, R = 2 729.  Packed FMAs (fwd, bwd) with
+// D_oe 622 -> 559 us, fused update 714 -> 624 us (R = 4, 12 warps per SM) against the
+// register kernel below; R = 3 with 16 warps 611, R = 2 729.  (A vote of the warp per
+// direction instead of per site group: D_oe 567.)  Packed FMAs (fwd, bwd) with
 // R = 3 took 705: the pairs cost a third more registers and a move per unpacked value.
 // Every wait is bounded: one that runs out records its code in *status, the warp gives up
 // the rest of its sites (the reduction still runs) and the launch ends.
@@ -1135,13 +1136,13 @@ __global__ void __launch_bounds__(MAXT, 1)
 #pragma unroll
                 for (int k = 0; k < 9; k++) mac(k / 3, k % 3, w[32 * (9 + k)]);
             }
-            ok = __all_sync(0xffffffffu, ok);
-            if (ok) tc::ring_release(&empty[slot]);
+            tc::ring_release(&empty[slot], ok);
             if (++slot == stages) {
                 slot = 0;
                 phase ^= 1;
             }
         }
+        ok = __all_sync(0xffffffffu, ok); // the lanes leave the loop together
         if (ok && at < Vh) epi.all(cb, jj, on, acc, red);
     }
     // copies still in flight (only after a wait gave up) land before the block ends
@@ -1327,7 +1328,7 @@ __global__ void __launch_bounds__(256, MINB)
                 }
             }
         }
-        tc::ring_release(&empty[it % stages]);
+        tc::ring_release(&empty[it % stages], true);
         if (mu == 3 && valid) {
 #pragma unroll
             for (int u = 0; u < R; u++)

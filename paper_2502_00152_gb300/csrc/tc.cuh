@@ -41,13 +41,14 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-// This warp's reads of a ring slot are done: lane 0 arrives on the slot's `empty` barrier.
-// The warp barrier orders the other lanes' reads before that arrival, and so before the
-// copy that refills the slot; a vote (__all_sync) would not: it orders no memory access.
-__device__ __forceinline__ void ring_release(uint64_t *empty)
+// This warp's reads of a ring slot are done: lane 0 arrives on the slot's `empty` barrier
+// (unless its wait for the slot gave up).  The warp barrier orders the other lanes' reads
+// before that arrival, and so before the copy that refills the slot; a vote (__all_sync)
+// would not: it orders no memory access.
+__device__ __forceinline__ void ring_release(uint64_t *empty, bool ok)
 {
     __syncwarp();
-    if ((threadIdx.x & 31) == 0) mbar_arrive(empty);
+    if ((threadIdx.x & 31) == 0 && ok) mbar_arrive(empty);
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)

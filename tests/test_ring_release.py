@@ -22,5 +22,5 @@ def test_ring_slots_are_released_after_a_warp_barrier():
         released += len(re.findall(r"ring_release\(\s*&empty\[", text))
     assert released >= 3  # both ring kernels and the older TMA-fed one
     tc = dict(sources())["tc.cuh"]
-    body = re.search(r"void ring_release\(uint64_t \*empty\)\s*\{(.*?)\n\}", tc, re.S).group(1)
+    body = re.search(r"void ring_release\(uint64_t \*empty[^)]*\)\s*\{(.*?)\n\}", tc, re.S).group(1)
     assert re.search(r"^\s*__syncwarp\(\);.*mbar_arrive\(empty\)", body, re.S)
