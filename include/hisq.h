@@ -231,18 +231,19 @@ hisq_status hisq_apply_dslash(hisq_ctx *ctx, int out_parity, int precision, int 
 hisq_status hisq_apply_dslash_batch(hisq_ctx *ctx, int out_parity, int precision, int nrhs, const double *in,
                                     double *out);
 
-/* Launch shape of the batched operator (testing and tuning; kind 0 = autotuned,
- * the default: with 16-bit vectors over the shapes of a kernel whose warps share
- * a shared-memory ring of links, with 32-bit ones also over kind 1).  kind 1: one site per thread for rhs_per_thread (2..4)
+/* Launch shape of the batched operator (testing and tuning).  kind 0 (the default):
+ * autotuned, with 16-bit vectors over the shapes of kind 4, with 32-bit ones also
+ * over those of kind 1.  kind 1: one site per thread for rhs_per_thread (2..4)
  * right-hand sides, links loaded by each thread, with (budget 0) or without
  * (budget 1) an L2 prefetch of the next direction's links; kind 2: the same
  * work split with the links of each site group and direction bulk-copied into
  * a shared-memory ring, `budget` (2..4) blocks per SM (12-real long links only;
  * never chosen by the autotuner, slower on GB300); kind 3: as kind 1 with the
  * right-hand sides in pairs whose colour algebra runs as packed two-wide FP32
- * FMAs (rhs_per_thread 2 or 4); kind 4: the kernel of the default, `budget` (1, 2
- * or 4) blocks per SM (18- or 12-real long links).  A shape that does not exist for a batch size
- * makes the batched calls fail with HISQ_ERR_INVALID_ARG. */
+ * FMAs (rhs_per_thread 2 or 4); kind 4: the warps of a block share a
+ * shared-memory ring of links, `budget` (1, 2 or 4) blocks per SM (18- or
+ * 12-real long links).  A shape that does not exist for a batch size makes the
+ * batched calls fail with HISQ_ERR_INVALID_ARG. */
 hisq_status hisq_set_batched_kernel(hisq_ctx *ctx, int kind, int rhs_per_thread, int budget);
 
 /* Even sites of `out` = (M^dag M)_ee applied to the even sites of `in`
